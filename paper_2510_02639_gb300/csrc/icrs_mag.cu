@@ -34,36 +34,26 @@
 #include "icrs_df64.cuh"
 #include "icrs_sectors.cuh"
 #include "icrs_ps.cuh"
+#include "icrs_rays.cuh"
 
 namespace icrs {
 
-// Threads per block (one block per SM).  The binary forward kernel's ray
-// stage evaluates two columns per paired FP32 instruction and is bound by
-// dependency latency more than by issue: registers for independent column
-// pairs pay more than further warps (at 1024 x 2048 on a 320-epoch sample:
-// 512 threads 6.66 ms, 576 6.86, 640 6.93, 768 7.01).  NT_WIDE is the binary
-// forward block size (with a 512-thread fallback where its layout does not
-// fit in shared memory); the derivative and triple instantiations keep 512
-// threads (128 registers): with fewer their FP64 phases spill kilobytes.
-constexpr int NT_WIDE = 512, NT_BASE = 512;
-__host__ __device__ constexpr int mag_threads(int nl, bool der) { return (nl == 2 && !der) ? NT_WIDE : NT_BASE; }
-constexpr int NW_MAX = NT_WIDE / 32;  // warps per block, largest instantiation
-constexpr int NW_DER = NT_BASE / 32;  // warps per block, derivative mode
+// Threads per block (one block per SM): 512, 128 registers each.  The ray
+// stage is bound by the FP32 pipes and the dependency latency of its chains:
+// registers for independent column pairs pay more than further warps.
+constexpr int NT_BASE = 512;
+constexpr int NW_MAX = NT_BASE / 32;  // warps per block
+constexpr int NW_DER = NT_BASE / 32;
+static_assert(TASK_WARPS == NW_MAX, "the ray stage's chunks are cut for this many warps");
 constexpr int QMAX = 2048;       // work queue
 constexpr int PMAX_MIN = 512;    // FP64-polished image-limb points per epoch (at least)
 constexpr int MAXT = 32;         // theta runs (more: ICRS_ST_OVERFLOW)
 constexpr int MAXRB = 32;        // r bins per theta run
 constexpr int MAXCELL = 96;      // (theta run, r run) cells
 constexpr int MAXBOX = 96;       // candidate sectors before merging
-constexpr int MAXANCH = 128;     // FP64 anchors per sector
-constexpr int GTH_MAX = 256;     // columns per theta group (at most)
-// Deferred boundary points per warp in the forward ray stage: 32 (one per
-// lane when the queue is flushed), each a (column, row) pair.
-__host__ __device__ constexpr int dq_entries(int) { return 32; }
 constexpr int MAXCELL_D = 32;    // cells with tracked derivatives
 constexpr int MAXBOX_D = 32;     // candidate sectors with tracked derivatives
 constexpr float TINY_EXTENT = 3e-4f;  // images smaller than this x rho skip FP64 decisions
-constexpr float EPS32 = 5.9604645e-8f;  // 2^-24
 // A refined FP32 image whose error bound exceeds EE_SUSPECT max(1, r), or two
 // images of one limb point closer than DUP_TOL max(1, r), send the limb point
 // to the FP64 re-solve.
@@ -75,33 +65,14 @@ constexpr float DUP_TOL = 1e-6f;
 constexpr float PAIR_TOL = (float)PS_PAIR_TOL;
 
 // Meta bits of an image-limb slot.
-constexpr uint8_t M_VALID = 1, M_EXACT = 2, M_UNSURE = 4, M_CAND = 8;
-
-// Anchor of a (theta group, r group) of a sector: the rays' squared distance
-// is evaluated about it in FP32 with U = sum_j K_j / Q_j (A_j = e^{-i th_m}
-// (z_m - a_j), K_j = eps_j / A_j, Q_j = A_j + dz, dz the ray's offset from the
-// anchor z_m in the anchor's rotated frame) as one quotient N / P of
-// polynomials in dz, with N = sum_j K_j prod_{k != j} Q_k and P = prod_j Q_j:
-//   binary:  N = n0 + n1 dz,             P = p0 + dz (p1 + dz)
-//   triple:  N = n0 + dz (n1 + dz n2),   P = p0 + dz (p1 + dz (p2 + dz))
-// (coefficients formed in FP64 and rounded once).
-struct AnchorF {
-  cf ws;        // e^{-i th_m} (f(z_m) - w_c)
-  cf n[3];      // numerator coefficients
-  cf p[3];      // denominator coefficients (monic)
-  float e0;     // error bound constant part
-  float pad;
-  float lo2;    // below: every ray of the group is inside the source (FP32 certain)
-  float hi2;    // above: every ray of the group is outside (FP32 certain)
-};
-
-using Box = BoxT<double>;
+constexpr uint8_t M_VALID = 1, M_EXACT = 2, M_UNSURE = 4, M_CAND = 8, M_CANDT = 16;
 
 struct Shared {
   // ---- per parameter set
   Lens L;
   double rho, u1, u2;
   double pa[4];        // a1..a4, the power series in mu^(1/2)
+  float I0, c0f, c1f, c2f;  // brightness coefficients of the set's law (see the set-up)
   float c1h, c3h;      // their half-integer-power brightness coefficients (ray stage)
   int half;            // c1h or c3h nonzero
   // spot: centre (rho units), radius^2 and contrast; 1 / (1 - c F_spot) and
@@ -126,21 +97,27 @@ struct Shared {
   uint32_t status;
   int warm;            // roots[] hold the previous epoch of this set
   int qn, pn;
-  unsigned long long tocc[2];   // occupied theta bins (up to 128)
+  double ht;           // width of a theta bin
+  float htf;
+  unsigned int tocc[4];         // occupied theta bins (up to 128)
   int nT, full;
   signed char runT[128];
   int startT[MAXT];
   unsigned int t_rlo_u[MAXT], t_rhi_l[MAXT];
   unsigned long long t_rlo[MAXT], t_rhi[MAXT];
   double rlo[MAXT], hr[MAXT];
+  float rlh[MAXT], rll[MAXT], ihr[MAXT];  // rlo as a float pair, 1 / hr
+  int rsmall[MAXT];    // 1: hr > 0 but the run is below TINY_EXTENT rho; 2: hr = 0
   unsigned int rocc[MAXT];
-  unsigned long long tmask[MAXT][MAXRB][2];  // theta bins of each (run, r bin)
+  unsigned int tmask[MAXT][MAXRB][4];  // theta bins of each (run, r bin)
   signed char rrun[MAXT][MAXRB];
   int cellbase[MAXT + 1];
   int ncell;
   int origin_in;
   int c_cnt[MAXCELL];
   unsigned int c_u[MAXCELL][4];             // FP32 keys: rmin_hi, rmax_lo, tmin_hi, tmax_lo
+  unsigned int c_s[MAXCELL][2];             // FP32 keys of the refined angle: tmin_hi, tmax_lo
+  float2 c_ref[MAXCELL][2];                 // direction of the FP32 angle extremes
   unsigned long long c_x[MAXCELL][4];       // FP64 keys: rmin, rmax, tmin, tmax
   int nbox;
   Box box[MAXBOX];
@@ -294,6 +271,14 @@ __device__ __noinline__ double ray_distance64(const Shared& sh, const Box& B, in
   return sqrt(abs2(w - sh.wc));
 }
 
+// Sine of the angle from direction X to the angle th, in FP64 (out of line: a
+// rare fallback).
+__device__ __noinline__ float sine_from64(float2 X, double th) {
+  double s, c;
+  sincos(th, &s, &c);
+  return (float)((double)X.x * s - (double)X.y * c);
+}
+
 // Tangents of an image-limb point z = r e^{i th} (the image of the source-limb
 // point w_c + rho u) with respect to (t0, tE, u0, alpha, s, q, rho, u1), binary
 // lens: the implicit derivative of the lens equation F(z; p) = f(z; p) - w(p)
@@ -403,50 +388,7 @@ __device__ __forceinline__ void q_push(Shared& sh, int* queue, int v) {
 }
 
 // ---------------------------------------------------------------- quadrature
-// Crossing of the interpolated distance with rho.  The stencil nodes are
-// consecutive integers x0, x0+1, ... (npt = 2..4), so the interpolant is
-// written in Newton's forward-difference form (the same polynomial as the
-// Lagrange form of Appendix A, without divisions).  The root on the bracket
-// between the inside sample (offset 0, p < rho) and the outside sample
-// (x_out = +-1, p >= rho) is found by the Illinois variant of regula falsi,
-// which keeps the bracket and converges superlinearly.
-template <class T>
-__device__ inline T crossing_solve(const T* y, T x0, int npt, T yin, T yout, T x_out, T rho, T tol, int iters) {
-  const T d1 = y[1] - y[0];
-  const T d2 = npt > 2 ? T(0.5) * (y[2] - T(2) * y[1] + y[0]) : T(0);
-  const T d3 = npt > 3 ? (y[3] - T(3) * y[2] + T(3) * y[1] - y[0]) * T(1.0 / 6.0) : T(0);
-  T a = T(0), ga = yin - rho;      // inside end  (g < 0)
-  T b = x_out, gb = yout - rho;    // outside end (g >= 0)
-  int side = 0;
-  for (int it = 0; it < iters; ++it) {
-    T den = gb - ga;
-    T c = (den != T(0)) ? b - gb * (b - a) / den : T(0.5) * (a + b);
-    T t = c - x0;
-    T gc = y[0] + t * (d1 + (t - T(1)) * (d2 + (t - T(2)) * d3)) - rho;
-    if (gc == T(0)) return c;
-    if ((gc < T(0)) == (gb < T(0))) {
-      b = c; gb = gc;
-      if (side == -1) ga *= T(0.5);
-      side = -1;
-    } else {
-      a = b; ga = gb;
-      b = c; gb = gc;
-      side = 1;
-    }
-    if (fabs(b - a) < tol) break;
-  }
-  return b;
-}
-
-// LD correction f(delta) (Appendix A.2) or the uniform rule delta + 1/2.
-template <class T>
-__device__ __forceinline__ T fdelta(T d, T delta_c, int uniform) {
-  if (uniform) return d + T(0.5);
-  if (d >= delta_c) return (T(0.5) + d) * (T(2.0 / 3.0) * sqrt(T(1) + T(1) / (T(2) * d)));
-  return T(2.0 / 3.0) * d + T(0.5);
-}
-
-// f'(delta) of the rule above.
+// f'(delta) of fdelta.
 template <class T>
 __device__ __forceinline__ T fdelta_prime(T d, T delta_c, int uniform) {
   if (uniform) return T(1);
@@ -488,18 +430,17 @@ __global__ void __launch_bounds__(NTB, 1)
 mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ T_, int E,
            icrs_grid g, int tiles_per_block, double* __restrict__ A_out, uint32_t* __restrict__ st_out,
            double* __restrict__ diag_sect, int32_t* __restrict__ diag_cnt, float* __restrict__ diag_pts, int PMAX,
-           int has_plo, DerOut dout, const int32_t* __restrict__ items, int n_items, int defer) {
+           int has_plo, int tabcap, DerOut dout, const int32_t* __restrict__ items, int n_items) {
   constexpr int N = NL * NL + 1;
   constexpr int NT = NTB;
   constexpr int NW = NT / 32;
   static_assert(NT % 32 == 0 && NW <= NW_MAX && (!DER || NW == NW_DER), "per-warp tables are sized for these block sizes");
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ Shared sh;
+  __shared__ typename std::conditional<DER, char, RayShared>::type rays_sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = g.n_limb, NP = K * N;
   const int BT = g.n_bins_theta, BR = g.n_bins_r;
-  const double ht = 2.0 * kPi / BT;
-
   // dynamic shared memory carve-up
   unsigned char* p = dyn;
   // per image-limb slot: root / refined image position in the lightest
@@ -507,32 +448,42 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
   // error bound, flags, bins, index into the FP64 table
   cf* phi = (cf*)p;              p += sizeof(cf) * NP;
   cf* plo = (cf*)p;              p += has_plo ? sizeof(cf) * NP : 0;   // lo part of refined positions
+  cdf* ulimb = (cdf*)p;          p += sizeof(cdf) * K;   // e^{2 pi i k / N_limb} as double-float
+  // derivative mode: its state
+  DerShared& ds = *(DerShared*)p;  p += DER ? sizeof(DerShared) : 0;
+  p = (unsigned char*)(((uintptr_t)p + 15) & ~(uintptr_t)15);
+  // the ray stage's tables take the place of the image-limb slots, which
+  // nothing reads once the sectors stand (16-byte rows of the offset table)
+  unsigned char* pr_ = p;
+  float* tabf = (float*)pr_;     pr_ += sizeof(cf) * tabcap;        // group offsets (cos d - 1, sin d)
+  cf* tab = (cf*)tabf;
+  AnchorF* anch = (AnchorF*)pr_; pr_ += sizeof(AnchorF) * MAXANCH;
+  float2* spc = (float2*)pr_;    pr_ += sizeof(float2) * MAXANCH;  // spot centre in each anchor's frame
+  int* wqueue = (int*)pr_;       // boundary points, a queue per warp
   float* r32 = (float*)p;        p += sizeof(float) * NP;
   float* rl32 = (float*)p;       p += sizeof(float) * NP;   // r = r32 + rl32 (double-float)
   float* t32 = (float*)p;        p += sizeof(float) * NP;
   float* e32 = (float*)p;        p += sizeof(float) * NP;
+  double* pr = (double*)p;       p += sizeof(double) * PMAX;
+  double* pt = (double*)p;       p += sizeof(double) * PMAX;
+  int* queue = (int*)p;          p += sizeof(int) * QMAX;
   short* pidx = (short*)p;       p += sizeof(short) * ((NP + 7) & ~7);
   uint8_t* meta = (uint8_t*)p;   p += (NP + 15) & ~15;
   uint8_t* tb = (uint8_t*)p;     p += (NP + 15) & ~15;
   uint8_t* rb = (uint8_t*)p;     p += (NP + 15) & ~15;
-  double* pr = (double*)p;       p += sizeof(double) * PMAX;
-  double* pt = (double*)p;       p += sizeof(double) * PMAX;
-  int* queue = (int*)p;          p += sizeof(int) * QMAX;
-  p = (unsigned char*)(((uintptr_t)p + 15) & ~(uintptr_t)15);  // 16-byte rows of the offset table
-  AnchorF* anch = (AnchorF*)p;   p += sizeof(AnchorF) * MAXANCH;
-  float2* spc = (float2*)p;      p += sizeof(float2) * MAXANCH;  // spot centre in each anchor's frame
-  cf* tab = (cf*)p;              p += sizeof(cf) * (GTH_MAX + 2);  // group offsets (cos d - 1, sin d)
-  cdf* ulimb = (cdf*)p;          p += sizeof(cdf) * K;   // e^{2 pi i k / N_limb} as double-float
-  // boundary points: a deferred queue per warp of (column, row) pairs
-  (void)defer;
-  int* wqueue = (int*)p;         p += sizeof(int) * NW * 2 * dq_entries(NL);
-  // derivative mode: its state
-  DerShared& ds = *(DerShared*)p;  p += DER ? sizeof(DerShared) : 0;
   DualD* cdual = ds.cx;
   BoxT<DualD>* bdual = ds.box;
   double* wder = &ds.wder[0][0];
 
-  if (tid == 0) { sh.cur_set = -1; sh.warm = 0; }
+  if (tid == 0) {
+    sh.cur_set = -1;
+    sh.warm = 0;
+    sh.ht = 2.0 * kPi / BT;
+    sh.htf = (float)sh.ht;
+    if constexpr (!DER)
+      rays_sh.P = {anch, spc, tabf, wqueue, tabcap, g.n_r, g.n_theta, g.uniform, g.ld_split && !g.uniform ? 1 : 0,
+                   diag_cnt ? 1 : 0, 1.0f, g.delta_c};
+  }
   for (int k = tid; k < K; k += NT) {
     double sn, cs;
     sincospi(2.0 * (double)k / (double)K, &sn, &cs);
@@ -564,7 +515,32 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
         sh.u1 = prm.u1;
         sh.u2 = prm.u2;
         sh.pa[0] = prm.a1; sh.pa[1] = prm.a2; sh.pa[2] = prm.a3; sh.pa[3] = prm.a4;
+        {
+          // limb darkening I = I0 [1 - u1 (1 - mu) - u2 (1 - mu)^2 - sum_k a_k
+          // (1 - mu^(k/2))], mu = sqrt(1 - d^2/rho^2), I0 = 1 / (pi (1 - u1/3 -
+          // u2/6 - sum_k a_k k/(k+4))) (the linear law of Appendix A.2 when
+          // the others are 0); uniform: I = 1/pi.  As a polynomial in s =
+          // mu^(1/2):
+          //   I = c0f + c1f mu + c2f mu^2 + s (c1h + c3h mu),
+          //   c0f = I0 (1 - u1 - u2 - sum a) (the limb value), c1f = I0 (u1 +
+          //   2 u2 + a2), c2f = I0 (a4 - u2), c1h = I0 a1, c3h = I0 a3.
+          // Formed once per set by one thread: every thread forming them for
+          // every epoch cost 38k of the 239k cycles that the ray stage of a
+          // 64 x 256 epoch took (an FP64 instruction occupies the SM for
+          // about 16 cycles, whatever its warp's active lanes).
+          const double sa_ = sh.pa[0] / 5.0 + sh.pa[1] * (2.0 / 6.0) + sh.pa[2] * (3.0 / 7.0) + sh.pa[3] * 0.5;
+          const double I0d = 1.0 / (kPi * (1.0 - sh.u1 / 3.0 - sh.u2 / 6.0 - sa_));
+          sh.I0 = g.uniform ? (float)(1.0 / kPi) : (float)I0d;
+          sh.c0f = g.uniform ? sh.I0
+                             : (float)(I0d * (1.0 - sh.u1 - sh.u2 - sh.pa[0] - sh.pa[1] - sh.pa[2] - sh.pa[3]));
+          sh.c1f = g.uniform ? 0.f : (float)(I0d * (sh.u1 + 2.0 * sh.u2 + sh.pa[1]));
+          sh.c2f = g.uniform ? 0.f : (float)(I0d * (sh.pa[3] - sh.u2));
+          sh.c1h = g.uniform ? 0.f : (float)(I0d * sh.pa[0]);
+          sh.c3h = g.uniform ? 0.f : (float)(I0d * sh.pa[2]);
+          sh.half = (sh.c1h != 0.f || sh.c3h != 0.f) ? 1 : 0;
+        }
         sh.spot = prm.spot_c != 0.0;
+        sh.generic = sh.half || sh.spot;
         sh.spot_x = prm.spot_x; sh.spot_y = prm.spot_y; sh.spot_r = prm.spot_r; sh.spot_c = prm.spot_c;
         sh.spot_bad = sh.spot && !(prm.spot_r >= 0.0 && prm.spot_c < 1.0 &&
                                    hypot(prm.spot_x, prm.spot_y) + prm.spot_r <= 1.0);
@@ -634,7 +610,7 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
       sh.pn = 0;
       for (int c = 0; c < 16; ++c) sh.cnt[c] = 0;
       sh.clk0 = clock64();
-      sh.tocc[0] = sh.tocc[1] = 0ull;
+      sh.tocc[0] = sh.tocc[1] = sh.tocc[2] = sh.tocc[3] = 0u;
     }
     __syncthreads();
     const int ll = sh.L.ll;
@@ -1075,6 +1051,34 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     }
     if (diag_cnt && tid == 0) { long long c_ = clock64(); sh.cnt[5] = (int)min(c_ - sh.clk0, 2000000000LL); sh.clk0 = c_; }
     // ------------------------------------------------ 2. theta bins
+    // The binning phases (2 to 7) walk the image-limb slots root by root (a
+    // warp takes 32 neighbouring limb points of one root, which mostly belong
+    // to one image): what they collect per angular interval or cell is then
+    // reduced over the warp before one shared-memory atomic per interval,
+    // instead of 32 atomics that queue on one word.
+    const double ht = sh.ht;
+    const float htf = sh.htf;
+    const int KW = (K + 31) & ~31;  // limb points of one root, padded to whole warps
+    // calls f(ps, valid) for every slot, all 32 lanes of a warp together
+    auto for_slots = [&](auto f) {
+      for (int idx = tid; idx < KW * N; idx += NT) {
+        const int j = idx / KW, k = idx - j * KW;
+        const int ps = k * N + j;
+        const bool ok = k < K && (meta[k < K ? ps : 0] & M_VALID);
+        f(ok ? ps : 0, ok);
+      }
+    };
+    // calls f(in, id) once for every distinct id of the warp's lanes with
+    // `has` set (in: this lane has that id), all lanes together
+    auto by_id = [&](bool has, int id, auto f) {
+      unsigned todo = __ballot_sync(0xffffffffu, has);
+      while (todo) {
+        const int id0 = __shfl_sync(0xffffffffu, id, __ffs(todo) - 1);
+        const bool in = has && id == id0;
+        f(in, id0);
+        todo &= ~__ballot_sync(0xffffffffu, in);
+      }
+    };
     for (int ps = tid; ps < NP; ps += NT) {
       if (!(meta[ps] & M_VALID) || (meta[ps] & M_EXACT)) continue;
       // distance of the FP32 angle from the nearest bin edge, against the
@@ -1083,87 +1087,140 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
       // and the division by the float bin width (<= 128 bins x 1.2e-7 bin
       // widths, 7.5e-7 rad): 1.6e-6 rad in all; 64 EPS32 = 3.8e-6 leaves a
       // factor of two.  Closer points get an FP64 angle.
-      float u = (t32[ps] + kPiF) / (float)ht;
+      float u = (t32[ps] + kPiF) / htf;
       float fr = u - floorf(u);
-      float d = fminf(fr, 1.0f - fr) * (float)ht;
+      float d = fminf(fr, 1.0f - fr) * htf;
       float eth = e32[ps] / fmaxf(r32[ps], 1e-30f) + 64.0f * EPS32;
       if (d <= eth) q_push(sh, queue, ps);
     }
     run_polish();
-    for (int ps = tid; ps < NP; ps += NT) {
-      if (!(meta[ps] & M_VALID)) continue;
-      int t;
-      if (meta[ps] & M_EXACT) t = (int)floor((pt[pidx[ps]] + kPi) / ht);
-      else t = (int)floorf((t32[ps] + kPiF) / (float)ht);
-      t = min(max(t, 0), BT - 1);
-      tb[ps] = (uint8_t)t;
-      atomicOr(&sh.tocc[t >> 6], 1ull << (t & 63));
+    for_slots([&](int ps, bool ok) {
+      int t = 0;
+      if (ok) {
+        if (meta[ps] & M_EXACT) t = (int)floor((pt[pidx[ps]] + kPi) / ht);
+        else t = (int)floorf((t32[ps] + kPiF) / htf);
+        t = min(max(t, 0), BT - 1);
+        tb[ps] = (uint8_t)t;
+      }
+      unsigned w_ = 0u;  // lane i (< 4): word i of the warp's bins
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const unsigned o = __reduce_or_sync(0xffffffffu, ok && (t >> 5) == i ? 1u << (t & 31) : 0u);
+        if (lane == i) w_ = o;
+      }
+      if (w_) atomicOr(&sh.tocc[lane], w_);
+    });
+    for (int i = tid; i < MAXT * MAXRB; i += NT) {
+      const int T = i / MAXRB, b = i - T * MAXRB;
+      sh.tmask[T][b][0] = sh.tmask[T][b][1] = sh.tmask[T][b][2] = sh.tmask[T][b][3] = 0u;
+      sh.rrun[T][b] = -1;
+      if (b == 0) {
+        sh.t_rlo_u[T] = 0xffffffffu; sh.t_rhi_l[T] = 0u;
+        sh.t_rlo[T] = ~0ull; sh.t_rhi[T] = 0ull;
+        sh.rocc[T] = 0u;
+      }
     }
     __syncthreads();
 
     if (diag_cnt && tid == 0) { long long c_ = clock64(); sh.cnt[6] = (int)min(c_ - sh.clk0, 2000000000LL); sh.clk0 = c_; }
     if (diag_cnt && tid == 0) sh.cnt[13] = sh.cnt[0];
     // ------------------------------------------------ 3. theta runs (cyclic)
-    if (tid == 0) {
-      auto occb = [&](int t) -> bool { return (sh.tocc[t >> 6] >> (t & 63)) & 1ull; };
-      bool full = true;
-      for (int t = 0; t < BT; ++t) if (!occb(t)) full = false;
-      for (int t = 0; t < 128; ++t) sh.runT[t] = -1;
+    // One warp, lane i the bins 32 i .. 32 i + 31 where words are formed and
+    // one lane per bin where runs are numbered: a run starts at an occupied
+    // bin whose predecessor (cyclic) is empty, and runs are numbered in cyclic
+    // order from the first empty bin t0.
+    if (warp == 0) {
+      auto occb = [&](int t) -> bool { return (sh.tocc[t >> 5] >> (t & 31)) & 1u; };
+      int nfree = BT, t0 = BT;  // empty bins, first empty bin
+      nfree = BT - (__popc(sh.tocc[0]) + __popc(sh.tocc[1]) + __popc(sh.tocc[2]) + __popc(sh.tocc[3]));
+      const bool full = nfree == 0;
       int nT = 0;
-      if (!(sh.tocc[0] | sh.tocc[1])) {
-        nT = 0;
+      if (nfree == BT) {
+        for (int t = lane; t < 128; t += 32) sh.runT[t] = -1;
       } else if (full) {
-        for (int t = 0; t < BT; ++t) sh.runT[t] = 0;
-        sh.startT[0] = 0;
+        for (int t = lane; t < 128; t += 32) sh.runT[t] = t < BT ? 0 : -1;
+        if (lane == 0) sh.startT[0] = 0;
         nT = 1;
       } else {
-        int t0 = 0;
-        while (occb(t0)) ++t0;
-        for (int kk = 1; kk <= BT; ++kk) {
-          int t = (t0 + kk) % BT;
-          if (!occb(t)) continue;
-          int prev = (t + BT - 1) % BT;
-          if (occb(prev)) sh.runT[t] = sh.runT[prev];
-          else if (nT < MAXT) { sh.runT[t] = (signed char)nT; sh.startT[nT] = t; ++nT; }
-          else { sh.runT[t] = (signed char)(MAXT - 1); atomicOr(&sh.status, ICRS_ST_OVERFLOW); }
+        for (int i = 3; i >= 0; --i) {
+          const unsigned fr = ~sh.tocc[i];
+          if (fr && 32 * i + __ffs(fr) - 1 < BT) t0 = 32 * i + __ffs(fr) - 1;
         }
+        for (int t = lane; t < 128; t += 32) if (t >= BT || !occb(t)) sh.runT[t] = -1;
+        // bins in cyclic order kk = 1 .. BT from t0: the run's number is the
+        // count of run starts up to the bin, less one
+        bool over = false;
+        for (int k0 = 1; k0 <= BT; k0 += 32) {
+          const int kk = k0 + lane;
+          int t = t0 + kk;
+          t = t >= BT ? t - BT : t;
+          const bool oc = kk <= BT && occb(t);
+          const bool st_ = oc && !occb(t == 0 ? BT - 1 : t - 1);
+          const unsigned sb = __ballot_sync(0xffffffffu, st_);
+          const int r = nT + __popc(sb & (0xffffffffu >> (31 - lane))) - 1;
+          if (oc) {
+            sh.runT[t] = (signed char)min(r, MAXT - 1);
+            if (st_ && r < MAXT) sh.startT[r] = t;
+          }
+          if (oc && r >= MAXT) over = true;
+          nT += __popc(sb);
+        }
+        nT = min(nT, MAXT);
+        if (over) atomicOr(&sh.status, ICRS_ST_OVERFLOW);
       }
-      sh.nT = nT;
-      sh.full = full ? 1 : 0;
-      for (int T = 0; T < MAXT; ++T) {
-        sh.t_rlo_u[T] = 0xffffffffu; sh.t_rhi_l[T] = 0u;
-        sh.t_rlo[T] = ~0ull; sh.t_rhi[T] = 0ull;
-        sh.rocc[T] = 0u;
-        for (int b = 0; b < MAXRB; ++b) { sh.tmask[T][b][0] = sh.tmask[T][b][1] = 0ull; sh.rrun[T][b] = -1; }
-      }
+      if (lane == 0) { sh.nT = nT; sh.full = full ? 1 : 0; }
     }
     __syncthreads();
     const int nT = sh.nT;
 
     // ------------------------------------------------ 4. r range per theta run
-    for (int ps = tid; ps < NP; ps += NT) {
-      if (!(meta[ps] & M_VALID)) continue;
-      int T = sh.runT[tb[ps]];
-      float r = r32[ps], er = (meta[ps] & M_EXACT) ? 4.0f * EPS32 * r : e32[ps] + 4.0f * EPS32 * r;
-      atomicMin(&sh.t_rlo_u[T], fkey(r + er));
-      atomicMax(&sh.t_rhi_l[T], fkey(r - er));
-    }
+    // Extremes in three narrowing passes: FP32 radii with their FP32 errors,
+    // then the double-float radii of the points those leave (error e32,
+    // mostly a few 1e-12), then FP64 polishes of the points still left whose
+    // e32 is above 1e-11.  (Polishing every point that the FP32 pass leaves
+    // took 255 polishes an epoch of the 64 x 256 batch; 54 are left, and phases
+    // 2 to 7 went from 218k to 164k cycles.)
+    for_slots([&](int ps, bool ok) {
+      const int T = ok ? sh.runT[tb[ps]] : 0;
+      const float r = r32[ps], er = (meta[ps] & M_EXACT) ? 4.0f * EPS32 * r : e32[ps] + 4.0f * EPS32 * r;
+      by_id(ok, T, [&](bool in, int T0) {
+        const unsigned lo = __reduce_min_sync(0xffffffffu, in ? fkey(r + er) : 0xffffffffu);
+        const unsigned hi = __reduce_max_sync(0xffffffffu, in ? fkey(r - er) : 0u);
+        if (lane == 0) { atomicMin(&sh.t_rlo_u[T0], lo); atomicMax(&sh.t_rhi_l[T0], hi); }
+      });
+    });
     __syncthreads();
     const float tiny = TINY_EXTENT * rho32;
+    // r of a slot and its error bound (FP64 if polished, else double-float)
+    auto re = [&](int ps) -> double { return (meta[ps] & M_EXACT) ? 0.0 : (double)e32[ps]; };
     for (int ps = tid; ps < NP; ps += NT) {
       if (!(meta[ps] & M_VALID)) continue;
       int T = sh.runT[tb[ps]];
       float r = r32[ps], er = (meta[ps] & M_EXACT) ? 4.0f * EPS32 * r : e32[ps] + 4.0f * EPS32 * r;
-      bool cand = fkey(r - er) <= sh.t_rlo_u[T] || fkey(r + er) >= sh.t_rhi_l[T];
+      if (fkey(r - er) <= sh.t_rlo_u[T] || fkey(r + er) >= sh.t_rhi_l[T]) {
+        meta[ps] |= M_CAND;
+        const double R = rv(ps), E_ = re(ps);
+        atomicMin(&sh.t_rlo[T], dkey(R + E_));
+        atomicMax(&sh.t_rhi[T], dkey(R - E_));
+      }
+    }
+    __syncthreads();
+    for (int ps = tid; ps < NP; ps += NT) {
+      if (!(meta[ps] & M_CAND)) continue;
+      int T = sh.runT[tb[ps]];
+      const double R = rv(ps), E_ = re(ps);
+      if (!(dkey(R - E_) <= sh.t_rlo[T] || dkey(R + E_) >= sh.t_rhi[T])) { meta[ps] &= (uint8_t)~M_CAND; continue; }
       // an image smaller than tiny contributes below the parity tolerance:
       // its decisions stay in FP32
       bool is_tiny = fkey_inv(sh.t_rhi_l[T]) - fkey_inv(sh.t_rlo_u[T]) < tiny;
       // the double-float r (error e32) is exact enough unless e32 is large
-      if (cand) { meta[ps] |= M_CAND; if (!(meta[ps] & M_EXACT) && !is_tiny && !(e32[ps] <= 1e-11f)) q_push(sh, queue, ps); }
+      if (!(meta[ps] & M_EXACT) && !is_tiny && !(e32[ps] <= 1e-11f)) q_push(sh, queue, ps);
     }
+    __syncthreads();
+    if (tid < nT) { sh.t_rlo[tid] = ~0ull; sh.t_rhi[tid] = 0ull; }
     run_polish();
     for (int ps = tid; ps < NP; ps += NT) {
-      if (!(meta[ps] & M_VALID) || !(meta[ps] & M_CAND)) continue;
+      if (!(meta[ps] & M_CAND)) continue;
       meta[ps] &= (uint8_t)~M_CAND;
       int T = sh.runT[tb[ps]];
       double r = rv(ps);
@@ -1173,8 +1230,13 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     __syncthreads();
     if (tid < nT) {
       double lo = dkey_inv(sh.t_rlo[tid]), hi = dkey_inv(sh.t_rhi[tid]);
+      const double h = (hi - lo) / BR;
       sh.rlo[tid] = lo;
-      sh.hr[tid] = (hi - lo) / BR;
+      sh.hr[tid] = h;
+      sh.rlh[tid] = (float)lo;
+      sh.rll[tid] = (float)(lo - (double)(float)lo);
+      sh.ihr[tid] = (float)(1.0 / h);
+      sh.rsmall[tid] = !(h > 0.0) ? 2 : (h * BR < (double)tiny ? 1 : 0);
     }
     __syncthreads();
 
@@ -1186,10 +1248,8 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     // error, else in FP64 (after an FP64 polish if the double-float r itself
     // is uncertain).
     auto rbin_u = [&](int ps, int T, float* err) -> float {
-      const float rlh = (float)sh.rlo[T];
-      const float rll = (float)(sh.rlo[T] - (double)rlh);
-      const float ihr = (float)(1.0 / sh.hr[T]);
-      float dr = (r32[ps] - rlh) + (rl32[ps] - rll);
+      const float ihr = sh.ihr[T];
+      float dr = (r32[ps] - sh.rlh[T]) + (rl32[ps] - sh.rll[T]);
       float u = dr * ihr;
       *err = 4.0f * EPS32 * fabsf(u) + e32[ps] * ihr + 1e-6f;
       return u;
@@ -1197,62 +1257,82 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     for (int ps = tid; ps < NP; ps += NT) {
       if (!(meta[ps] & M_VALID) || (meta[ps] & M_EXACT)) continue;
       int T = sh.runT[tb[ps]];
-      double hr = sh.hr[T];
-      if (!(hr > 0.0) || hr * BR < (double)tiny || e32[ps] <= 1e-11f) continue;
+      if (sh.rsmall[T] || e32[ps] <= 1e-11f) continue;
       float eu;
       float u = rbin_u(ps, T, &eu);
       float fr = u - floorf(u);
       if (fminf(fr, 1.0f - fr) <= eu && u > 0.5f && u < (float)BR - 0.5f) q_push(sh, queue, ps);
     }
     run_polish();
-    for (int ps = tid; ps < NP; ps += NT) {
-      if (!(meta[ps] & M_VALID)) continue;
-      int T = sh.runT[tb[ps]];
-      double hr = sh.hr[T];
-      int b;
-      if (!(hr > 0.0)) b = 0;
-      else {
+    for_slots([&](int ps, bool ok) {
+      const int T = ok ? sh.runT[tb[ps]] : 0;
+      int b = 0;
+      if (ok && sh.rsmall[T] != 2) {
         float eu;
         float u = rbin_u(ps, T, &eu);
         float fr = u - floorf(u);
         if (fminf(fr, 1.0f - fr) > eu) b = (int)floorf(u);
-        else b = (int)floor((rv(ps) - sh.rlo[T]) / hr);
+        else b = (int)floor((rv(ps) - sh.rlo[T]) / sh.hr[T]);
+        b = min(max(b, 0), BR - 1);
       }
-      b = min(max(b, 0), BR - 1);
-      rb[ps] = (uint8_t)b;
-      atomicOr(&sh.rocc[T], 1u << b);
-      atomicOr(&sh.tmask[T][b][tb[ps] >> 6], 1ull << (tb[ps] & 63));
+      if (ok) {
+        rb[ps] = (uint8_t)b;
+        atomicOr(&sh.tmask[T][b][tb[ps] >> 5], 1u << (tb[ps] & 31));
+      }
+      by_id(ok, T, [&](bool in, int T0) {
+        const unsigned o = __reduce_or_sync(0xffffffffu, in ? 1u << b : 0u);
+        if (lane == 0) atomicOr(&sh.rocc[T0], o);
+      });
+    });
+    for (int i = tid; i < MAXCELL * 4; i += NT) {
+      const int c = i >> 2, k = i & 3;
+      sh.c_u[c][k] = (k & 1) ? 0u : 0xffffffffu;
+      sh.c_x[c][k] = (k & 1) ? 0ull : ~0ull;
+      if (k < 2) sh.c_s[c][k] = k ? 0u : 0xffffffffu;
+      if (k == 0) sh.c_cnt[c] = 0;
+    }
+    if constexpr (DER) {
+      for (int i = tid; i < MAXCELL_D * 4; i += NT) ds.cell_arg[i >> 2][i & 3] = 0x7fffffff;
     }
     __syncthreads();
 
     if (diag_cnt && tid == 0) { long long c_ = clock64(); sh.cnt[8] = (int)min(c_ - sh.clk0, 2000000000LL); sh.clk0 = c_; }
     if (diag_cnt && tid == 0) sh.cnt[15] = sh.cnt[0];
     // ------------------------------------------------ 6. gap probes, r runs, origin
-    // One warp: for every theta run, every empty gap with points of a shared
-    // theta bin on both sides is probed at its middle radius (FP32 with a
-    // guard band, FP64 when the guard cannot decide).
-    if (warp == 0) {
-      for (int T = 0; T < nT; ++T) {
-        unsigned int occ = sh.rocc[T];
-        unsigned int fill = 0u;
-        for (int b = 1; b < BR; ++b) {
-          if (((occ >> b) & 1u) || !((occ >> (b - 1)) & 1u)) continue;
-          int e2 = b;
-          while (e2 < BR && !((occ >> e2) & 1u)) ++e2;
-          if (e2 >= BR) break;
-          unsigned long long shared_[2];
-          for (int h = 0; h < 2; ++h) {
-            unsigned long long below = 0ull, above = 0ull;
-            for (int k = 0; k < b; ++k) below |= sh.tmask[T][k][h];
-            for (int k = e2; k < BR; ++k) above |= sh.tmask[T][k][h];
-            shared_[h] = below & above;
-          }
-          double rg = sh.rlo[T] + sh.hr[T] * 0.5 * (double)(b + e2);
-          bool hit = false;
-          for (int t0 = 0; t0 < BT && !hit; t0 += 32) {
-            int t = t0 + lane;
+    // One warp per theta run (round robin): every empty gap with points of a
+    // shared theta bin on both sides is probed at its middle radius (FP32 with
+    // a guard band, FP64 when the guard cannot decide).  The last warp tests
+    // the origin meanwhile.
+    if (warp == NW - 1 && lane == 0) {
+      cd w0 = lens_map<NL, double>(sh.L.eps, sh.L.a, mk(0.0, 0.0));
+      sh.origin_in = sqrt(abs2(w0 - sh.wc)) < sh.rho;
+    }
+    for (int T = warp; T < nT; T += NW) {
+      unsigned int occ = sh.rocc[T];
+      unsigned int fill = 0u;
+      // this lane's r bin: its theta bins
+      unsigned mine[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) mine[h] = lane < BR ? sh.tmask[T][lane < MAXRB ? lane : 0][h] : 0u;
+      for (int b = 1; b < BR; ++b) {
+        if (((occ >> b) & 1u) || !((occ >> (b - 1)) & 1u)) continue;
+        int e2 = b;
+        while (e2 < BR && !((occ >> e2) & 1u)) ++e2;
+        if (e2 >= BR) break;
+        unsigned shared_[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h)
+          shared_[h] = __reduce_or_sync(0xffffffffu, lane < b ? mine[h] : 0u) &
+                       __reduce_or_sync(0xffffffffu, lane >= e2 ? mine[h] : 0u);
+        bool hit = false;
+        if (shared_[0] | shared_[1] | shared_[2] | shared_[3]) {
+          const double rg = sh.rlo[T] + sh.hr[T] * 0.5 * (double)(b + e2);
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            if (hit || !shared_[h]) continue;
+            const int t = 32 * h + lane;
             bool in = false;
-            if (t < BT && ((shared_[t >> 6] >> (t & 63)) & 1ull)) {
+            if (t < BT && ((shared_[h] >> lane) & 1u)) {
               double th = -kPi + (t + 0.5) * ht;
               float sth, cth;
               sincosf((float)th, &sth, &cth);
@@ -1277,41 +1357,25 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
             }
             hit = __any_sync(0xffffffffu, in);
           }
-          if (hit) for (int k = b; k < e2; ++k) fill |= 1u << k;
         }
-        if (lane == 0) {
-          occ |= fill;
-          sh.rocc[T] = occ;
-          int nR = 0;
-          for (int b = 0; b < BR; ++b) {
-            if (!((occ >> b) & 1u)) continue;
-            if (b > 0 && ((occ >> (b - 1)) & 1u)) sh.rrun[T][b] = sh.rrun[T][b - 1];
-            else sh.rrun[T][b] = (signed char)(nR++);
-          }
-          sh.cellbase[T + 1] = nR;
-        }
-        __syncwarp();
+        if (hit) fill |= ((e2 < 32 ? 1u << e2 : 0u) - 1u) & ~((1u << b) - 1u);
       }
-      if (lane == 0) {
-        sh.cellbase[0] = 0;
-        int tot = 0;
-        for (int T = 0; T < nT; ++T) { int c = sh.cellbase[T + 1]; sh.cellbase[T] = tot; tot += c; }
-        sh.cellbase[nT] = tot;
-        if (tot > MAXCELL) { tot = MAXCELL; atomicOr(&sh.status, ICRS_ST_OVERFLOW); }
-        sh.ncell = tot;
-        cd w0 = lens_map<NL, double>(sh.L.eps, sh.L.a, mk(0.0, 0.0));
-        sh.origin_in = sqrt(abs2(w0 - sh.wc)) < sh.rho;
-        for (int c = 0; c < MAXCELL; ++c) {
-          sh.c_cnt[c] = 0;
-          sh.c_u[c][0] = 0xffffffffu; sh.c_u[c][1] = 0u; sh.c_u[c][2] = 0xffffffffu; sh.c_u[c][3] = 0u;
-          sh.c_x[c][0] = ~0ull; sh.c_x[c][1] = 0ull; sh.c_x[c][2] = ~0ull; sh.c_x[c][3] = 0ull;
-        }
-        if (DER) {
-          for (int c = 0; c < MAXCELL_D; ++c)
-            for (int k = 0; k < 4; ++k) ds.cell_arg[c][k] = 0x7fffffff;
-          if (tot > MAXCELL_D) atomicOr(&sh.status, ICRS_ST_OVERFLOW);
-        }
-      }
+      occ |= fill;
+      // r runs: numbered by their first bins
+      const unsigned starts = occ & ~(occ << 1);
+      if (lane < BR && ((occ >> lane) & 1u))
+        sh.rrun[T][lane] = (signed char)(__popc(starts & (0xffffffffu >> (31 - lane))) - 1);
+      if (lane == 0) { sh.rocc[T] = occ; sh.cellbase[T + 1] = __popc(starts); }
+    }
+    __syncthreads();
+    if (tid == 0) {
+      sh.cellbase[0] = 0;
+      int tot = 0;
+      for (int T = 0; T < nT; ++T) { int c = sh.cellbase[T + 1]; sh.cellbase[T] = tot; tot += c; }
+      sh.cellbase[nT] = tot;
+      if (tot > MAXCELL) { tot = MAXCELL; atomicOr(&sh.status, ICRS_ST_OVERFLOW); }
+      sh.ncell = tot;
+      if (DER && tot > MAXCELL_D) atomicOr(&sh.status, ICRS_ST_OVERFLOW);
     }
     __syncthreads();
 
@@ -1327,54 +1391,136 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     // on the angle: a point binned in FP64 next to the interval's first edge
     // can have an FP32 angle on the other side of that edge, and the FP32
     // candidate pass and the FP64 extreme pass must unwrap it alike.
-    auto unwrap_t = [&](int ps, double th) -> double {
-      int T = sh.runT[tb[ps]];
-      return (int)tb[ps] < sh.startT[T] ? th + 2.0 * kPi : th;
+    auto past_wrap = [&](int ps) -> bool { return (int)tb[ps] < sh.startT[sh.runT[tb[ps]]]; };
+    auto unwrap_t = [&](int ps, double th) -> double { return past_wrap(ps) ? th + 2.0 * kPi : th; };
+    // the FP32 angle, unwrapped (2 pi and the sum rounded: 4.1e-7 more, inside
+    // the 16 EPS32 of et together with atan2f's 4.8e-7)
+    auto unwrap_f = [&](int ps) -> float { return past_wrap(ps) ? t32[ps] + 2.0f * kPiF : t32[ps]; };
+    auto er_et = [&](int ps, float* er, float* et) {
+      const float r = r32[ps];
+      const bool ex = meta[ps] & M_EXACT;
+      *er = ex ? 4.0f * EPS32 * r : e32[ps] + 4.0f * EPS32 * r;
+      *et = ex ? 16.0f * EPS32 : e32[ps] / fmaxf(r, 1e-30f) + 16.0f * EPS32;
+    };
+    for_slots([&](int ps, bool ok) {
+      const int c = ok ? cell_of(ps) : 0;
+      const float r = r32[ps];
+      float er, et;
+      er_et(ps, &er, &et);
+      const float th = ok ? unwrap_f(ps) : 0.f;
+      by_id(ok, c, [&](bool in, int c0) {
+        const unsigned k0 = __reduce_min_sync(0xffffffffu, in ? fkey(r + er) : 0xffffffffu);
+        const unsigned k1 = __reduce_max_sync(0xffffffffu, in ? fkey(r - er) : 0u);
+        const unsigned k2 = __reduce_min_sync(0xffffffffu, in ? fkey(th + et) : 0xffffffffu);
+        const unsigned k3 = __reduce_max_sync(0xffffffffu, in ? fkey(th - et) : 0u);
+        if (lane == 0) {
+          sh.c_cnt[c0] = 1;
+          atomicMin(&sh.c_u[c0][0], k0);
+          atomicMax(&sh.c_u[c0][1], k1);
+          atomicMin(&sh.c_u[c0][2], k2);
+          atomicMax(&sh.c_u[c0][3], k3);
+        }
+      });
+    });
+    __syncthreads();
+    // the same narrowing passes as for the r ranges.  Angles: the points that
+    // the FP32 pass leaves are compared by the sine of their angle from the
+    // FP32 extreme's direction X, cross(X, z) / |z| with z in double-float
+    // (it differs by a few 1e-6 at most, so the sine keeps 1e-13)
+    const bool refine = has_plo && !sh.full;
+    if (refine) {
+      for (int i = tid; i < sh.ncell * 2; i += NT) {
+        float sn_, cs_;
+        sincosf(fkey_inv(sh.c_u[i >> 1][2 + (i & 1)]), &sn_, &cs_);
+        sh.c_ref[i >> 1][i & 1] = make_float2(cs_, sn_);
+      }
+      __syncthreads();
+    }
+    auto sine_from = [&](int ps, int c, int k, float* err) -> float {
+      const float r = r32[ps];
+      if (meta[ps] & M_EXACT) {
+        *err = 4e-13f;
+        return sine_from64(sh.c_ref[c][k], pt[pidx[ps]]);
+      }
+      const float2 X = sh.c_ref[c][k];
+      const df zx = df_add(df_make(phi[ps].x, plo[ps].x), sh.adf_ll[0]);
+      const df zy = df_add(df_make(phi[ps].y, plo[ps].y), sh.adf_ll[1]);
+      const df cr = df_sub(df_mul(df_make(X.x, 0.f), zy), df_mul(df_make(X.y, 0.f), zx));
+      const float s_ = (cr.hi + cr.lo) / r;
+      *err = 1.01f * e32[ps] / r + 4e-13f + 4e-7f * fabsf(s_);
+      return s_;
+    };
+    // FP32 extents of a point's cell below tiny: its decisions stay in FP32
+    auto tiny_cell = [&](int c, float r) -> bool {
+      return fkey_inv(sh.c_u[c][1]) - fkey_inv(sh.c_u[c][0]) < tiny &&
+             (fkey_inv(sh.c_u[c][3]) - fkey_inv(sh.c_u[c][2])) * r < tiny;
     };
     for (int ps = tid; ps < NP; ps += NT) {
       if (!(meta[ps] & M_VALID)) continue;
-      int c = cell_of(ps);
-      atomicAdd(&sh.c_cnt[c], 1);
-      float r = r32[ps];
-      float th = (float)unwrap_t(ps, (double)t32[ps]);
-      bool ex = meta[ps] & M_EXACT;
-      float er = ex ? 4.0f * EPS32 * r : e32[ps] + 4.0f * EPS32 * r;
-      float et = ex ? 16.0f * EPS32 : e32[ps] / fmaxf(r, 1e-30f) + 16.0f * EPS32;
-      atomicMin(&sh.c_u[c][0], fkey(r + er));
-      atomicMax(&sh.c_u[c][1], fkey(r - er));
-      atomicMin(&sh.c_u[c][2], fkey(th + et));
-      atomicMax(&sh.c_u[c][3], fkey(th - et));
+      const int c = cell_of(ps);
+      const float r = r32[ps], th = unwrap_f(ps);
+      float er, et;
+      er_et(ps, &er, &et);
+      if (fkey(r - er) <= sh.c_u[c][0] || fkey(r + er) >= sh.c_u[c][1]) {
+        meta[ps] |= M_CAND;
+        const double R = rv(ps), E_ = re(ps);
+        atomicMin(&sh.c_x[c][0], dkey(R + E_));
+        atomicMax(&sh.c_x[c][1], dkey(R - E_));
+      }
+      const bool lo = fkey(th - et) <= sh.c_u[c][2], hi = fkey(th + et) >= sh.c_u[c][3];
+      if (lo || hi) {
+        meta[ps] |= M_CANDT;
+        if (refine && !tiny_cell(c, r)) {
+          float e_;
+          if (lo) { const float s_ = sine_from(ps, c, 0, &e_); atomicMin(&sh.c_s[c][0], fkey(s_ + e_)); }
+          if (hi) { const float s_ = sine_from(ps, c, 1, &e_); atomicMax(&sh.c_s[c][1], fkey(s_ - e_)); }
+        }
+      }
     }
     __syncthreads();
     for (int ps = tid; ps < NP; ps += NT) {
-      if (!(meta[ps] & M_VALID)) continue;
-      int c = cell_of(ps);
-      float r = r32[ps];
-      float th = (float)unwrap_t(ps, (double)t32[ps]);
-      bool ex = meta[ps] & M_EXACT;
-      float er = ex ? 4.0f * EPS32 * r : e32[ps] + 4.0f * EPS32 * r;
-      float et = ex ? 16.0f * EPS32 : e32[ps] / fmaxf(r, 1e-30f) + 16.0f * EPS32;
-      bool cand_r = fkey(r - er) <= sh.c_u[c][0] || fkey(r + er) >= sh.c_u[c][1];
-      bool cand_t = fkey(th - et) <= sh.c_u[c][2] || fkey(th + et) >= sh.c_u[c][3];
-      bool cand = cand_r || cand_t;
-      float ext_r = fkey_inv(sh.c_u[c][1]) - fkey_inv(sh.c_u[c][0]);
-      float ext_t = (fkey_inv(sh.c_u[c][3]) - fkey_inv(sh.c_u[c][2])) * r;
-      bool is_tiny = ext_r < tiny && ext_t < tiny;
+      const uint8_t m_ = meta[ps];
+      if (!(m_ & (M_CAND | M_CANDT))) continue;
+      const int c = cell_of(ps);
+      const float r = r32[ps];
+      const bool is_tiny = tiny_cell(c, r);
+      bool cand_r = m_ & M_CAND, cand_t = m_ & M_CANDT;
+      if (cand_r) {
+        const double R = rv(ps), E_ = re(ps);
+        cand_r = dkey(R - E_) <= sh.c_x[c][0] || dkey(R + E_) >= sh.c_x[c][1];
+      }
+      if (cand_t && refine && !is_tiny) {
+        const float th = unwrap_f(ps);
+        float er, et, e_;
+        er_et(ps, &er, &et);
+        cand_t = false;
+        if (fkey(th - et) <= sh.c_u[c][2]) { const float s_ = sine_from(ps, c, 0, &e_); cand_t = fkey(s_ - e_) <= sh.c_s[c][0]; }
+        if (fkey(th + et) >= sh.c_u[c][3]) { const float s_ = sine_from(ps, c, 1, &e_); cand_t = cand_t || fkey(s_ + e_) >= sh.c_s[c][1]; }
+      }
+      meta[ps] = (uint8_t)((m_ & ~(M_CAND | M_CANDT)) | (cand_r ? M_CAND : 0) | (cand_t ? M_CANDT : 0));
       // theta extremes need an FP64 angle; r extremes only if the
       // double-float r is uncertain
-      bool need = (cand_t && !sh.full) || !(e32[ps] <= 1e-11f);
-      if (cand) { meta[ps] |= M_CAND; if (!ex && !is_tiny && need) q_push(sh, queue, ps); }
+      const bool need = (cand_t && !sh.full) || ((cand_r || cand_t) && !(e32[ps] <= 1e-11f));
+      if (need && !(m_ & M_EXACT) && !is_tiny) q_push(sh, queue, ps);
     }
+    __syncthreads();
+    for (int i = tid; i < sh.ncell * 2; i += NT) sh.c_x[i >> 1][i & 1] = (i & 1) ? 0ull : ~0ull;
     run_polish();
     for (int ps = tid; ps < NP; ps += NT) {
-      if (!(meta[ps] & M_VALID) || !(meta[ps] & M_CAND)) continue;
-      meta[ps] &= (uint8_t)~M_CAND;
+      const uint8_t m_ = meta[ps];
+      if (!(m_ & (M_CAND | M_CANDT))) continue;
+      meta[ps] = (uint8_t)(m_ & ~(M_CAND | M_CANDT));
       int c = cell_of(ps);
-      double r = rv(ps), th = unwrap_t(ps, tv(ps));
-      atomicMin(&sh.c_x[c][0], dkey(r));
-      atomicMax(&sh.c_x[c][1], dkey(r));
-      atomicMin(&sh.c_x[c][2], dkey(th));
-      atomicMax(&sh.c_x[c][3], dkey(th));
+      if (m_ & M_CAND) {
+        const double r = rv(ps);
+        atomicMin(&sh.c_x[c][0], dkey(r));
+        atomicMax(&sh.c_x[c][1], dkey(r));
+      }
+      if (m_ & M_CANDT) {
+        const double th = unwrap_t(ps, tv(ps));
+        atomicMin(&sh.c_x[c][2], dkey(th));
+        atomicMax(&sh.c_x[c][3], dkey(th));
+      }
     }
     __syncthreads();
     if (DER) {
@@ -1465,33 +1611,16 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
 
     if (diag_cnt && tid == 0) { long long c_ = clock64(); sh.cnt[11] = (int)min(c_ - sh.clk0, 2000000000LL); sh.clk0 = c_; }
     // ------------------------------------------------ 9. rays
+    double raysum = 0.0;  // this thread's share
+    if constexpr (!DER) {
+      raysum = ray_stage<NL, LAW>(sh, rays_sh);
+    } else {
     const int NR = g.n_r, NTH = g.n_theta;
-    // limb darkening I = I0 [1 - u1 (1 - mu) - u2 (1 - mu)^2 - sum_k a_k (1 -
-    // mu^(k/2))], mu = sqrt(1 - d^2/rho^2), I0 = 1 / (pi (1 - u1/3 - u2/6 -
-    // sum_k a_k k/(k+4))) (the linear law of Appendix A.2 when the others are
-    // 0); uniform: I = 1/pi.  As a polynomial in s = mu^(1/2):
-    //   I = c0f + c1f mu + c2f mu^2 + s (c1h + c3h mu),
-    //   c0f = I0 (1 - u1 - u2 - sum a) (the limb value), c1f = I0 (u1 + 2 u2 +
-    //   a2), c2f = I0 (a4 - u2), c1h = I0 a1, c3h = I0 a3
-    const double sa_ = sh.pa[0] / 5.0 + sh.pa[1] * (2.0 / 6.0) + sh.pa[2] * (3.0 / 7.0) + sh.pa[3] * 0.5;
-    const double I0d = 1.0 / (kPi * (1.0 - sh.u1 / 3.0 - sh.u2 / 6.0 - sa_));
-    const float I0 = g.uniform ? (float)(1.0 / kPi) : (float)I0d;
+    // the set's brightness law (see the set-up)
+    const float I0 = sh.I0, c0f = sh.c0f, c1f = sh.c1f, c2f = sh.c2f;
     const float irho2 = 1.0f / (rho32 * rho32);
     const float irho = 1.0f / rho32;
     const float dcf = (float)g.delta_c;
-    const float c0f = g.uniform ? I0 : (float)(I0d * (1.0 - sh.u1 - sh.u2 - sh.pa[0] - sh.pa[1] - sh.pa[2] - sh.pa[3]));
-    const float c1f = g.uniform ? 0.f : (float)(I0d * (sh.u1 + 2.0 * sh.u2 + sh.pa[1]));
-    const float c2f = g.uniform ? 0.f : (float)(I0d * (sh.pa[3] - sh.u2));
-    // c1h, c3h and their flag live in shared memory: the default sweep
-    // never reads them
-    if (tid == 0) {
-      sh.c1h = g.uniform ? 0.f : (float)(I0d * sh.pa[0]);
-      sh.c3h = g.uniform ? 0.f : (float)(I0d * sh.pa[2]);
-      sh.half = (sh.c1h != 0.f || sh.c3h != 0.f) ? 1 : 0;
-      sh.generic = sh.half || sh.spot;
-    }
-    __syncthreads();
-    const bool split = g.ld_split && !g.uniform;  // split-profile boundary rule
     const float sfac = (float)g.s_fac;            // sigmoid steepness of the paper's gradient rule
     float acc_s = 0.f, acc_c = 0.f;  // Kahan sum of this thread
     uint32_t st_local = 0u;
@@ -1576,7 +1705,6 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
           af.ws = ws;
           for (int k = 0; k < 3; ++k) { af.n[k] = tof(nc[k]); af.p[k] = tof(pc[k]); }
           af.e0 = e0;
-          af.pad = 0.f;
           // the group's band: every ray has |dz| <= half, so |Q_j| >= |A_j| -
           // half, |P| >= prod_j (|A_j| - half) and |U| <= sum_j |K_j| / (|A_j|
           // - half); the rounding error of the FP32 quotient is bounded by
@@ -1835,8 +1963,6 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
         // (Appendix A per-point rule).  The adjoint adds, for every inside
         // ray, its seed dI/dd times the gradient of d, and the queue flush
         // the boundary points' seeds.
-        constexpr int DQ = dq_entries(NL);
-        constexpr int KB = 8;  // columns per block (even: column pairs load as 16 bytes)
         int2* dq = reinterpret_cast<int2*>(wqueue + warp * 2 * DQ);
         int dq_n = 0;
         const int CH = sh.chunk;
@@ -1938,280 +2064,7 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
           if (fso) *fso = spot_factor(gi_ * mth + mgrp, dw, eb, irow, lw);
           return in;
         };
-        if constexpr (!DER) {
-        // the anchor as broadcast pairs for two columns at once (binary)
-        struct AnchorP { float2 wsx, wsy, n0x, n0y, n1x, n1y, nn1y, p0x, p0y, p1x, p1y; };
-        auto pairs_of = [](const AnchorF& a) -> AnchorP {
-          AnchorP r;
-          r.wsx = make_float2(a.ws.x, a.ws.x);     r.wsy = make_float2(a.ws.y, a.ws.y);
-          r.n0x = make_float2(a.n[0].x, a.n[0].x); r.n0y = make_float2(a.n[0].y, a.n[0].y);
-          r.n1x = make_float2(a.n[1].x, a.n[1].x); r.n1y = make_float2(a.n[1].y, a.n[1].y);
-          r.nn1y = make_float2(-a.n[1].y, -a.n[1].y);
-          r.p0x = make_float2(a.p[0].x, a.p[0].x); r.p0y = make_float2(a.p[0].y, a.p[0].y);
-          r.p1x = make_float2(a.p[1].x, a.p[1].x); r.p1y = make_float2(a.p[1].y, a.p[1].y);
-          return r;
-        };
-        // rays of columns (l, l + 1) of one row with paired FP32 operations
-        // (binary lens): component k is rounded exactly as ray_eval rounds
-        // ray l + k, operation by operation, so both give the same bits
-        auto ray_eval2 = [&](const AnchorP& a, float2 tx, float2 ty, float2 ri2, float2 dri2) -> float2 {
-          const float2 dzx = __ffma2_rn(ri2, tx, dri2), dzy = __fmul2_rn(ri2, ty);
-          const float2 ndzy = make_float2(-dzy.x, -dzy.y);
-          const float2 Fx = __fadd2_rn(a.p1x, dzx), Fy = __fadd2_rn(a.p1y, dzy);
-          const float2 Px = __ffma2_rn(dzx, Fx, __ffma2_rn(ndzy, Fy, a.p0x));
-          const float2 Py = __ffma2_rn(dzx, Fy, __ffma2_rn(dzy, Fx, a.p0y));
-          const float2 Nx = __ffma2_rn(a.n1x, dzx, __ffma2_rn(a.nn1y, dzy, a.n0x));
-          const float2 Ny = __ffma2_rn(a.n1x, dzy, __ffma2_rn(a.n1y, dzx, a.n0y));
-          const float2 q = __ffma2_rn(Px, Px, __fmul2_rn(Py, Py));
-          const float2 ip = make_float2(rcp_fast(q.x), rcp_fast(q.y));
-          const float2 m1 = __fmul2_rn(Nx, Py);
-          const float2 Vx = __ffma2_rn(Nx, Px, __fmul2_rn(Ny, Py));
-          const float2 Vy = __ffma2_rn(Ny, Px, make_float2(-m1.x, -m1.y));
-          const float2 m2 = __fmul2_rn(dzy, Vy);
-          const float2 pvx = __ffma2_rn(dzx, Vx, make_float2(-m2.x, -m2.y));
-          const float2 pvy = __ffma2_rn(dzx, Vy, __fmul2_rn(dzy, Vx));
-          const float2 dwx = __ffma2_rn(pvx, ip, __fadd2_rn(a.wsx, dzx));
-          const float2 dwy = __ffma2_rn(make_float2(-pvy.x, -pvy.y), ip, __fadd2_rn(a.wsy, dzy));
-          return __ffma2_rn(dwx, dwx, __fmul2_rn(dwy, dwy));
-        };
-        const float2 irho22 = make_float2(irho2, irho2), one2 = make_float2(1.0f, 1.0f);
-        const float2 c1f2 = make_float2(c1f, c1f), c2f2 = make_float2(c2f, c2f);
-        // the half-power coefficients, read only by the generic instantiation
-        const float2 c1h2 = LAW == 1 ? make_float2(sh.c1h, sh.c1h) : one2;
-        const float2 c3h2 = LAW == 1 ? make_float2(sh.c3h, sh.c3h) : one2;
-        // the queued points: one per lane, each re-evaluates its stencil
-        // (rays m - 2 .. m + 2, signed squared distances, negative inside)
-        auto flush_queue = [&]() {
-          __syncwarp();
-          if (lane < dq_n) {
-            const int2 q_ = dq[lane];
-            const int m = q_.x, irow = q_.y;
-            const int gi_ = irow / gr;
-            const float dri_ = ((float)(irow - gi_ * gr) + 0.5f - 0.5f * (float)gr) * dr32;
-            const float ri_ = (float)(B.r_lo + (gi_ * gr + 0.5 * gr) * sh.dr64) + dri_;
-            float sv[5], fsc = 1.f;
-#pragma unroll
-            for (int k = 0; k < 5; ++k) {
-              float d2;
-              const bool in = classify(gi_, ri_, dri_, irow, m - 2 + k, &d2, k == 2 ? &fsc : nullptr);
-              sv[k] = in ? __int_as_float(__float_as_int(d2) | 0x80000000) : d2;
-            }
-            if (signbit(sv[2])) {
-              const float I = brightness(-sv[2]);
-              float WU;
-              const float W = boundary_weight(0, sv, m, irow, nullptr, &WU);
-              const float rw = ri_ * bxw;
-              // literal rule: I (W - 1); split-profile rule: the limb value c0f
-              // with the uniform weight, the rest with f(delta)
-              // (a spot scales the point's whole brightness)
-              const float term = fsc * (split ? rw * (c0f * (WU - 1.0f) + (I - c0f) * (W - 1.0f)) : rw * I * (W - 1.0f));
-              const float y = term - acc_c;
-              const float tt = acc_s + y;
-              acc_c = (tt - acc_s) - y;
-              acc_s = tt;
-            }
-          }
-          __syncwarp();
-          dq_n = 0;
-        };
-        // static task order (warp, warp + NW, ...): the same sums in the same
-        // order on every run (dynamic assignment measured no faster)
-        for (int task = warp; task < ntask; task += NW) {
-          const int rbk = task / nch, chk = task - rbk * nch;
-          const int i = rbk * 32 + lane;
-          const bool rowok = i < NR;
-          const int ii = rowok ? i : NR - 1;
-          const int gi = ii / gr;
-          const float dri = ((float)(ii - gi * gr) + 0.5f - 0.5f * (float)gr) * dr32;
-          const float ri = (float)(B.r_lo + (gi * gr + 0.5 * gr) * sh.dr64) + dri;
-          const int c0 = chk * CH, c1 = min(c0 + CH, NTH);
-          // the row's inside rays: their count, and the sums of I - c0f =
-          // mu (c1f + c2f mu) of the scalar and of the paired evaluations
-          int cnt = 0;
-          float sj = 0.f;
-          float2 sj2 = make_float2(0.f, 0.f);
-          float dh;
-          // inside flags: bit k = column l - 1 - k before column l; the left
-          // halo column c0 - 1 first
-          unsigned win = classify(gi, ri, dri, ii, c0 - 1, &dh) ? 1u : 0u;
-          float lo2g = 0.f, hi2g = 0.f;  // the current group's band
-          int aidx = 0;                  // and its anchor
-          AnchorF ar;     // the anchor in registers (triple)
-          AnchorP ap;     // the anchor as broadcast pairs (binary)
-          // binary: the scalar evaluations read the anchor from the table
-          auto anchor = [&]() -> const AnchorF& {
-            if constexpr (NL == 2) return anf[aidx];
-            else return ar;
-          };
-          int gbase = 0;  // first column of the current group
-          const float* tpf = tabf;  // offsets of the current group: pair rows by column
-          const float2 ri2 = make_float2(ri, ri), dri2 = make_float2(dri, dri);
-          // queue the boundary points among bits of bm, bit j = column base - j
-          auto push_bits = [&](unsigned bm, int base) {
-            while (__any_sync(0xffffffffu, bm != 0u)) {
-              const bool has = bm != 0u;
-              const int m = base - (has ? __ffs(bm) - 1 : 0);
-              bm &= bm - 1u;
-              unsigned rem = __ballot_sync(0xffffffffu, has);
-              // up to 32 points, the queue holds DQ: take the lowest set
-              // lanes that fit, flushing whenever the queue is full
-              while (rem) {
-                if (dq_n == DQ) flush_queue();
-                unsigned take = rem;
-                const int room = DQ - dq_n;
-                if (__popc(take) > room) {
-                  take = 0u;
-                  unsigned r = rem;
-                  for (int k = 0; k < room; ++k) {
-                    const unsigned low = r & (0u - r);
-                    take |= low;
-                    r ^= low;
-                  }
-                }
-                if (take & (1u << lane)) dq[dq_n + __popc(take & lt_mask)] = make_int2(m, i);
-                dq_n += __popc(take);
-                rem &= ~take;
-              }
-            }
-          };
-          // boundary centres among columns l0 - 1 .. l0 + nb - 2 (bit j =
-          // column l0 + nb - 2 - j) after the block [l0, l0 + nb); the first
-          // block's column c0 - 1 belongs to the previous chunk
-          auto centres = [&](int nb, bool first) -> unsigned {
-            unsigned bm = ((win & ~((win << 1) & (win >> 1))) >> 1) & ((1u << nb) - 1u);
-            if (first) bm &= ~(1u << (nb - 1));
-            return rowok ? bm : 0u;
-          };
-          // an inside ray's share of the row beyond c0f: mu (c1f + c2f mu),
-          // plus s (c1h + c3h mu), s = mu^(1/2), when h (half-integer powers)
-          // fs: the spot factor (the count adds c0f, so a spotted ray adds
-          // fs (c0f + J) - c0f here)
-          auto add_in = [&](bool in, float mu, bool h, float fs) {
-            float J = mu * fmaf(c2f, mu, c1f);
-            if (h) J = fmaf(mu * rsqrt_fast(mu), fmaf(sh.c3h, mu, sh.c1h), J);
-            J = fmaf(fs, J, -c0f * (1.0f - fs));
-            sj = __fadd_rn(sj, in ? J : 0.0f);
-          };
-          auto block_end = [&](int l0, int nb, bool first, bool unc) {
-            unsigned bm = centres(nb, first);
-            if (__any_sync(0xffffffffu, unc || bm != 0u)) {
-              if (unc) {
-                for (int k = 0; k < nb; ++k) {
-                  const cf t = tab_at(l0 + k - gbase);
-                  float eb;
-                  cf dw;
-                  float d2 = ray_eval(anchor(), t.x, t.y, ri, dri, &eb, nullptr, &dw);
-                  if (d2 < lo2g || d2 > hi2g) continue;
-                  if (decide(d2, eb, ii, l0 + k)) {
-                    win |= 1u << (nb - 1 - k);
-                    add_in(true, sqrtf(fmaxf(__fmaf_rn(-d2, irho2, 1.0f), 1e-30f)), LAW != 0 && sh.half != 0,
-                           spot_factor(aidx, dw, eb, ii, l0 + k));
-                  }
-                }
-                bm = centres(nb, first);
-              }
-              push_bits(bm, l0 + nb - 2);
-            }
-            cnt += __popc(win & ((1u << nb) - 1u));
-          };
-          // one column: classify against the band, flag, and if inside add
-          // its share (x > 5 u there, as d^2 < lo2 <= rho^2 (1 - 8 u)); hc:
-          // std::true_type for the generic law (half-integer powers of mu or
-          // a spot, checked at run time)
-          auto col = [&](int l, float tx, float ty, bool& unc, auto hc) {
-            cf dw;
-            float eb = 0.f;
-            constexpr bool GEN = decltype(hc)::value;
-            const float d2 = ray_eval(anchor(), tx, ty, ri, dri, GEN ? &eb : nullptr, nullptr, GEN ? &dw : nullptr);
-            const bool in = d2 < lo2g;
-            unc = unc || !(in || d2 > hi2g);
-            win = (win << 1) | (in ? 1u : 0u);
-            const float x = __fmaf_rn(-d2, irho2, 1.0f);
-            if constexpr (GEN)
-              add_in(in, __fmul_rn(x, rsqrt_fast(x)), sh.half != 0, in ? spot_factor(aidx, dw, eb, ii, l) : 1.0f);
-            else
-              add_in(in, __fmul_rn(x, rsqrt_fast(x)), false, 1.0f);
-            (void)l;
-          };
-          // two columns (l, l + 1) with paired operations (binary lens); the
-          // pair row t4 = (x_l, x_l+1, y_l, y_l+1); hh: std::true_type adds the
-          // half-integer powers s (c1h + c3h mu), s = mu^(1/2) (no spot)
-          auto col2 = [&](const float4 t4, bool& unc, auto hh) {
-            const float2 d2 = ray_eval2(ap, make_float2(t4.x, t4.y), make_float2(t4.z, t4.w), ri2, dri2);
-            const bool in0 = d2.x < lo2g, in1 = d2.y < lo2g;
-            unc = unc || !(in0 || d2.x > hi2g) || !(in1 || d2.y > hi2g);
-            win = (win << 2) | (in0 ? 2u : 0u) | (in1 ? 1u : 0u);
-            const float2 x = __ffma2_rn(make_float2(-d2.x, -d2.y), irho22, one2);
-            const float2 mu = __fmul2_rn(x, make_float2(rsqrt_fast(x.x), rsqrt_fast(x.y)));
-            float2 J = __fmul2_rn(mu, __ffma2_rn(c2f2, mu, c1f2));
-            if constexpr (decltype(hh)::value) {
-              const float2 sq = __fmul2_rn(mu, make_float2(rsqrt_fast(mu.x), rsqrt_fast(mu.y)));
-              J = __ffma2_rn(sq, __ffma2_rn(c3h2, mu, c1h2), J);
-            }
-            sj2 = __fadd2_rn(sj2, make_float2(in0 ? J.x : 0.0f, in1 ? J.y : 0.0f));
-          };
-          int l = c0;
-          bool first = true;
-          while (l < c1) {
-            const int mgrp = (int)__umulhi((unsigned int)l, gmagic);
-            aidx = gi * mth + mgrp;
-            lo2g = anf[aidx].lo2;
-            hi2g = anf[aidx].hi2;
-            if constexpr (NL == 2) ap = pairs_of(anf[aidx]);
-            else ar = anf[aidx];
-            gbase = mgrp * gth;
-            tpf = tabf - 2 * gbase;
-            const int lend = min(gbase + gth, c1);
-            while (l < lend) {
-              const int nb = min(KB, lend - l);
-              bool unc = false;
-              // a full block, columns l + k, l + k + 1 from one 16-byte row
-              // (l + k - gbase even); hc selects the half-power terms
-              auto full_block = [&](auto hc) {
-#pragma unroll
-                for (int k = 0; k < KB; k += 2) {
-                  const float4 t4 = *reinterpret_cast<const float4*>(tpf + 2 * (l + k));
-                  if constexpr (NL == 2) {
-                    col2(t4, unc, hc);
-                  } else {
-                    col(l + k, t4.x, t4.z, unc, hc);
-                    col(l + k + 1, t4.y, t4.w, unc, hc);
-                  }
-                }
-              };
-              // (a spot, or the half-integer powers outside the generic
-              // instantiation's paired sweep: the scalar loop)
-              if (nb == KB && (LAW == 0 || !sh.generic)) {
-                full_block(std::false_type{});
-              } else if (LAW == 1 && NL == 2 && nb == KB && !sh.spot) {
-                full_block(std::true_type{});
-              } else {
-#pragma unroll 1
-                for (int k = 0; k < nb; ++k) {
-                  const cf t = tab_at(l + k - gbase);
-                  if (LAW != 0 && sh.generic) col(l + k, t.x, t.y, unc, std::true_type{});
-                  else col(l + k, t.x, t.y, unc, std::false_type{});
-                }
-              }
-              block_end(l, nb, first, unc);
-              first = false;
-              l += nb;
-            }
-          }
-          // right halo column c1: finalizes column c1 - 1
-          win = (win << 1) | (classify(gi, ri, dri, ii, c1, &dh) ? 1u : 0u);
-          push_bits(rowok ? (((win & ~((win << 1) & (win >> 1))) >> 1) & 1u) : 0u, c1 - 1);
-          if (rowok) {
-            const float rowacc = c0f * (float)cnt + (sj + (sj2.x + sj2.y));
-            const float term = ri * rowacc * bxw;
-            const float y = term - acc_c;
-            const float tt = acc_s + y;
-            acc_c = (tt - acc_s) - y;
-            acc_s = tt;
-          }
-        }
-        flush_queue();
-        } else {
+        {
           // ---- derivative ray stage (binary lens).  Per ray with seed a =
           // dRow/dd (dI/dd inside; the paper's sigmoid rule adds its own),
           // the row's sums pg[k] += a dd/dq_k are taken from the ray's FP32
@@ -2518,9 +2371,11 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
       }
     }
     if (st_local) atomicOr(&sh.status, st_local);
+    raysum = (double)acc_s - (double)acc_c;
+    }
     if (diag_cnt && tid == 0) { long long c_ = clock64(); sh.cnt[12] = (int)min(c_ - sh.clk0, 2000000000LL); sh.clk0 = c_; }
     // ------------------------------------------------ 10. reduction
-    double v = (double)acc_s - (double)acc_c;
+    double v = raysum;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (lane == 0) sh.red[warp] = v;
     __syncthreads();
@@ -2676,21 +2531,21 @@ marginal_nll_kernel(const double* __restrict__ A, const double* __restrict__ F, 
 }
 
 // ---------------------------------------------------------------- host side
-static size_t mag_smem_bytes(int NL, const icrs_grid& g, int pmax, int has_plo, bool der, int defer, int nt) {
+// Columns of the ray stage's offset tables: every sector of an epoch at once
+// (forward), one sector (derivative).
+static int mag_tabcap(int NL, bool der) { return der ? GTH_MAX + 2 : (NL * NL + 1) * (GTH_MAX + 2); }
+
+static size_t mag_smem_bytes(int NL, const icrs_grid& g, int pmax, int has_plo, bool der, int nt) {
   const int N = NL * NL + 1;
   const size_t NP = (size_t)g.n_limb * N;
-  size_t b = has_plo ? sizeof(cf) * NP : 0;
-  b += sizeof(cf) * NP + 4 * sizeof(float) * NP;
-  b += sizeof(short) * ((NP + 7) & ~(size_t)7);
-  b += 3 * ((NP + 15) & ~(size_t)15);
-  b += 2 * sizeof(double) * pmax + sizeof(int) * QMAX + 16 + (sizeof(AnchorF) + sizeof(float2)) * MAXANCH;
-  const int NW = nt / 32;
-  (void)defer;
-  b += sizeof(int) * NW * 2 * dq_entries(NL);  // per-warp boundary queues
+  size_t b = sizeof(cf) * NP * (has_plo ? 2 : 1) + sizeof(cdf) * g.n_limb + 16;
   if (der) b += sizeof(DerShared);               // derivative state
-  b += sizeof(cf) * (GTH_MAX + 2);
-  b += sizeof(cdf) * g.n_limb;
-  return b;
+  // image-limb slots; the ray stage's tables take their place
+  size_t slots = 4 * sizeof(float) * NP + sizeof(short) * ((NP + 7) & ~(size_t)7) + 3 * ((NP + 15) & ~(size_t)15);
+  slots += 2 * sizeof(double) * pmax + sizeof(int) * QMAX;
+  const size_t rays = sizeof(cf) * mag_tabcap(NL, der) + (sizeof(AnchorF) + sizeof(float2)) * MAXANCH +
+                      sizeof(int) * (nt / 32) * DQ * (der ? 2 : 1);
+  return b + (slots > rays ? slots : rays);
 }
 
 static int check_grid(const icrs_grid* g) {
@@ -2729,7 +2584,7 @@ template <int NL, bool DER, int NTB, int LAW>
 static int launch_nt(const icrs_params* p, int S, const double* t, int E, const icrs_grid* g, double* A,
                      uint32_t* status, double* dsect, int32_t* dcnt, float* dpts, const DerOut& dout,
                      cudaStream_t st, const int32_t* items, int n_items, int nsm, size_t smem, int pmax,
-                     int has_plo, int defer) {
+                     int has_plo) {
   if (cudaFuncSetAttribute(mag_kernel<NL, DER, NTB, LAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return ICRS_ECUDA;
@@ -2743,17 +2598,15 @@ static int launch_nt(const icrs_params* p, int S, const double* t, int E, const 
   if (per_block < 1) per_block = 1;
   long long blocks = (tiles + per_block - 1) / per_block;
   mag_kernel<NL, DER, NTB, LAW><<<(unsigned)blocks, NTB, smem, st>>>(p, S, t, E, *g, (int)per_block, A, status,
-                                                                      dsect, dcnt, dpts, pmax, has_plo, dout, items,
-                                                                      n_items, defer);
+                                                                      dsect, dcnt, dpts, pmax, has_plo,
+                                                                      mag_tabcap(NL, DER), dout, items, n_items);
   return cudaGetLastError() == cudaSuccess ? ICRS_OK : ICRS_ECUDA;
 }
 
-// Shared-memory sizing of one (NL, DER) launch: the block size (the
-// preferred one, else 512 threads when the preferred layout does not fit),
-// the deferred boundary queue (binary forward) if it fits; then, forward,
-// the FP64 point table grows (up to one entry per image-limb slot) before
-// the lo parts of image positions are added; derivative mode takes the lo
-// parts first (fewer FP64 polishes).
+// Shared-memory sizing of one (NL, DER) launch: forward, the FP64 point table
+// grows (up to one entry per image-limb slot) before the lo parts of image
+// positions are added; derivative mode takes the lo parts first (fewer FP64
+// polishes).
 template <int NL, bool DER, int LAW>
 static int launch_inst(const icrs_params* p, int S, const double* t, int E, const icrs_grid* g, double* A,
                        uint32_t* status, double* dsect, int32_t* dcnt, float* dpts, const DerOut& dout,
@@ -2763,39 +2616,24 @@ static int launch_inst(const icrs_params* p, int S, const double* t, int E, cons
   int optin = 0, nsm = 0;
   if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return ICRS_ECUDA;
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return ICRS_ECUDA;
-  int nt = mag_threads(NL, DER);
-  auto fits = [&](int pm, int plo, int df) {
-    return mag_smem_bytes(NL, *g, pm, plo, DER, df, nt) + sizeof(Shared) <= (size_t)optin;
+  // shared memory beside the dynamic part
+  cudaFuncAttributes fa;
+  if (cudaFuncGetAttributes(&fa, mag_kernel<NL, DER, NT_BASE, LAW>) != cudaSuccess) return ICRS_ECUDA;
+  auto fits = [&](int pm, int plo) {
+    return mag_smem_bytes(NL, *g, pm, plo, DER, NT_BASE) + fa.sharedSizeBytes <= (size_t)optin;
   };
   int pmax = PMAX_MIN;
-  int defer = (NL == 2 && !DER) ? 1 : 0;
-  if (!fits(pmax, 0, defer)) defer = 0;
-  if (!fits(pmax, 0, defer) && nt != NT_BASE) {
-    nt = NT_BASE;
-    defer = (NL == 2 && !DER) ? 1 : 0;
-    if (!fits(pmax, 0, defer)) defer = 0;
-  }
-  if (!fits(pmax, 0, defer)) return ICRS_EUNSUPPORTED;
-  int has_plo = (DER && fits(pmax, 1, defer)) ? 1 : 0;
+  if (!fits(pmax, 0)) return ICRS_EUNSUPPORTED;
+  int has_plo = (DER && fits(pmax, 1)) ? 1 : 0;
   const int np_all = g->n_limb * (NL * NL + 1);
   // the FP64 point table takes the remaining room (16 bytes per entry), up to
   // one entry per image-limb slot
-  {
-    const size_t used = mag_smem_bytes(NL, *g, 0, has_plo, DER, defer, nt) + sizeof(Shared);
-    const size_t room = used < (size_t)optin ? (size_t)optin - used : 0;
-    const size_t cap = room / (2 * sizeof(double));
-    pmax = (int)(cap < (size_t)np_all ? cap : (size_t)np_all);
-    if (pmax < PMAX_MIN) pmax = PMAX_MIN;
-  }
-  if (!DER) has_plo = fits(pmax, 1, defer) ? 1 : 0;
-  const size_t smem = mag_smem_bytes(NL, *g, pmax, has_plo, DER, defer, nt);
-  if constexpr (mag_threads(NL, DER) != NT_BASE) {
-    if (nt == mag_threads(NL, DER))
-      return launch_nt<NL, DER, mag_threads(NL, DER), LAW>(p, S, t, E, g, A, status, dsect, dcnt, dpts, dout, st,
-                                                           items, n_items, nsm, smem, pmax, has_plo, defer);
-  }
+  pmax = np_all < PMAX_MIN ? PMAX_MIN : np_all;
+  while (pmax > PMAX_MIN && !fits(pmax, has_plo)) pmax = pmax - 64 > PMAX_MIN ? pmax - 64 : PMAX_MIN;
+  if (!DER) has_plo = fits(pmax, 1) ? 1 : 0;
+  const size_t smem = mag_smem_bytes(NL, *g, pmax, has_plo, DER, NT_BASE);
   return launch_nt<NL, DER, NT_BASE, LAW>(p, S, t, E, g, A, status, dsect, dcnt, dpts, dout, st, items, n_items, nsm,
-                                          smem, pmax, has_plo, defer);
+                                          smem, pmax, has_plo);
 }
 
 // Binary forward: the linear instantiation, then the generic one (each takes

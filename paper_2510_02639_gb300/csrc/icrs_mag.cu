@@ -35,6 +35,7 @@
 #include "icrs_sectors.cuh"
 #include "icrs_ps.cuh"
 #include "icrs_rays.cuh"
+#include "icrs_rays_der.cuh"
 
 namespace icrs {
 
@@ -125,11 +126,6 @@ struct Shared {
   int cnt[16];         // diagnostics: FP64 polishes, FP64 validations, FP64 rays, FP64 crossings, phase clocks
   long long clk0;
   // ---- ray stage (current sector)
-  int mth, mr, gth, gr;
-  double dr64, dth64;
-  float dr32, dth32;
-  int nanch;
-  int chunk;           // columns per theta chunk
   double red[NW_MAX];
 };
 
@@ -144,9 +140,6 @@ struct DerShared {
   double depsq[2];          // d eps_j / d q
   DualD cx[MAXCELL_D * 4];  // cell extremes with tangents
   BoxT<DualD> box[MAXBOX_D];  // sectors with tangents
-  double wder[NW_DER][12];      // per-warp sums of the row derivatives
-  float2 acs[MAXANCH];      // cos, sin of each anchor angle
-  float4 aA[MAXANCH];       // A_0, A_1 of each anchor (FP32)
 };
 
 // Order-preserving integer keys for signed FP32 / FP64 values.
@@ -247,30 +240,6 @@ __device__ inline int validate_root64(const Shared& sh, cd z0, cd w, double img_
   return 1;
 }
 
-// FP64 offset of ray (i, l) of a sector from the source centre (and its
-// distance below), with the grid of Sec. 3.3: r_i = r_lo + (i + 1/2) dr,
-// th_l = th_lo + (l + 1/2) dth.  Out of line: these are the rare fallbacks,
-// and inlined they cost the ray sweeps registers.
-template <int NL>
-__device__ __noinline__ cd ray_offset64(const Shared& sh, const Box& B, int i, int l) {
-  double r = B.r_lo + (i + 0.5) * sh.dr64;
-  double th = B.th_lo + (l + 0.5) * sh.dth64;
-  double s, c;
-  sincos(th, &s, &c);
-  cd z = mk(r * c, r * s);
-  return lens_map<NL, double>(sh.L.eps, sh.L.a, z) - sh.wc;
-}
-template <int NL>
-__device__ __noinline__ double ray_distance64(const Shared& sh, const Box& B, int i, int l) {
-  double r = B.r_lo + (i + 0.5) * sh.dr64;
-  double th = B.th_lo + (l + 0.5) * sh.dth64;
-  double s, c;
-  sincos(th, &s, &c);
-  cd z = mk(r * c, r * s);
-  cd w = lens_map<NL, double>(sh.L.eps, sh.L.a, z);
-  return sqrt(abs2(w - sh.wc));
-}
-
 // Sine of the angle from direction X to the angle th, in FP64 (out of line: a
 // rare fallback).
 __device__ __noinline__ float sine_from64(float2 X, double th) {
@@ -312,30 +281,6 @@ __device__ inline void point_tangents(const Shared& sh, const DerShared& ds, dou
     dr[q] = (z.x * dx + z.y * dy) / r;
     dth[q] = (z.x * dy - z.y * dx) / (r * r);
   }
-}
-
-// Lagrange basis of the nodes 0 .. npt-1 (npt = 2..4) at t, and the slope
-// of the interpolant through y there.
-template <class T>
-__device__ inline T lagrange_basis(const T* y, int npt, T t, T* l) {
-  const T d1 = y[1] - y[0];
-  const T d2 = npt > 2 ? T(0.5) * (y[2] - T(2) * y[1] + y[0]) : T(0);
-  const T d3 = npt > 3 ? (y[3] - T(3) * y[2] + T(3) * y[1] - y[0]) * T(1.0 / 6.0) : T(0);
-  const T t1 = t - T(1), t2 = t - T(2), t3 = t - T(3);
-  if (npt == 4) {
-    l[0] = -t1 * t2 * t3 * T(1.0 / 6.0);
-    l[1] = T(0.5) * t * t2 * t3;
-    l[2] = T(-0.5) * t * t1 * t3;
-    l[3] = t * t1 * t2 * T(1.0 / 6.0);
-  } else if (npt == 3) {
-    l[0] = T(0.5) * t1 * t2;
-    l[1] = -t * t2;
-    l[2] = T(0.5) * t * t1;
-  } else {
-    l[0] = -t1;
-    l[1] = t;
-  }
-  return d1 + (T(2) * t - T(1)) * d2 + ((T(3) * t - T(6)) * t + T(2)) * d3;
 }
 
 // FP64 re-solve of limb point k (all roots, FP64 Ehrlich-Aberth warm-started
@@ -387,19 +332,6 @@ __device__ __forceinline__ void q_push(Shared& sh, int* queue, int v) {
   else atomicOr(&sh.status, ICRS_ST_OVERFLOW);
 }
 
-// ---------------------------------------------------------------- quadrature
-// f'(delta) of fdelta.
-template <class T>
-__device__ __forceinline__ T fdelta_prime(T d, T delta_c, int uniform) {
-  if (uniform) return T(1);
-  if (d >= delta_c) {
-    T h = T(1) + T(1) / (T(2) * d);
-    T sq = sqrt(h);
-    return T(2.0 / 3.0) * sq - (T(0.5) + d) / (T(6) * d * d * sq);
-  }
-  return T(2.0 / 3.0);
-}
-
 // ---------------------------------------------------------------- kernel
 // A set whose law has half-integer powers of mu (a1 or a3, on a limb-darkened
 // grid) or a spot: the binary forward launch gives these sets to the kernel's
@@ -430,14 +362,15 @@ __global__ void __launch_bounds__(NTB, 1)
 mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ T_, int E,
            icrs_grid g, int tiles_per_block, double* __restrict__ A_out, uint32_t* __restrict__ st_out,
            double* __restrict__ diag_sect, int32_t* __restrict__ diag_cnt, float* __restrict__ diag_pts, int PMAX,
-           int has_plo, int tabcap, DerOut dout, const int32_t* __restrict__ items, int n_items) {
+           int has_plo, int tabcap, int ccap, DerOut dout, const int32_t* __restrict__ items, int n_items) {
   constexpr int N = NL * NL + 1;
   constexpr int NT = NTB;
   constexpr int NW = NT / 32;
   static_assert(NT % 32 == 0 && NW <= NW_MAX && (!DER || NW == NW_DER), "per-warp tables are sized for these block sizes");
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ Shared sh;
-  __shared__ typename std::conditional<DER, char, RayShared>::type rays_sh;
+  __shared__ RayShared rays_sh;
+  __shared__ typename std::conditional<DER, DerRays, char>::type der_sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = g.n_limb, NP = K * N;
   const int BT = g.n_bins_theta, BR = g.n_bins_r;
@@ -456,10 +389,9 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
   // nothing reads once the sectors stand (16-byte rows of the offset table)
   unsigned char* pr_ = p;
   float* tabf = (float*)pr_;     pr_ += sizeof(cf) * tabcap;        // group offsets (cos d - 1, sin d)
-  cf* tab = (cf*)tabf;
   AnchorF* anch = (AnchorF*)pr_; pr_ += sizeof(AnchorF) * MAXANCH;
   float2* spc = (float2*)pr_;    pr_ += sizeof(float2) * MAXANCH;  // spot centre in each anchor's frame
-  int* wqueue = (int*)pr_;       // boundary points, a queue per warp
+  int* wqueue = (int*)pr_;       pr_ += sizeof(int) * NW * DQ;     // boundary points, a queue per warp
   float* r32 = (float*)p;        p += sizeof(float) * NP;
   float* rl32 = (float*)p;       p += sizeof(float) * NP;   // r = r32 + rl32 (double-float)
   float* t32 = (float*)p;        p += sizeof(float) * NP;
@@ -473,16 +405,20 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
   uint8_t* rb = (uint8_t*)p;     p += (NP + 15) & ~15;
   DualD* cdual = ds.cx;
   BoxT<DualD>* bdual = ds.box;
-  double* wder = &ds.wder[0][0];
 
   if (tid == 0) {
     sh.cur_set = -1;
     sh.warm = 0;
     sh.ht = 2.0 * kPi / BT;
     sh.htf = (float)sh.ht;
-    if constexpr (!DER)
-      rays_sh.P = {anch, spc, tabf, wqueue, tabcap, g.n_r, g.n_theta, g.uniform, g.ld_split && !g.uniform ? 1 : 0,
-                   diag_cnt ? 1 : 0, 1.0f, g.delta_c};
+    if constexpr (DER) {
+      float4* aA = (float4*)pr_;
+      float2* acs = (float2*)(aA + MAXANCH), *sums = acs + MAXANCH;
+      double* ws = (double*)(sums + NW * DSUM * 32);
+      der_sh = {acs, aA, sums, ws, ccap ? (double2*)(ws + 5 * DSUM * TASK_WARPS) : nullptr};
+    }
+    rays_sh.P = {anch, spc, tabf, wqueue, tabcap, ccap, g.n_r, g.n_theta, g.uniform, g.ld_split && !g.uniform ? 1 : 0,
+                 diag_cnt ? 1 : 0, 1.0f, (float)g.s_fac, g.grad_rule, g.delta_c};
   }
   for (int k = tid; k < K; k += NT) {
     double sn, cs;
@@ -596,8 +532,6 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
         ds.dadp[1][0] = 1.0 / oq;    ds.dadp[1][1] = -pp.s / (oq * oq);
         ds.depsq[0] = -1.0 / (oq * oq);
         ds.depsq[1] = 1.0 / (oq * oq);
-        for (int b = 0; b < MAXBOX_D; ++b) for (int k = 0; k < 4; ++k) ds.Gb[b][k] = 0.0;
-        for (int k = 0; k < 8; ++k) ds.H[k] = 0.0;
       }
       for (int j = 0; j < NL; ++j) {
         cd d = sh.wc - sh.L.a[j];
@@ -1605,8 +1539,6 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
       }
       sh.nbox = nb;
     }
-    if (DER)
-      for (int k = tid; k < NW * 12; k += NT) wder[k] = 0.0;
     __syncthreads();
 
     if (diag_cnt && tid == 0) { long long c_ = clock64(); sh.cnt[11] = (int)min(c_ - sh.clk0, 2000000000LL); sh.clk0 = c_; }
@@ -1615,763 +1547,8 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     if constexpr (!DER) {
       raysum = ray_stage<NL, LAW>(sh, rays_sh);
     } else {
-    const int NR = g.n_r, NTH = g.n_theta;
-    // the set's brightness law (see the set-up)
-    const float I0 = sh.I0, c0f = sh.c0f, c1f = sh.c1f, c2f = sh.c2f;
-    const float irho2 = 1.0f / (rho32 * rho32);
-    const float irho = 1.0f / rho32;
-    const float dcf = (float)g.delta_c;
-    const float sfac = (float)g.s_fac;            // sigmoid steepness of the paper's gradient rule
-    float acc_s = 0.f, acc_c = 0.f;  // Kahan sum of this thread
-    uint32_t st_local = 0u;
-    for (int bxi = 0; bxi < sh.nbox; ++bxi) {
-      const Box B = sh.box[bxi];
-      if (tid == 0) {
-        sh.dr64 = (B.r_hi - B.r_lo) / NR;
-        sh.dth64 = B.width / NTH;
-        sh.dr32 = (float)sh.dr64;
-        sh.dth32 = (float)sh.dth64;
-        // anchors: enough groups that an anchor is within ~0.025 of its rays
-        const double LMAX = 0.05;
-        int mth = (int)ceil(B.r_hi * B.width / LMAX);
-        int mr = (int)ceil((B.r_hi - B.r_lo) / LMAX);
-        mth = min(max(mth, 1), min(64, NTH));
-        // groups of at most GTH_MAX columns (the offset table's size; for
-        // n_theta <= 8192 this needs at most 32 groups)
-        mth = max(mth, (NTH + GTH_MAX - 1) / GTH_MAX);
-        mr = min(max(mr, 1), min(4, NR));
-        mth = min(mth, MAXANCH / mr);  // the anchor table holds MAXANCH entries
-        // theta groups of an even width: the forward ray stage evaluates
-        // column pairs (l, l + 1), l even, which then share their group
-        sh.gth = 2 * ((NTH + 2 * mth - 1) / (2 * mth));
-        sh.gr = (NR + mr - 1) / mr;
-        sh.mth = (NTH + sh.gth - 1) / sh.gth;
-        sh.mr = (NR + sh.gr - 1) / sh.gr;
-        sh.nanch = sh.mth * sh.mr;
-        // ray stage: tasks of 32 rows (one per lane) x a theta chunk
-        // of an even number of columns, about 8 tasks per warp per sector
-        const int nrb = (NR + 31) >> 5;
-        const int nch = max(1, (8 * NW + nrb - 1) / nrb);
-        sh.chunk = min(NTH, max(16, 2 * ((NTH + 2 * nch - 1) / (2 * nch))));
-      }
-      __syncthreads();
-      const int gth = sh.gth, gr = sh.gr, mth = sh.mth;
-      // group of ray l: l / gth as a multiply-high by ceil(2^32 / gth), exact
-      // for l, gth < 2^16 (here both <= 8192)
-      const unsigned int gmagic = (unsigned int)((0xFFFFFFFFull / (unsigned long long)gth) + 1ull);
-      // anchors (FP64, one per thread)
-      for (int an = tid; an < sh.nanch; an += NT) {
-        int gi = an / mth, mi = an % mth;
-        double rc = B.r_lo + (gi * gr + 0.5 * gr) * sh.dr64;
-        double thc = B.th_lo + (mi * gth + 0.5 * gth) * sh.dth64;
-        double sn, cs;
-        sincos(thc, &sn, &cs);
-        cd R = mk(cs, -sn);  // e^{-i th_c}
-        cd zc = mk(rc * cs, rc * sn);
-        cd wsd = lens_map<NL, double>(sh.L.eps, sh.L.a, zc) - sh.wc;
-        const cf ws = tof(R * wsd);
-        if (LAW != 0 && sh.spot) spc[an] = make_float2((float)(sh.rho * (cs * sh.spot_x + sn * sh.spot_y)),
-                                           (float)(sh.rho * (cs * sh.spot_y - sn * sh.spot_x)));
-        // error bound of |Delta w'|: anchor term plus rounding of the ray's
-        // offset (at most the group half-diagonal) and of its image term
-        const double half = 0.5 * gr * sh.dr64 + (B.r_hi) * 0.5 * gth * sh.dth64;
-        const float e0 = (float)(16.0 * EPS32 * (fabs(ws.x) + fabs(ws.y) + 2.0 * half));
-        const double rr = (double)rho32 * (double)rho32;
-        float lo2 = -1.0f, hi2 = __int_as_float(0x7f800000);
-        {
-          // U = N / P (AnchorF), coefficients from the FP64 A_j, K_j
-          cd A64[NL], K64[NL];
-          for (int j = 0; j < NL; ++j) {
-            A64[j] = R * (zc - sh.L.a[j]);
-            K64[j] = scl(inv(A64[j]), sh.L.eps[j]);
-          }
-          cd nc[3], pc[3];
-          if constexpr (NL == 2) {
-            nc[0] = K64[0] * A64[1] + K64[1] * A64[0];
-            nc[1] = K64[0] + K64[1];
-            nc[2] = mk(0.0, 0.0);
-            pc[0] = A64[0] * A64[1];
-            pc[1] = A64[0] + A64[1];
-            pc[2] = mk(0.0, 0.0);
-          } else {
-            nc[0] = K64[0] * (A64[1] * A64[2]) + K64[1] * (A64[0] * A64[2]) + K64[2] * (A64[0] * A64[1]);
-            nc[1] = K64[0] * (A64[1] + A64[2]) + K64[1] * (A64[0] + A64[2]) + K64[2] * (A64[0] + A64[1]);
-            nc[2] = K64[0] + K64[1] + K64[2];
-            pc[0] = A64[0] * A64[1] * A64[2];
-            pc[1] = A64[0] * A64[1] + A64[0] * A64[2] + A64[1] * A64[2];
-            pc[2] = A64[0] + A64[1] + A64[2];
-          }
-          AnchorF af;
-          af.ws = ws;
-          for (int k = 0; k < 3; ++k) { af.n[k] = tof(nc[k]); af.p[k] = tof(pc[k]); }
-          af.e0 = e0;
-          // the group's band: every ray has |dz| <= half, so |Q_j| >= |A_j| -
-          // half, |P| >= prod_j (|A_j| - half) and |U| <= sum_j |K_j| / (|A_j|
-          // - half); the rounding error of the FP32 quotient is bounded by
-          // u (cN M_N + (cP + 9) |U| M_P) / |P| (M_N, M_P: the polynomials
-          // with coefficient moduli, at |dz| = half) and that of dz U by
-          // |dz| (that + 3 u |U|), times 2 for the FP32 evaluation of the
-          // bound itself (see ray_eval)
-          bool bounded = true;
-          double um = 0.0, pmin = 1.0;
-          for (int j = 0; j < NL; ++j) {
-            const double aa = sqrt(abs2(A64[j]));
-            if (!(aa > 1.0625 * half)) bounded = false;
-            else { um += sqrt(abs2(K64[j])) / (aa - half); pmin *= aa - half; }
-          }
-          if (bounded) {
-            const double mn = sqrt(abs2(nc[0])) + half * (sqrt(abs2(nc[1])) + half * sqrt(abs2(nc[2])));
-            const double mp = NL == 2 ? sqrt(abs2(pc[0])) + half * (sqrt(abs2(pc[1])) + half)
-                                      : sqrt(abs2(pc[0])) + half * (sqrt(abs2(pc[1])) + half * (sqrt(abs2(pc[2])) + half));
-            const double cN = NL == 2 ? 4.0 : 9.0, cP = NL == 2 ? 6.0 : 13.0;
-            const double du = EPS32 * (cN * mn + (cP + 9.0) * um * mp) / pmin;
-            const double eb = (double)e0 + 2.0 * half * (du + 3.0 * EPS32 * um);
-            const double X = 1.01 * (2.0 * (double)rho32 * eb + eb * eb) + 8.0 * EPS32 * rr;
-            if (X < 0.5 * rr) {
-              lo2 = __double2float_rd(rr - X);
-              hi2 = __double2float_ru(rr + X);
-            }
-          }
-          af.lo2 = lo2;
-          af.hi2 = hi2;
-          anch[an] = af;
-          if constexpr (DER) {
-            // the adjoint's ray gradients: A_j in FP32 and the anchor angle
-            ds.aA[an] = make_float4((float)A64[0].x, (float)A64[0].y, (float)A64[1].x, (float)A64[1].y);
-            ds.acs[an] = make_float2((float)cs, (float)sn);
-          }
-        }
-      }
-      // offsets within a theta group, (cos d - 1, sin d) with d = (o + 1/2 -
-      // gth/2) dth; column pairs (o, o + 1), o even, are stored as 16 bytes
-      // (x_o, x_o+1, y_o, y_o+1), so that the forward ray stage loads a pair's
-      // x and y as two adjacent float2 (gth is even)
-      float* tabf = reinterpret_cast<float*>(tab);
-      for (int o = tid; o < gth; o += NT) {
-        float d = ((float)o + 0.5f - 0.5f * (float)gth) * sh.dth32;
-        float s, c;
-        sincosf(d, &s, &c);
-        float sh2 = sinf(0.5f * d);
-        tabf[4 * (o >> 1) + (o & 1)] = -2.0f * sh2 * sh2;
-        tabf[4 * (o >> 1) + 2 + (o & 1)] = s;
-        (void)c;
-      }
-      __syncthreads();
-      auto tab_at = [&](int o) -> cf {
-        const float* t_ = tabf + 4 * (o >> 1) + (o & 1);
-        return mk(t_[0], t_[2]);
-      };
-      const float dr32 = sh.dr32;
-      const float bxw = (float)(sh.dr64 * sh.dth64);
-      auto wrapl = [&](int l) -> int { return l < 0 ? l + NTH : (l >= NTH ? l - NTH : l); };
-      // per-point weights (Appendix A).  Points with both neighbours
-      // inside (W = 1) are summed directly; points next to the image
-      // boundary are queued per warp and their crossings solved with one
-      // point per lane.
-      // I(d) = c0f + c1f mu + c2f mu^2, mu^2 = x = 1 - d^2/rho^2
-      auto brightness = [&](float d2) -> float {
-        const float x = fmaxf(fmaf(-d2, irho2, 1.0f), 1e-30f);
-        const float mu = x * rsqrtf(x);
-        float I = fmaf(c2f, x, fmaf(c1f, mu, c0f));
-        if (LAW != 0 && sh.half) I = fmaf(sqrtf(mu), fmaf(sh.c3h, mu, sh.c1h), I);
-        return I;
-      };
-      // I and dI/dd, dI/drho, dI/du1 at squared distance d2:
-      //   dI/dx = c1/(2 mu) + c2, dx/dd = -2 d/rho^2, dx/drho = 2 d^2/rho^3,
-      //   dI/du1 = I (pi/3) I0 - I0 (1 - mu)   (dI0/du1 = (pi/3) I0^2)
-      // (hc: std::true_type for the generic law: half-integer powers of mu
-      // checked at run time)
-      auto brightness_der = [&](float d2, float* Id, float* Ir, float* Iu, auto hc) -> float {
-        if (g.uniform) { *Id = 0.f; *Ir = 0.f; *Iu = 0.f; return I0; }
-        // (hardware reciprocal square roots: 2^-22.9 relative, far inside
-        // the derivative's tolerance)
-        float x = fmaxf(0.f, 1.0f - d2 * irho2);
-        const float rs = x > 0.f ? rsqrt_fast(x) : 0.f;  // 1 / mu
-        float sx = x * rs;
-        float I = c0f + c1f * sx + c2f * x;
-        float d = d2 * rsqrt_fast(fmaxf(d2, 1e-37f));
-        // k = (dI/dmu) / mu / rho^2
-        float k = x > 0.f ? (c1f * rs + 2.0f * c2f) * irho2 : 0.f;
-        if constexpr (decltype(hc)::value) {
-          if (LAW != 0 && sh.half && x > 0.f) {
-            // s (c1h + c3h mu): dI/dmu = c1h / (2 s) + 1.5 c3h s, s = mu^(1/2)
-            const float c1h = sh.c1h, c3h = sh.c3h;
-            const float s_ = sqrtf(sx);
-            I += s_ * (c1h + c3h * sx);
-            k += (0.5f * c1h / s_ + 1.5f * c3h * s_) * rs * irho2;
-          }
-        }
-        *Id = -k * d;
-        *Ir = k * d2 * irho;
-        *Iu = I * (float)(kPi / 3.0) * I0 + I0 * (sx - 1.0f);
-        return I;
-      };
-      // derivative mode: per side, d delta / d(stencil distances) and
-      // d delta / d rho times f'(delta) (crossing p(x) = rho, dx = (drho -
-      // sum_m l_m(x) dy_m) / p'(x); delta = -x on the left, x on the right).
-      // p'(x) is a difference of nearly equal distances, so the stencil
-      // and the crossing are taken in FP64 in this mode.
-      float sd_c[2], sd_l[2][4];
-      int sd_b[2], sd_n[2];
-      // dist (derivative mode): FP64 distances of rays mi-2 .. mi+2 (inf
-      // beyond a non-periodic edge), or NULL to compute them here
-      // sv[k] = signed squared distance of ray l - 2 + k (sv[2] is the
-      // point), lab = l (absolute index), irow = its row
-      // WU (forward mode, optional): the same point's weight under the
-      // uniform rule f_U(delta) = delta + 1/2, for the split-profile rule
-      auto boundary_weight = [&](int mi, const float* sv, int lab, int irow, const double* dist,
-                                 float* WU = nullptr) -> float {
-        float d2 = -sv[2];
-        float vl = sv[1], vr = sv[3];
-        bool Lin = signbit(vl), Rin = signbit(vr);
-        float W;
-          float fL = 0.f, fR = 0.f, uL = 0.f, uR = 0.f;
-          if (DER) { sd_n[0] = sd_n[1] = 0; sd_c[0] = sd_c[1] = 0.f; }
-          for (int side = 0; side < 2; ++side) {
-            bool isL = side == 0;
-            if (isL ? Lin : Rin) continue;
-            float vo = isL ? vl : vr;
-            float delta;
-            if (isinf(vo)) {
-              delta = 0.5f;
-              st_local |= ICRS_ST_EDGE;
-            } else if (DER) {
-              // FP64 stencil; FP32 regula falsi, then Newton on the FP64
-              // cubic; f, f' and the basis in FP32 at the FP64 crossing
-              const int c0 = isL ? -2 : -1;
-              double xsd[4], ysd[4];
-              float ysf[4];
-              int nd = 0;
-              double yin = 0, yout = 0;
-              for (int c = 0; c < 4; ++c) {
-                const int off = c0 + c;
-                double v;
-                if (dist) {
-                  v = dist[off + 2];
-                } else {
-                  const int l2_ = lab + off;
-                  v = (!B.periodic && (l2_ < 0 || l2_ >= NTH)) ? __longlong_as_double(0x7ff0000000000000LL)
-                                                               : ray_distance64<NL>(sh, B, irow, wrapl(l2_));
-                }
-                if (isinf(v)) { st_local |= ICRS_ST_EDGE; continue; }
-                xsd[nd] = (double)off;
-                ysd[nd] = v;
-                ysf[nd] = (float)v;
-                if (off == 0) yin = v;
-                if (off == (isL ? -1 : 1)) yout = v;
-                ++nd;
-              }
-              const double dd1 = ysd[1] - ysd[0];
-              const double dd2 = nd > 2 ? 0.5 * (ysd[2] - 2.0 * ysd[1] + ysd[0]) : 0.0;
-              const double dd3 = nd > 3 ? (ysd[3] - 3.0 * ysd[2] + 3.0 * ysd[1] - ysd[0]) * (1.0 / 6.0) : 0.0;
-              double xd = crossing_solve<float>(ysf, (float)xsd[0], nd, (float)yin, (float)yout, isL ? -1.0f : 1.0f,
-                                                rho32, 1e-5f, 12);
-              bool ok = true;
-              for (int it = 0; it < 2; ++it) {
-                const double tt = xd - xsd[0];
-                const double pv = ysd[0] + tt * (dd1 + (tt - 1.0) * (dd2 + (tt - 2.0) * dd3)) - sh.rho;
-                const double pd = dd1 + (2.0 * tt - 1.0) * dd2 + ((3.0 * tt - 6.0) * tt + 2.0) * dd3;
-                if (!(pd != 0.0)) { ok = false; break; }
-                xd -= pv / pd;
-              }
-              if (!ok || !(isL ? (xd >= -1.0 && xd <= 0.0) : (xd >= 0.0 && xd <= 1.0)))
-                xd = crossing_solve<double>(ysd, xsd[0], nd, yin, yout, isL ? -1.0 : 1.0, sh.rho, 1e-14, 60);
-              const double dd = isL ? -xd : xd;
-              const float dl = (float)dd;
-              float fv, fp;
-              if (g.uniform) { fv = dl + 0.5f; fp = 1.0f; }
-              else if (dd >= g.delta_c) {
-                const float sq = sqrtf(1.0f + 0.5f / dl);
-                fv = (0.5f + dl) * (2.0f / 3.0f) * sq;
-                fp = (2.0f / 3.0f) * sq - (0.5f + dl) / (6.0f * dl * dl * sq);
-              } else { fv = (2.0f / 3.0f) * dl + 0.5f; fp = 2.0f / 3.0f; }
-              // the paper's gradient rule: the fixed derivative of the
-              // second-order branch on both branches
-              if (g.grad_rule && !g.uniform) fp = 2.0f / 3.0f;
-              if (isL) fL = fv; else fR = fv;
-              const double tt = xd - xsd[0];
-              const double slope = dd1 + (2.0 * tt - 1.0) * dd2 + ((3.0 * tt - 6.0) * tt + 2.0) * dd3;
-              (void)lagrange_basis<float>(ysf, nd, (float)tt, sd_l[side]);
-              sd_c[side] = (float)((isL ? -fp : fp) / slope);
-              sd_b[side] = mi + (int)xsd[0];
-              sd_n[side] = nd;
-              continue;
-            } else {
-              // stencil: entering (-2,-1,0,+1), exiting (-1,0,+1,+2)
-              float xs[4], ys[4];
-              int np_ = 0;
-              const int c0 = isL ? -2 : -1;
-              for (int c = 0; c < 4; ++c) {
-                float vv = sv[2 + c0 + c];
-                if (isinf(vv)) { st_local |= ICRS_ST_EDGE; continue; }
-                xs[np_] = (float)(c0 + c);
-                ys[np_] = sqrtf(fabsf(vv));
-                ++np_;
-              }
-              float xo = isL ? -1.0f : 1.0f;
-              float x = crossing_solve<float>(ys, xs[0], np_, sqrtf(d2), sqrtf(fabsf(vo)), xo, rho32, 1e-5f, 12);
-              delta = isL ? -x : x;
-              if (!g.uniform && fabsf(delta - dcf) < 2e-3f) {
-                // branch of f(delta) too close to call in FP32: redo the
-                // crossing from FP64 distances
-                int l = lab;
-                double xsd[4], ysd[4];
-                int nd = 0;
-                double yin = 0, yout = 0;
-                for (int c = 0; c < 4; ++c) {
-                  int ll2 = l + c0 + c;
-                  if (!B.periodic && (ll2 < 0 || ll2 >= NTH)) continue;
-                  int lw2 = ((ll2 % NTH) + NTH) % NTH;
-                  xsd[nd] = (double)(c0 + c);
-                  ysd[nd] = ray_distance64<NL>(sh, B, irow, lw2);
-                  if (c0 + c == 0) yin = ysd[nd];
-                  if (c0 + c == (isL ? -1 : 1)) yout = ysd[nd];
-                  ++nd;
-                }
-                if (diag_cnt) atomicAdd(&sh.cnt[3], 1);
-                double xd = crossing_solve<double>(ysd, xsd[0], nd, yin, yout, isL ? -1.0 : 1.0, sh.rho, 1e-14, 60);
-                double dd = isL ? -xd : xd;
-                delta = (float)dd;
-                float fv = (float)fdelta<double>(dd, g.delta_c, 0);
-                if (isL) { fL = fv; uL = delta + 0.5f; } else { fR = fv; uR = delta + 0.5f; }
-                continue;
-              }
-            }
-            float fv = fdelta<float>(delta, dcf, g.uniform);
-            if (isL) { fL = fv; uL = delta + 0.5f; } else { fR = fv; uR = delta + 0.5f; }
-          }
-          if (WU) *WU = Lin ? uR : (Rin ? uL : fmaxf(0.f, uL + uR - 1.0f));
-          if (Lin) W = fR;
-          else if (Rin) W = fL;
-          else W = fmaxf(0.f, fL + fR - 1.0f);
-          if (DER && !(Lin || Rin) && !(fL + fR - 1.0f > 0.f)) sd_n[0] = sd_n[1] = 0, sd_c[0] = sd_c[1] = 0.f;
-        return W;
-      };
-      {
-        // ---- ray stage.  A warp takes a task of 32 rows (lane = row i) and
-        // a chunk [c0, c1) of theta columns, and sweeps the columns in blocks
-        // of KB (all lanes at the same column, so the group offsets and,
-        // within an r group, the anchor are shared and held in registers).
-        // Each ray's squared distance is classified against the group's FP32
-        // band: inside (I(d) added to the row), outside, or undecided.  The
-        // inside flags go into a per-lane bit window.  At the end of a block
-        // one warp vote covers both rare events: a ray the band left
-        // undecided (its own bound, else FP64, decides it) and a boundary
-        // point (inside with an outside neighbour), which goes to the
-        // per-warp deferred queue as (column, row).  A queue flush
-        // re-evaluates each point's five-ray stencil and adds I (W - 1)
-        // (Appendix A per-point rule).  The adjoint adds, for every inside
-        // ray, its seed dI/dd times the gradient of d, and the queue flush
-        // the boundary points' seeds.
-        int2* dq = reinterpret_cast<int2*>(wqueue + warp * 2 * DQ);
-        int dq_n = 0;
-        const int CH = sh.chunk;
-        const int nch = (NTH + CH - 1) / CH;
-        const int ntask = ((NR + 31) >> 5) * nch;
-        const float rr32 = rho32 * rho32;
-        const unsigned lt_mask = (1u << lane) - 1u;
-        const AnchorF* anf = reinterpret_cast<const AnchorF*>(anch);
-        // c + a b in FP32, each operation rounded as written
-        auto cfma = [](const cf a, const cf b, const cf c) -> cf {
-          return mk(__fmaf_rn(a.x, b.x, __fmaf_rn(-a.y, b.y, c.x)), __fmaf_rn(a.x, b.y, __fmaf_rn(a.y, b.x, c.y)));
-        };
-        // squared distance |Delta w'|^2 of the ray at group offset (tx, ty)
-        // in the row (ri_, dri_) of anchor an: Delta w' = ws + dz + conj(dz
-        // N / P), dz = (ri_ tx + dri_, ri_ ty).  Every operation is rounded
-        // as written, so each evaluation of a ray gives the same bits.  With
-        // eb: the ray's own bound on the error of |Delta w'|, e0 + 2 |dz| u
-        // (cN M_N + cU |U| M_P) / |P|, from |dN| <= cN u M_N, |dP| <= cP u
-        // M_P (Horner in complex FMAs, plus the rounded coefficients) and cU
-        // = 3 cP + 10 (the quotient, |P|^2, the reciprocal and the products),
-        // times 2 for the FP32 evaluation of the bound.
-        // (dzo, dwo: optionally dz and Delta w' themselves, for the adjoint)
-        auto ray_eval = [&](const AnchorF& an, float tx, float ty, float ri_, float dri_, float* eb, cf* dzo = nullptr,
-                            cf* dwo = nullptr) -> float {
-          const cf dz = mk(__fmaf_rn(ri_, tx, dri_), __fmul_rn(ri_, ty));
-          cf Pq, Nq;
-          if constexpr (NL == 2) {
-            const cf F = mk(__fadd_rn(an.p[1].x, dz.x), __fadd_rn(an.p[1].y, dz.y));
-            Pq = cfma(dz, F, an.p[0]);
-            Nq = cfma(an.n[1], dz, an.n[0]);
-          } else {
-            const cf F2 = mk(__fadd_rn(an.p[2].x, dz.x), __fadd_rn(an.p[2].y, dz.y));
-            Pq = cfma(dz, cfma(dz, F2, an.p[1]), an.p[0]);
-            Nq = cfma(dz, cfma(an.n[2], dz, an.n[1]), an.n[0]);
-          }
-          const float q = __fmaf_rn(Pq.x, Pq.x, __fmul_rn(Pq.y, Pq.y));
-          const float ip = rcp_fast(q);  // <= 1 ulp
-          // V = N conj(P), pv = dz V, Delta w' = (ws + dz) + conj(pv) / |P|^2
-          const cf V = mk(__fmaf_rn(Nq.x, Pq.x, __fmul_rn(Nq.y, Pq.y)), __fmaf_rn(Nq.y, Pq.x, -__fmul_rn(Nq.x, Pq.y)));
-          const cf pv = mk(__fmaf_rn(dz.x, V.x, -__fmul_rn(dz.y, V.y)), __fmaf_rn(dz.x, V.y, __fmul_rn(dz.y, V.x)));
-          const cf dw = mk(__fmaf_rn(pv.x, ip, __fadd_rn(an.ws.x, dz.x)), __fmaf_rn(-pv.y, ip, __fadd_rn(an.ws.y, dz.y)));
-          if (dzo) *dzo = dz;
-          if (dwo) *dwo = dw;
-          if (eb) {
-            const float md = sqrtf(abs2(dz)), aP = sqrtf(q), aU = sqrtf(abs2(V)) * ip;
-            const float mn = sqrtf(abs2(an.n[0])) + md * (sqrtf(abs2(an.n[1])) + md * sqrtf(abs2(an.n[2])));
-            const float mp = NL == 2 ? sqrtf(abs2(an.p[0])) + md * (sqrtf(abs2(an.p[1])) + md)
-                                     : sqrtf(abs2(an.p[0])) + md * (sqrtf(abs2(an.p[1])) + md * (sqrtf(abs2(an.p[2])) + md));
-            constexpr float cN = NL == 2 ? 4.0f : 9.0f, cU = NL == 2 ? 28.0f : 49.0f;
-            *eb = an.e0 + 2.0f * md * EPS32 * (cN * mn + cU * aU * mp) / aP;
-          }
-          return __fmaf_rn(dw.x, dw.x, __fmul_rn(dw.y, dw.y));
-        };
-        // a ray the group band left open: its own bound decides in FP32 where
-        // it can, else the FP64 distance (d2 is then replaced by its square)
-        auto decide = [&](float& d2, float eb, int irow, int lw) -> bool {
-          const float X = 1.01f * (2.0f * rho32 * eb + eb * eb) + 8.0f * EPS32 * rr32;
-          if (fabsf(d2 - rr32) > X) return d2 < rr32;
-          const double d64 = ray_distance64<NL>(sh, B, irow, lw);
-          if (diag_cnt) atomicAdd(&sh.cnt[2], 1);
-          d2 = (float)(d64 * d64);
-          return d64 < sh.rho;
-        };
-        // any column l of row irow (wrapped; beyond a non-periodic edge: outside, +inf)
-        // a ray's spot factor: 1 - c inside the spot, else 1.  dw: the ray's
-        // offset from the source centre in the frame of anchor ai, with error
-        // bound eb; the spot centre's FP32 rounding adds 4 u rho.  Decided in
-        // FP32 outside the band, else from the FP64 offset as the oracle
-        // decides it.
-        const float spot_rr = (float)(sh.rho * sh.spot_r);
-        const float spot_r2 = spot_rr * spot_rr;
-        const float spot_f = (float)(1.0 - sh.spot_c);
-        auto spot_factor = [&](int ai, const cf dw, float eb, int irow, int lw) -> float {
-          if (LAW == 0 || !sh.spot) return 1.f;
-          const float2 c = spc[ai];
-          const float ex = dw.x - c.x, ey = dw.y - c.y;
-          const float q = fmaf(ex, ex, ey * ey);
-          const float e = eb + 4.0f * EPS32 * rho32;
-          const float X = 1.01f * (2.0f * spot_rr * e + e * e) + 8.0f * EPS32 * spot_r2;
-          if (fabsf(q - spot_r2) > X) return q < spot_r2 ? spot_f : 1.f;
-          const cd d64 = ray_offset64<NL>(sh, B, irow, lw);
-          const double fx = d64.x / sh.rho - sh.spot_x, fy = d64.y / sh.rho - sh.spot_y;
-          return fx * fx + fy * fy < sh.spot_r * sh.spot_r ? spot_f : 1.f;
-        };
-        // (fso: optionally the ray's spot factor)
-        auto classify = [&](int gi_, float ri_, float dri_, int irow, int l, float* d2o,
-                            float* fso = nullptr) -> bool {
-          if (!B.periodic && (l < 0 || l >= NTH)) { *d2o = __int_as_float(0x7f800000); if (fso) *fso = 1.f; return false; }
-          const int lw = wrapl(l);
-          const int mgrp = (int)__umulhi((unsigned int)lw, gmagic);
-          const AnchorF& an = anf[gi_ * mth + mgrp];
-          const cf t = tab_at(lw - mgrp * gth);
-          float eb;
-          cf dw;
-          float d2 = ray_eval(an, t.x, t.y, ri_, dri_, &eb, nullptr, &dw);
-          bool in = d2 < an.lo2;
-          if (!in && !(d2 > an.hi2)) in = decide(d2, eb, irow, lw);
-          *d2o = d2;
-          if (fso) *fso = spot_factor(gi_ * mth + mgrp, dw, eb, irow, lw);
-          return in;
-        };
-        {
-          // ---- derivative ray stage (binary lens).  Per ray with seed a =
-          // dRow/dd (dI/dd inside; the paper's sigmoid rule adds its own),
-          // the row's sums pg[k] += a dd/dq_k are taken from the ray's FP32
-          // geometry (rotated frame R = e^{-i th_m}: Q_j = A_j + dz, u =
-          // Delta w' / d, gamma = sum eps_j / Q_j^2):
-          //   dd/dz = J u, J = [[1 + g.x, -g.y], [-g.y, 1 - g.x]]
-          //   dd/dr_i = (J u) . e^{i phi},  dd/dth_l = (J u) . (i z)
-          //   dd/dw_c = -conj(R) u,  dd/da_j.x = -eps_j Re(conj(u) conj(R) Q_j^2) / |Q_j|^4
-          //   dd/deps_j = -(u . Q_j) / |Q_j|^2
-          // pg: sum a dd/dr_i, sum a dd/dth_l, sum a dd/dth_l (l + 1/2), then
-          // d/d(w_c.x, w_c.y, rho, u1, a1.x, a2.x, eps1, eps2).
-          const float eps0 = sh.eps32[0], eps1 = sh.eps32[1];
-          const bool gradrule = g.grad_rule != 0;
-          auto grad_core = [&](const cf dz, const cf dw, float tx, float ty, float ri_, float lwf, const float4 A01,
-                               const float2 cs_, float a, float* pgx) {
-            const cf Q0 = mk(A01.x + dz.x, A01.y + dz.y), Q1 = mk(A01.z + dz.x, A01.w + dz.y);
-            const float i0 = rcp_fast(abs2(Q0)), i1 = rcp_fast(abs2(Q1));
-            const float id = rsqrt_fast(fmaxf(abs2(dw), 1e-37f));
-            const float ux = dw.x * id, uy = dw.y * id;
-            const cf q0 = Q0 * Q0, q1 = Q1 * Q1;
-            const cf gm = scl(cj(q0), eps0 * i0 * i0) + scl(cj(q1), eps1 * i1 * i1);
-            const float gzx = (1.0f + gm.x) * ux - gm.y * uy;
-            const float gzy = -gm.y * ux + (1.0f - gm.x) * uy;
-            const float ex = 1.0f + tx, ey = ty;
-            const float gr_ = gzx * ex + gzy * ey;
-            const float gt_ = ri_ * (gzy * ex - gzx * ey);
-            pgx[0] += a * gr_;
-            pgx[1] += a * gt_;
-            pgx[2] += a * gt_ * lwf;
-            const float ct = cs_.x, st = cs_.y;
-            pgx[3] -= a * (ct * ux - st * uy);
-            pgx[4] -= a * (st * ux + ct * uy);
-            // conj(R) Q_j^2 with conj(R) = (ct, st)
-            const cf P0 = mk(ct, st) * q0, P1 = mk(ct, st) * q1;
-            pgx[7] -= a * eps0 * (ux * P0.x + uy * P0.y) * i0 * i0;
-            pgx[8] -= a * eps1 * (ux * P1.x + uy * P1.y) * i1 * i1;
-            pgx[9] -= a * (ux * Q0.x + uy * Q0.y) * i0;
-            pgx[10] -= a * (ux * Q1.x + uy * Q1.y) * i1;
-          };
-          // a ray's seed, its value I (inside) into racc and the brightness
-          // derivatives into pgx[5], pgx[6]; the paper's gradient rule (Sec.
-          // 3.5) gives the indicator chi = Theta(x), x = (rho - d) / rho, the
-          // sigmoid derivative S s (1 - s), s = 1 / (1 + e^{-S x}), with the
-          // interior weight: seed -I S s (1 - s) / rho on d and I S s (1 - s)
-          // d / rho^2 on rho (tangents only)
-          // (fs: the ray's spot factor, which scales its brightness)
-          auto seed_of = [&](bool in, float d2, float* pgx, float& racc, auto hc, float fs) -> float {
-            float a = 0.f;
-            if (in) {
-              float Id, Ir, Iu;
-              racc += fs * brightness_der(d2, &Id, &Ir, &Iu, hc);
-              a = fs * Id;
-              pgx[5] += fs * Ir;
-              pgx[6] += fs * Iu;
-            }
-            if (gradrule) {
-              const float dd_ = sqrtf(d2);
-              const float sx = sfac * (1.0f - dd_ / rho32);
-              if (fabsf(sx) < 40.0f) {
-                const float sg = 1.0f / (1.0f + __expf(-sx));
-                const float c = fs * brightness(d2) * sfac * sg * (1.0f - sg);
-                a -= c / rho32;
-                pgx[5] += c * dd_ / (rho32 * rho32);
-              }
-            }
-            return a;
-          };
-          // ray l (any column, wrapped) of row irow: its seed a times the
-          // gradient of its distance into pgx (generic: anchor from the table)
-          auto grad_at = [&](int gi_, float ri_, float dri_, int l, float a, float* pgx) {
-            if (a == 0.f || (!B.periodic && (l < 0 || l >= NTH))) return;
-            const int lw = wrapl(l);
-            const int mgrp = (int)__umulhi((unsigned int)lw, gmagic);
-            const int ai = gi_ * mth + mgrp;
-            const cf t = tab_at(lw - mgrp * gth);
-            cf dz, dw;
-            (void)ray_eval(anf[ai], t.x, t.y, ri_, dri_, nullptr, &dz, &dw);
-            grad_core(dz, dw, t.x, t.y, ri_, (float)lw + 0.5f, ds.aA[ai], ds.acs[ai], a, pgx);
-          };
-          // a row's sums (v[0] = sum of I W, v[1 + k] = pg[k]) as its terms
-          // of dS_b / d(r_lo, r_hi, th_lo, width) and of H: S_b = sum_i K_i
-          // Row_i, K_i = r_i dr dth, r_i = r_lo + (i + 1/2) dr, dr = (r_hi -
-          // r_lo) / N_r, dth = width / N_theta
-          auto row_terms = [&](int irow, float ri_, const float* v, double* x) {
-            const double Rw = (double)v[0], rid = (double)ri_, drd = sh.dr64, dtd = sh.dth64;
-            const double Ki = rid * drd * dtd, fi = (irow + 0.5) / NR;
-            x[0] = Ki * v[1] * (1.0 - fi) + Rw * ((1.0 - fi) * drd * dtd - rid * dtd / NR);
-            x[1] = Ki * v[1] * fi + Rw * (fi * drd * dtd + rid * dtd / NR);
-            x[2] = Ki * v[2];
-            x[3] = Ki * v[3] / NTH + Rw * rid * drd / NTH;
-#pragma unroll
-            for (int k = 4; k < 12; ++k) x[k] = Ki * v[k];
-          };
-          auto kahan = [&](float term) {
-            const float y = term - acc_c;
-            const float tt = acc_s + y;
-            acc_c = (tt - acc_s) - y;
-            acc_s = tt;
-          };
-          // the queued boundary points: one per lane.  FP32 stencil values
-          // (the flags), FP64 stencil distances for the crossing and its
-          // derivative; the point's value I (W - 1) beyond the I the sweep
-          // added, its seed (W - 1) dI/dd, and the crossing seeds on the
-          // stencil rays; its row's terms go to the warp's sums directly
-          auto flush_queue = [&]() {
-            __syncwarp();
-            double xq[12];
-#pragma unroll
-            for (int k = 0; k < 12; ++k) xq[k] = 0.0;
-            if (lane < dq_n) {
-              const int2 q_ = dq[lane];
-              const int m = q_.x, irow = q_.y;
-              const int gi_ = irow / gr;
-              const float dri_ = ((float)(irow - gi_ * gr) + 0.5f - 0.5f * (float)gr) * dr32;
-              const float ri_ = (float)(B.r_lo + (gi_ * gr + 0.5 * gr) * sh.dr64) + dri_;
-              float sv[5], fsc = 1.f;
-              double dist[5];
-#pragma unroll 1
-              for (int k = 0; k < 5; ++k) {
-                const int l = m - 2 + k;
-                float d2;
-                const bool in = classify(gi_, ri_, dri_, irow, l, &d2, k == 2 ? &fsc : nullptr);
-                sv[k] = in ? __int_as_float(__float_as_int(d2) | 0x80000000) : d2;
-                dist[k] = (!B.periodic && (l < 0 || l >= NTH)) ? __longlong_as_double(0x7ff0000000000000LL)
-                                                               : ray_distance64<NL>(sh, B, irow, wrapl(l));
-              }
-              if (signbit(sv[2])) {
-                float Id, Ir, Iu;
-                float I = (LAW != 0 && sh.generic) ? brightness_der(-sv[2], &Id, &Ir, &Iu, std::true_type{})
-                                     : brightness_der(-sv[2], &Id, &Ir, &Iu, std::false_type{});
-                // a spot scales the point's brightness and its derivatives
-                I *= fsc; Id *= fsc; Ir *= fsc; Iu *= fsc;
-                const float W = boundary_weight(m, sv, m, irow, dist);
-                float v[12];
-#pragma unroll
-                for (int k = 0; k < 12; ++k) v[k] = 0.f;
-                v[0] = I * (W - 1.0f);
-                v[1 + 5] += (W - 1.0f) * Ir;
-                v[1 + 6] += (W - 1.0f) * Iu;
-                grad_at(gi_, ri_, dri_, m, (W - 1.0f) * Id, v + 1);
-                for (int sd = 0; sd < 2; ++sd) {
-                  if (!sd_n[sd]) continue;
-                  const float c = I * sd_c[sd];
-                  v[1 + 5] += c;
-                  for (int k = 0; k < sd_n[sd]; ++k) grad_at(gi_, ri_, dri_, sd_b[sd] + k, -c * sd_l[sd][k], v + 1);
-                }
-                row_terms(irow, ri_, v, xq);
-                kahan(ri_ * v[0] * bxw);
-              }
-            }
-            // the points' row terms summed over the warp in a fixed order
-#pragma unroll 1
-            for (int k = 0; k < 12; ++k) {
-              double xs = xq[k];
-              for (int o2 = 16; o2 > 0; o2 >>= 1) xs += __shfl_xor_sync(0xffffffffu, xs, o2);
-              if (lane == k) wder[warp * 12 + k] += xs;
-            }
-            __syncwarp();
-            dq_n = 0;
-          };
-          // static task order (warp, warp + NW, ...): every sum of the
-          // adjoint is taken in the same order on every run
-          for (int task = warp; task < ntask; task += NW) {
-            const int rbk = task / nch, chk = task - rbk * nch;
-            const int i = rbk * 32 + lane;
-            const bool rowok = i < NR;
-            const int ii = rowok ? i : NR - 1;
-            const int gi = ii / gr;
-            const float dri = ((float)(ii - gi * gr) + 0.5f - 0.5f * (float)gr) * dr32;
-            const float ri = (float)(B.r_lo + (gi * gr + 0.5 * gr) * sh.dr64) + dri;
-            const int c0 = chk * CH, c1 = min(c0 + CH, NTH);
-            float rowacc = 0.f;  // sum of I over the row's inside rays
-            float pg[11];
-#pragma unroll
-            for (int k = 0; k < 11; ++k) pg[k] = 0.f;
-            float dh;
-            unsigned win = classify(gi, ri, dri, ii, c0 - 1, &dh) ? 1u : 0u;
-            AnchorF ar;  // the current group's anchor, A_j and angle
-            int aiD = 0;  // its index
-            float4 A01 = make_float4(0.f, 0.f, 0.f, 0.f);
-            float2 cs = make_float2(1.f, 0.f);
-            int gbase = 0;
-            auto push_bits = [&](unsigned bm, int base) {
-              while (__any_sync(0xffffffffu, bm != 0u)) {
-                const bool has = bm != 0u;
-                const int m = base - (has ? __ffs(bm) - 1 : 0);
-                bm &= bm - 1u;
-                unsigned rem = __ballot_sync(0xffffffffu, has);
-                while (rem) {
-                  if (dq_n == DQ) flush_queue();
-                  unsigned take = rem;
-                  const int room = DQ - dq_n;
-                  if (__popc(take) > room) {
-                    take = 0u;
-                    unsigned r = rem;
-                    for (int k = 0; k < room; ++k) {
-                      const unsigned low = r & (0u - r);
-                      take |= low;
-                      r ^= low;
-                    }
-                  }
-                  if (take & (1u << lane)) dq[dq_n + __popc(take & lt_mask)] = make_int2(m, i);
-                  dq_n += __popc(take);
-                  rem &= ~take;
-                }
-              }
-            };
-            auto centres = [&](int nb, bool first) -> unsigned {
-              unsigned bm = ((win & ~((win << 1) & (win >> 1))) >> 1) & ((1u << nb) - 1u);
-              if (first) bm &= ~(1u << (nb - 1));
-              return rowok ? bm : 0u;
-            };
-            // one column: value, flag and, for a decided ray, its seed and
-            // gradient; an undecided ray waits for the block end
-            auto colD = [&](int l, const cf t, bool& unc, auto hc) {
-              cf dz, dw;
-              float eb = 0.f;
-              const float d2 = ray_eval(ar, t.x, t.y, ri, dri, decltype(hc)::value ? &eb : nullptr, &dz, &dw);
-              const bool in = d2 < ar.lo2;
-              const bool u_ = !(in || d2 > ar.hi2);
-              unc = unc || u_;
-              win = (win << 1) | (in ? 1u : 0u);
-              if (!u_) {
-                float fs = 1.f;
-                if constexpr (decltype(hc)::value) fs = in ? spot_factor(aiD, dw, eb, ii, l) : 1.f;
-                const float a = seed_of(in, d2, pg, rowacc, hc, fs);
-                if (a != 0.f) grad_core(dz, dw, t.x, t.y, ri, (float)l + 0.5f, A01, cs, a, pg);
-              }
-            };
-            auto block_end = [&](int l0, int nb, bool first, bool unc) {
-              unsigned bm = centres(nb, first);
-              if (__any_sync(0xffffffffu, unc || bm != 0u)) {
-                if (unc) {
-                  for (int k = 0; k < nb; ++k) {
-                    const cf t = tab_at(l0 + k - gbase);
-                    float eb;
-                    cf dz, dw;
-                    float d2 = ray_eval(ar, t.x, t.y, ri, dri, &eb, &dz, &dw);
-                    if (d2 < ar.lo2 || d2 > ar.hi2) continue;
-                    const bool in = decide(d2, eb, ii, l0 + k);
-                    if (in) win |= 1u << (nb - 1 - k);
-                    const float fs = in ? spot_factor(aiD, dw, eb, ii, l0 + k) : 1.f;
-                    const float a = (LAW != 0 && sh.generic) ? seed_of(in, d2, pg, rowacc, std::true_type{}, fs)
-                                               : seed_of(in, d2, pg, rowacc, std::false_type{}, fs);
-                    if (a != 0.f) grad_core(dz, dw, t.x, t.y, ri, (float)(l0 + k) + 0.5f, A01, cs, a, pg);
-                  }
-                  bm = centres(nb, first);
-                }
-                push_bits(bm, l0 + nb - 2);
-              }
-            };
-            int l = c0;
-            bool first = true;
-            while (l < c1) {
-              const int mgrp = (int)__umulhi((unsigned int)l, gmagic);
-              const int ai = gi * mth + mgrp;
-              aiD = ai;
-              ar = anf[ai];
-              A01 = ds.aA[ai];
-              cs = ds.acs[ai];
-              gbase = mgrp * gth;
-              const int lend = min(gbase + gth, c1);
-              while (l < lend) {
-                const int nb = min(KB, lend - l);
-                bool unc = false;
-                if (LAW != 0 && sh.generic) {
-#pragma unroll 1
-                  for (int k = 0; k < nb; ++k) colD(l + k, tab_at(l + k - gbase), unc, std::true_type{});
-                } else {
-#pragma unroll 1
-                  for (int k = 0; k < nb; ++k) colD(l + k, tab_at(l + k - gbase), unc, std::false_type{});
-                }
-                block_end(l, nb, first, unc);
-                first = false;
-                l += nb;
-              }
-            }
-            win = (win << 1) | (classify(gi, ri, dri, ii, c1, &dh) ? 1u : 0u);
-            push_bits(rowok ? (((win & ~((win << 1) & (win >> 1))) >> 1) & 1u) : 0u, c1 - 1);
-            // the row's terms, summed over the warp's rows
-            double x[12];
-            float v[12];
-            v[0] = rowacc;
-#pragma unroll
-            for (int k = 0; k < 11; ++k) v[k + 1] = pg[k];
-            row_terms(ii, ri, v, x);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-              double xs = rowok ? x[k] : 0.0;
-              for (int o2 = 16; o2 > 0; o2 >>= 1) xs += __shfl_xor_sync(0xffffffffu, xs, o2);
-              if (lane == k) wder[warp * 12 + k] += xs;
-            }
-            if (rowok) kahan(ri * rowacc * bxw);
-          }
-          flush_queue();
-        }
-      }
-      __syncthreads();
-      if (DER && tid < 12) {
-        double sum = 0.0;
-        for (int w = 0; w < NW; ++w) { sum += wder[w * 12 + tid]; wder[w * 12 + tid] = 0.0; }
-        if (tid < 4) ds.Gb[bxi][tid] = sum;
-        else ds.H[tid - 4] += sum;
-      }
-    }
-    if (st_local) atomicOr(&sh.status, st_local);
-    raysum = (double)acc_s - (double)acc_c;
+      raysum = der_stage(sh, rays_sh, der_sh);
+      der_sums(rays_sh, der_sh, sh.nbox, ds.Gb, ds.H);
     }
     if (diag_cnt && tid == 0) { long long c_ = clock64(); sh.cnt[12] = (int)min(c_ - sh.clk0, 2000000000LL); sh.clk0 = c_; }
     // ------------------------------------------------ 10. reduction
@@ -2379,53 +1556,51 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (lane == 0) sh.red[warp] = v;
     __syncthreads();
-    if (tid == 0) {
-      double tot = 0.0;
-      for (int w = 0; w < NW; ++w) tot += sh.red[w];
+    if (warp == 0) {
+      double tot = lane < NW ? sh.red[lane] : 0.0;
+      for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
       // unspotted normalisation A0 = S / rho^2; a spot divides by the
       // unlensed flux 1 - c F_spot (N = spot_norm); an invalid spot gives NaN
       const double A0 = tot / (sh.rho * sh.rho);
       double A = A0 * sh.spot_norm;
       if (LAW != 0 && sh.spot_bad) A = __longlong_as_double(0x7ff8000000000000LL);
-      if (!(A == A) || isinf(A)) sh.status |= ICRS_ST_NAN;
+      bool nan_ = !(A == A) || isinf(A);
       size_t o = (size_t)s * E + e;
       if (DER) {
         // dA/dp = (sum_b G_b . d bounds_b/dp + H . d(w_c, rho, u1, a, eps)/dp) / rho^2
-        //         - 2 S / rho^3 [p = rho]
-        double dS[NPAR];
-        for (int q = 0; q < NPAR; ++q) dS[q] = 0.0;
+        //         - 2 S / rho^3 [p = rho], one parameter per lane
+        const int q = lane & 7;
+        double dS = 0.0;
         for (int b = 0; b < sh.nbox; ++b)
-          for (int q = 0; q < NPAR; ++q)
-            dS[q] += ds.Gb[b][0] * bdual[b].r_lo.d[q] + ds.Gb[b][1] * bdual[b].r_hi.d[q] +
-                     ds.Gb[b][2] * bdual[b].th_lo.d[q] + ds.Gb[b][3] * bdual[b].width.d[q];
-        for (int q = 0; q < 4; ++q) dS[q] += ds.H[0] * ds.dwc[q].x + ds.H[1] * ds.dwc[q].y;
-        dS[4] += ds.H[4] * ds.dadp[0][0] + ds.H[5] * ds.dadp[1][0];
-        dS[5] += ds.H[4] * ds.dadp[0][1] + ds.H[5] * ds.dadp[1][1] + ds.H[6] * ds.depsq[0] + ds.H[7] * ds.depsq[1];
-        dS[6] += ds.H[2];
-        dS[7] += ds.H[3];
-        const double ir2 = 1.0 / (sh.rho * sh.rho);
-        double dA[NPAR];
-        for (int q = 0; q < NPAR; ++q) dA[q] = dS[q] * ir2;
-        dA[6] -= 2.0 * A0 / sh.rho;
+          dS += ds.Gb[b][0] * bdual[b].r_lo.d[q] + ds.Gb[b][1] * bdual[b].r_hi.d[q] +
+                ds.Gb[b][2] * bdual[b].th_lo.d[q] + ds.Gb[b][3] * bdual[b].width.d[q];
+        if (q < 4) dS += ds.H[0] * ds.dwc[q].x + ds.H[1] * ds.dwc[q].y;
+        else if (q == 4) dS += ds.H[4] * ds.dadp[0][0] + ds.H[5] * ds.dadp[1][0];
+        else if (q == 5)
+          dS += ds.H[4] * ds.dadp[0][1] + ds.H[5] * ds.dadp[1][1] + ds.H[6] * ds.depsq[0] + ds.H[7] * ds.depsq[1];
+        else if (q == 6) dS += ds.H[2];
+        else dS += ds.H[3];
+        double dA = dS * (1.0 / (sh.rho * sh.rho));
+        if (q == 6) dA -= 2.0 * A0 / sh.rho;
         // the spot's normalisation: dA = N dA0 + A0 dN, dN/du1 = N^2 c dF/du1
-        for (int q = 0; q < NPAR; ++q) dA[q] *= sh.spot_norm;
-        dA[7] += A * sh.spot_gu;
-        bool bad = false;
-        for (int q = 0; q < NPAR; ++q) bad |= !(dA[q] == dA[q]) || isinf(dA[q]);
-        if (bad) sh.status |= ICRS_ST_NAN;
-        if (dout.dA)
-          for (int q = 0; q < NPAR; ++q) dout.dA[o * NPAR + q] = dA[q];
-        double wgt = 0.0;
-        if (dout.gA) wgt = dout.gA[o];
-        if (dout.yobs) {
-          // chi^2 = sum_e ((y_e - A_e) / sigma_e)^2 with the flux F = A
-          const double r_ = (dout.yobs[o] - A) / dout.sig[o];
-          wgt = -2.0 * r_ / dout.sig[o];
-          if (dout.chi2) atomicAdd(&dout.chi2[s], r_ * r_);
+        dA *= sh.spot_norm;
+        if (q == 7) dA += A * sh.spot_gu;
+        nan_ = __any_sync(0xffffffffu, nan_ || !(dA == dA) || isinf(dA));
+        if (lane < NPAR) {
+          if (dout.dA) dout.dA[o * NPAR + q] = dA;
+          double wgt = 0.0;
+          if (dout.gA) wgt = dout.gA[o];
+          if (dout.yobs) {
+            // chi^2 = sum_e ((y_e - A_e) / sigma_e)^2 with the flux F = A
+            const double r_ = (dout.yobs[o] - A) / dout.sig[o];
+            wgt = -2.0 * r_ / dout.sig[o];
+            if (dout.chi2 && lane == 0) atomicAdd(&dout.chi2[s], r_ * r_);
+          }
+          if (dout.grad) atomicAdd(&dout.grad[(size_t)s * NPAR + q], wgt * dA);
         }
-        if (dout.grad)
-          for (int q = 0; q < NPAR; ++q) atomicAdd(&dout.grad[(size_t)s * NPAR + q], wgt * dA[q]);
       }
+      if (nan_ && lane == 0) sh.status |= ICRS_ST_NAN;
+      if (lane == 0) {
       if (A_out) A_out[o] = A;
       if (st_out) st_out[o] = (sh.status & 0xffu) | ((uint32_t)min(sh.nbox, 255) << 8);
       if (diag_cnt)
@@ -2436,6 +1611,7 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
           if (b < sh.nbox) { d[0] = sh.box[b].r_lo; d[1] = sh.box[b].r_hi; d[2] = sh.box[b].th_lo; d[3] = sh.box[b].width; d[4] = sh.box[b].periodic; }
           else { d[0] = d[1] = d[2] = d[3] = d[4] = 0.0; }
         }
+      }
     }
     __syncthreads();
   }
@@ -2532,10 +1708,10 @@ marginal_nll_kernel(const double* __restrict__ A, const double* __restrict__ F, 
 
 // ---------------------------------------------------------------- host side
 // Columns of the ray stage's offset tables: every sector of an epoch at once
-// (forward), one sector (derivative).
-static int mag_tabcap(int NL, bool der) { return der ? GTH_MAX + 2 : (NL * NL + 1) * (GTH_MAX + 2); }
+// (forward), about three (derivative, where shared memory is shorter).
+static int mag_tabcap(int NL, bool der) { return (der ? 3 : NL * NL + 1) * (GTH_MAX + 2); }
 
-static size_t mag_smem_bytes(int NL, const icrs_grid& g, int pmax, int has_plo, bool der, int nt) {
+static size_t mag_smem_bytes(int NL, const icrs_grid& g, int pmax, int has_plo, bool der, int nt, int ccap = 0) {
   const int N = NL * NL + 1;
   const size_t NP = (size_t)g.n_limb * N;
   size_t b = sizeof(cf) * NP * (has_plo ? 2 : 1) + sizeof(cdf) * g.n_limb + 16;
@@ -2544,7 +1720,7 @@ static size_t mag_smem_bytes(int NL, const icrs_grid& g, int pmax, int has_plo, 
   size_t slots = 4 * sizeof(float) * NP + sizeof(short) * ((NP + 7) & ~(size_t)7) + 3 * ((NP + 15) & ~(size_t)15);
   slots += 2 * sizeof(double) * pmax + sizeof(int) * QMAX;
   const size_t rays = sizeof(cf) * mag_tabcap(NL, der) + (sizeof(AnchorF) + sizeof(float2)) * MAXANCH +
-                      sizeof(int) * (nt / 32) * DQ * (der ? 2 : 1);
+                      sizeof(int) * (nt / 32) * DQ + (der ? der_rays_bytes(nt / 32) : 0) + sizeof(double2) * ccap;
   return b + (slots > rays ? slots : rays);
 }
 
@@ -2584,7 +1760,7 @@ template <int NL, bool DER, int NTB, int LAW>
 static int launch_nt(const icrs_params* p, int S, const double* t, int E, const icrs_grid* g, double* A,
                      uint32_t* status, double* dsect, int32_t* dcnt, float* dpts, const DerOut& dout,
                      cudaStream_t st, const int32_t* items, int n_items, int nsm, size_t smem, int pmax,
-                     int has_plo) {
+                     int has_plo, int ccap) {
   if (cudaFuncSetAttribute(mag_kernel<NL, DER, NTB, LAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return ICRS_ECUDA;
@@ -2599,7 +1775,7 @@ static int launch_nt(const icrs_params* p, int S, const double* t, int E, const 
   long long blocks = (tiles + per_block - 1) / per_block;
   mag_kernel<NL, DER, NTB, LAW><<<(unsigned)blocks, NTB, smem, st>>>(p, S, t, E, *g, (int)per_block, A, status,
                                                                       dsect, dcnt, dpts, pmax, has_plo,
-                                                                      mag_tabcap(NL, DER), dout, items, n_items);
+                                                                      mag_tabcap(NL, DER), ccap, dout, items, n_items);
   return cudaGetLastError() == cudaSuccess ? ICRS_OK : ICRS_ECUDA;
 }
 
@@ -2631,9 +1807,16 @@ static int launch_inst(const icrs_params* p, int S, const double* t, int E, cons
   pmax = np_all < PMAX_MIN ? PMAX_MIN : np_all;
   while (pmax > PMAX_MIN && !fits(pmax, has_plo)) pmax = pmax - 64 > PMAX_MIN ? pmax - 64 : PMAX_MIN;
   if (!DER) has_plo = fits(pmax, 1) ? 1 : 0;
-  const size_t smem = mag_smem_bytes(NL, *g, pmax, has_plo, DER, NT_BASE);
+  // derivative: the cosine table of the columns, for all sectors at once or as
+  // many as fit
+  int ccap = 0;
+  if (DER)
+    for (int k = NL * NL + 1; k > 0 && !ccap; --k)
+      if (mag_smem_bytes(NL, *g, pmax, has_plo, DER, NT_BASE, k * g->n_theta) + fa.sharedSizeBytes <= (size_t)optin)
+        ccap = k * g->n_theta;
+  const size_t smem = mag_smem_bytes(NL, *g, pmax, has_plo, DER, NT_BASE, ccap);
   return launch_nt<NL, DER, NT_BASE, LAW>(p, S, t, E, g, A, status, dsect, dcnt, dpts, dout, st, items, n_items, nsm,
-                                          smem, pmax, has_plo);
+                                          smem, pmax, has_plo, ccap);
 }
 
 // Binary forward: the linear instantiation, then the generic one (each takes

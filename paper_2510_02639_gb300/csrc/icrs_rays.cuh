@@ -66,6 +66,7 @@ struct Sec {
   int periodic;
   int gth, gr, mth, nanch;  // columns and rows per group, theta groups, anchors
   int abase, tbase;      // first anchor, first offset-table column
+  int cbase;             // first column of the cosine table (derivative)
   int ch, nch;           // columns per chunk, chunks
   int ntask;
   int sb;                // columns per superblock
@@ -152,21 +153,32 @@ __device__ __noinline__ double band64(const cd* A64, const cd* K64, const cd* nc
   return 1.01 * (2.0 * (double)rho32 * eb + eb * eb) + 8.0 * EPS32 * ((double)rho32 * (double)rho32);
 }
 
+// An anchor's quantities in FP64.
+template <int NL>
+struct AnchorX {
+  double cs, sn;  // of the anchor's angle
+  cd ws, A[NL], n[3], p[3];
+};
+
 // Anchor an of sector S (one thread).
 template <int NL>
 __device__ inline AnchorF make_anchor(const Sec& S, const double* eps, const cd* a, cd wc, float rho32, int an,
-                                      double* cs_, double* sn_, cd* A64) {
+                                      AnchorX<NL>& ax) {
+  cd* const A64 = ax.A;
+  cd* const nc = ax.n;
+  cd* const pc = ax.p;
   const int gi = an / S.mth, mi = an % S.mth;
   const double rc = S.r_lo + (gi * S.gr + 0.5 * S.gr) * S.dr64;
   const double thc = S.th_lo + (mi * S.gth + 0.5 * S.gth) * S.dth64;
   double sn, cs;
   sincos(thc, &sn, &cs);
-  *cs_ = cs; *sn_ = sn;
+  ax.cs = cs; ax.sn = sn;
   const cd R = mk(cs, -sn);  // e^{-i th_c}
   const cd zc = mk(rc * cs, rc * sn);
   const cd w = lens_map<NL, double>(eps, a, zc) - wc;
   AnchorF af;
-  af.ws = tof(R * w);
+  ax.ws = R * w;
+  af.ws = tof(ax.ws);
   cd K64[NL];
   float aa[NL], kk[NL];
   for (int j = 0; j < NL; ++j) {
@@ -175,7 +187,6 @@ __device__ inline AnchorF make_anchor(const Sec& S, const double* eps, const cd*
     aa[j] = sqrtf(abs2(tof(A64[j])));
     kk[j] = (float)eps[j] / aa[j];
   }
-  cd nc[3], pc[3];
   nc[2] = pc[2] = mk(0.0, 0.0);
   if constexpr (NL == 2) {
     nc[0] = K64[0] * A64[1] + K64[1] * A64[0];
@@ -329,8 +340,11 @@ struct RayArgs {
   float* tabf;      // group offsets (cos d - 1, sin d) of the batch's sectors
   int* wqueue;      // boundary points, DQ per warp
   int tabcap;       // columns that tabf holds
+  int ccap;         // columns that the derivative's cosine table holds (0: none)
   int NR, NTH, uniform, split, diag;
   float one;        // 1
+  float sfac;       // sigmoid steepness of the paper's gradient rule
+  int gradrule;
   double delta_c;
 };
 
@@ -354,10 +368,10 @@ __device__ __forceinline__ cf cfma_rn(const cf a, const cf b, const cf c) {
 // M_N, |dP| <= cP u M_P (Horner in complex FMAs, plus the rounded
 // coefficients) and cU = 3 cP + 10 (the quotient, |P|^2, the reciprocal and
 // the products), times 2 for the FP32 evaluation of the bound.  dwo: Delta w'
-// itself.
+// itself, dzo: dz.
 template <int NL>
 __device__ __forceinline__ float ray_eval(const AnchorF& an, float tx, float ty, float ri_, float dri_, float* eb,
-                                          cf* dwo) {
+                                          cf* dwo, cf* dzo = nullptr) {
   const cf dz = mk(__fmaf_rn(ri_, tx, dri_), __fmul_rn(ri_, ty));
   cf Pq, Nq;
   if constexpr (NL == 2) {
@@ -376,6 +390,7 @@ __device__ __forceinline__ float ray_eval(const AnchorF& an, float tx, float ty,
   const cf pv = mk(__fmaf_rn(dz.x, V.x, -__fmul_rn(dz.y, V.y)), __fmaf_rn(dz.x, V.y, __fmul_rn(dz.y, V.x)));
   const cf dw = mk(__fmaf_rn(pv.x, ip, __fadd_rn(an.ws.x, dz.x)), __fmaf_rn(-pv.y, ip, __fadd_rn(an.ws.y, dz.y)));
   if (dwo) *dwo = dw;
+  if (dzo) *dzo = dz;
   if (eb) {
     const float md = sqrtf(abs2(dz)), aP = sqrtf(q), aU = sqrtf(abs2(V)) * ip;
     const float mn = sqrtf(abs2(an.n[0])) + md * (sqrtf(abs2(an.n[1])) + md * sqrtf(abs2(an.n[2])));
@@ -390,6 +405,20 @@ __device__ __forceinline__ float ray_eval(const AnchorF& an, float tx, float ty,
 __device__ __forceinline__ cf tab_at(const float* tp, int o) {
   const float* t_ = tp + 4 * (o >> 1) + (o & 1);
   return mk(t_[0], t_[2]);
+}
+
+// A superblock of one row from the offsets wa, wb of its ends (db2 = |wb|^2):
+// out: every ray between them is outside, inn: inside.  The distance of the
+// chord from the source centre counts; its rounding, a few u of the
+// coordinates, is added to rout.
+__device__ __forceinline__ void chord_test(const AnchorF& an, const cf wa, const cf wb, float db2, bool& out, bool& inn) {
+  const cf d = wb - wa;
+  const float da2 = abs2(wa);
+  const float tt = __saturatef(-(wa.x * d.x + wa.y * d.y) * rcp_fast(fmaxf(abs2(d), 1e-37f)));
+  const cf cl = mk(fmaf(tt, d.x, wa.x), fmaf(tt, d.y, wa.y));
+  const float ro = an.rout + 1e-6f * (fabsf(wa.x) + fabsf(wa.y) + fabsf(d.x) + fabsf(d.y));
+  out = abs2(cl) > ro * ro;
+  inn = fmaxf(da2, db2) < an.in2;
 }
 
 // A ray the group band left open: its own bound decides in FP32 where it can,
@@ -709,9 +738,14 @@ __device__ __noinline__ float2 flush_points(SH& sh, RayShared& rs, const int* q,
 }
 
 // The next batch of sectors (rs.b0 .. rs.b1 - 1, none left: b0 = b1): its
-// anchors and offset tables.
-template <int NL, int LAW, class SH>
-__device__ __noinline__ void ray_tables(SH& sh, RayShared& rs) {
+// anchors and offset tables.  dr.store(an, x) takes what the derivative keeps
+// of an anchor besides, dr.columns its own tables.
+struct NoDer {
+  template <int NL> __device__ void store(int, const AnchorX<NL>&) const {}
+  __device__ void columns(const RayShared&, int, int) const {}
+};
+template <int NL, int LAW, class SH, class DR>
+__device__ __noinline__ void ray_tables(SH& sh, RayShared& rs, const DR& dr) {
   const int tid = threadIdx.x, NT = blockDim.x;
   const RayArgs& P = rs.P;
   const float rho32 = (float)sh.rho;
@@ -722,8 +756,10 @@ __device__ __noinline__ void ray_tables(SH& sh, RayShared& rs) {
     rs.b0 = b;
     for (; b < nbox; ++b) {
       Sec& S = rs.sec[b];
-      if (b > rs.b0 && (na + S.nanch > MAXANCH || nc + S.gth + 2 > P.tabcap)) break;
-      S.abase = na; S.tbase = nc;
+      if (b > rs.b0 && (na + S.nanch > MAXANCH || nc + S.gth + 2 > P.tabcap ||
+                        (P.ccap && (b - rs.b0 + 1) * P.NTH > P.ccap)))
+        break;
+      S.abase = na; S.tbase = nc; S.cbase = (b - rs.b0) * P.NTH;
       na += S.nanch; nc += S.gth + 2;
     }
     rs.b1 = b; rs.nanch = na; rs.ncol = nc;
@@ -734,11 +770,11 @@ __device__ __noinline__ void ray_tables(SH& sh, RayShared& rs) {
     int b = b0;
     while (b + 1 < b1 && an >= rs.sec[b + 1].abase) ++b;
     const Sec& S = rs.sec[b];
-    double cs, sn;
-    cd A64[NL];
-    P.anch[an] = make_anchor<NL>(S, sh.L.eps, sh.L.a, sh.wc, rho32, an - S.abase, &cs, &sn, A64);
-    if (spot) P.spc[an] = make_float2((float)(sh.rho * (cs * sh.spot_x + sn * sh.spot_y)),
-                                      (float)(sh.rho * (cs * sh.spot_y - sn * sh.spot_x)));
+    AnchorX<NL> x;
+    P.anch[an] = make_anchor<NL>(S, sh.L.eps, sh.L.a, sh.wc, rho32, an - S.abase, x);
+    if (spot) P.spc[an] = make_float2((float)(sh.rho * (x.cs * sh.spot_x + x.sn * sh.spot_y)),
+                                      (float)(sh.rho * (x.cs * sh.spot_y - x.sn * sh.spot_x)));
+    dr.store(an, x);
   }
   // offsets within a theta group, (cos d - 1, sin d) with d = (o + 1/2 -
   // gth/2) dth; column pairs (o, o + 1), o even, are stored as 16 bytes (x_o,
@@ -755,6 +791,7 @@ __device__ __noinline__ void ray_tables(SH& sh, RayShared& rs) {
     P.tabf[4 * (o >> 1) + (o & 1)] = -2.0f * sh2 * sh2;
     P.tabf[4 * (o >> 1) + 2 + (o & 1)] = s;
   }
+  dr.columns(rs, b0, b1);
   __syncthreads();
 }
 
@@ -831,7 +868,7 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
 
   for (;;) {
     // ---- the next batch of sectors: their anchors and offset tables
-    ray_tables<NL, LAW>(sh, rs);
+    ray_tables<NL, LAW>(sh, rs, NoDer{});
     const int b0 = rs.b0, b1 = rs.b1;
     if (b0 >= b1) break;
 
@@ -995,15 +1032,8 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
             cf wb;
             const cf t = tab_at(tps, ls - gbase);
             const float db2 = ray_eval<NL>(anchor(), t.x, t.y, ri, dri, nullptr, &wb);
-            // distance of the chord from the source centre (rounding: a few u
-            // of the coordinates, added to rout)
-            const cf d = wb - wa;
-            const float da2 = abs2(wa);
-            const float tt = __saturatef(-(wa.x * d.x + wa.y * d.y) * rcp_fast(fmaxf(abs2(d), 1e-37f)));
-            const cf cl = mk(fmaf(tt, d.x, wa.x), fmaf(tt, d.y, wa.y));
-            const AnchorF& an = anf[aidx];
-            const float ro = an.rout + 1e-6f * (fabsf(wa.x) + fabsf(wa.y) + fabsf(d.x) + fabsf(d.y));
-            const bool out = abs2(cl) > ro * ro, inn = fmaxf(da2, db2) < an.in2;
+            bool out, inn;
+            chord_test(anf[aidx], wa, wb, db2, out, inn);
             wa = wb;
             const bool all_out = __all_sync(0xffffffffu, out);
             const bool all_in = !spot && ls - l >= 2 && __all_sync(0xffffffffu, inn);

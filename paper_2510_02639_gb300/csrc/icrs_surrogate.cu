@@ -36,7 +36,6 @@ constexpr int NIN = 7, H = 128, NOUT = 2;
 constexpr int KIN = 16;    // layer-0 contraction, padded (one MMA K-step)
 constexpr int NOUTP = 16;  // layer-4 outputs, padded (smallest N for M = 128)
 constexpr int TM = 128;    // samples per tile (the MMA M)
-constexpr int NT = 128;    // threads: one per tile row / TMEM lane
 constexpr int NPARAM = ICRS_MLP_NPARAM;
 
 // offsets in the FP32 parameter vector (row-major [out][in] weights)
@@ -91,9 +90,10 @@ __global__ void pack_kernel(const float* __restrict__ theta, uint8_t* __restrict
   *reinterpret_cast<uint4*>(pack + byte) = *reinterpret_cast<const uint4*>(v);
 }
 
-__device__ __forceinline__ float silu(float z) { return z / (1.0f + expf(-z)); }
 __device__ __forceinline__ float silu_prime(float z) {
-  const float sg = 1.0f / (1.0f + expf(-z));
+  // (the reciprocal with one Newton correction)
+  const float d = 1.0f + expf(-z), r = rcp_fast(d);
+  const float sg = d < 1e37f ? fmaf(fmaf(-d, r, 1.0f), r, r) : 0.0f;
   return sg * (1.0f + z * (1.0f - sg));
 }
 
@@ -102,11 +102,6 @@ __device__ __forceinline__ void store8(uint8_t* dst, const float* x) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) h[i] = __float2bfloat16_rn(x[i]);
   *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(h);
-}
-
-__device__ __forceinline__ void copy16(uint8_t* dst, const uint8_t* src, int bytes, int tid) {
-  for (int i = tid; i < bytes / 16; i += NT)
-    reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(src)[i];
 }
 
 // Issue D = A B^T over K (multiple of 16) from K-major tiles: thread 0 only.
@@ -130,7 +125,7 @@ __device__ __forceinline__ void load_input_row(const float* __restrict__ feat, i
   }
 }
 
-// z / (1 + e^-z) as silu(), the division written out: the reciprocal's
+// SiLU z / (1 + e^-z), the division written out: the reciprocal's
 // approximation, one correction of the quotient by its exact remainder (the
 // usual correctly rounded division without its range handling: d >= 1; d = inf
 // gives 0, where the plain division gives -0).
@@ -245,121 +240,154 @@ mlp_infer_kernel(const uint8_t* __restrict__ pack, const float* __restrict__ the
 }
 
 // ---------------------------------------------------------------- training
-// One CTA per tile of 128 samples: forward (pre-activations and BF16
-// activations kept in the workspace), loss, backward, and the tile's
+// One CTA per tile of 128 samples: forward, loss, backward, and the tile's
 // gradient written to the workspace; reduce_adam_kernel sums the tiles in a
-// fixed order and applies Adam.
-constexpr size_t WS_Z = (size_t)4 * TM * H * 4;           // Z_l  [4][128][128] f32
-constexpr size_t WS_X0 = (size_t)TM * KIN * 2;            // X_0  [128][16] bf16
-constexpr size_t WS_X = (size_t)4 * TM * H * 2;           // X_1..X_4 [4][128][128] bf16
+// fixed order, applies Adam and repacks.
+//
+// The step is a chain of ten small contractions with an elementwise pass
+// between each two (64 tiles at a batch of 8192: fewer than SMs), so its time
+// is that chain's latency.  512 threads take a tile's passes (four per row,
+// 32 columns each); the activations X_0 .. X_4 stay in shared memory and the
+// backward contractions read them, and dZ, in place as MN-major operands (no
+// transposed copies); the bias gradients are contractions with a tile of ones;
+// the next weights arrive by bulk copies meanwhile.  128 threads with
+// transposed 2-byte stores, activations through the workspace and weights
+// copied by hand took 185 us of a 245 us step.
+constexpr int TR_NT = 512;
+constexpr int XB = H * H * 2, XB0 = H * KIN * 2;          // bytes of a [128][128] and a [128][16] tile
+constexpr size_t WS_Z = (size_t)4 * TM * H * 4;           // Z_l  [4][8][512] float4
 constexpr size_t WS_G = (((size_t)NPARAM * 4 + 255) / 256) * 256;
-constexpr size_t WS_TILE = WS_Z + WS_X0 + WS_X + WS_G + 256;  // + the tile's loss
-constexpr int TR_SMEM = 5 * H * H * 2 + TM * 2 * 4;
+constexpr size_t WS_TILE = WS_Z + WS_G + 256;             // + the tile's loss
+// shared memory: W_0 (later W_4^T) | W_4 | ones | X_0 | W_1, W_3, W_3^T, W_1^T |
+// X_1 | X_2 | X_3 | X_4 (first W_2, later W_2^T) | dZ
+constexpr int TR_S0 = 0, TR_S1 = XB0, TR_ONE = 2 * XB0, TR_X0 = 3 * XB0, TR_WA = 4 * XB0, TR_X1 = TR_WA + XB,
+              TR_DZ = TR_X1 + 4 * XB, TR_SMEM = TR_DZ + XB;
 
-__global__ void __launch_bounds__(NT, 1)
+__global__ void __launch_bounds__(TR_NT, 1)
 mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict__ theta,
                       const float* __restrict__ feat, const float* __restrict__ target, int n,
                       uint8_t* __restrict__ ws, int* __restrict__ err) {
   extern __shared__ __align__(1024) uint8_t sm[];
-  uint8_t* Wb = sm;                  // current layer's operand tile (W_l or W_l^T)
-  uint8_t* Xb = Wb + H * H * 2;      // forward A operand X_l [m][k]
-  uint8_t* DZ = Xb + H * H * 2;      // dZ_l [m][n]
-  uint8_t* DZT = DZ + H * H * 2;     // dZ_l^T [n][m]
-  uint8_t* XT = DZT + H * H * 2;     // X_l^T [k][m]
-  float* dz4 = reinterpret_cast<float*>(XT + H * H * 2);  // [128][2]
-  __shared__ uint64_t bar;
+  __shared__ __align__(16) float bias[4 * H + NOUT];
+  __shared__ uint64_t bar, wbar[3];  // contractions; copies into S0 / S1, WA, X_4's place
   __shared__ uint32_t tmem_sh;
-  __shared__ float red[NT / 32];
+  __shared__ float red[4];
   const int tid = threadIdx.x, warp = tid >> 5, lanei = tid & 31;
+  const int row = (warp & 3) * 32 + lanei;  // a warp reads its quarter of the TMEM lanes
+  const int col0 = (warp >> 2) * 32;        // first of this thread's 32 columns
   const int tile = blockIdx.x;
-  const int q = tile * TM + tid;
+  const int q = tile * TM + row;
   const bool valid = q < n;
   uint8_t* wt = ws + (size_t)tile * WS_TILE;
-  float* Zs = reinterpret_cast<float*>(wt);
-  __nv_bfloat16* X0s = reinterpret_cast<__nv_bfloat16*>(wt + WS_Z);
-  __nv_bfloat16* Xs = reinterpret_cast<__nv_bfloat16*>(wt + WS_Z + WS_X0);
-  float* Gs = reinterpret_cast<float*>(wt + WS_Z + WS_X0 + WS_X);
-  float* lossp = reinterpret_cast<float*>(wt + WS_Z + WS_X0 + WS_X + WS_G);
+  float4* Zs = reinterpret_cast<float4*>(wt);
+  float* Gs = reinterpret_cast<float*>(wt + WS_Z);
+  float* lossp = reinterpret_cast<float*>(wt + WS_Z + WS_G);
+  uint8_t* const DZ = sm + TR_DZ;
+  auto Xt = [&](int l) -> uint8_t* { return sm + (l == 0 ? TR_X0 : TR_X1 + (l - 1) * XB); };
 
-  if (tid == 0) tc::mbar_init(&bar, 1);
-  if (warp == 0) { tc::tmem_alloc(&tmem_sh, 256); tc::tmem_relinquish(); }
+  if (tid == 0) {
+    tc::mbar_init(&bar, 1);
+    for (int i = 0; i < 3; ++i) tc::mbar_init(&wbar[i], 1);
+    tc::fence_mbar_init();
+    tc::bulk_load2(sm + TR_S0, pack + PB_W0, XB0, sm + TR_S1, pack + PB_W4, XB0, &wbar[0]);
+    tc::bulk_load(sm + TR_WA, pack + PB_W1, XB, &wbar[1]);
+    tc::bulk_load(Xt(4), pack + PB_W1 + XB, XB, &wbar[2]);
+  }
+  if (warp == 0) { tc::tmem_alloc(&tmem_sh, 512); tc::tmem_relinquish(); }
+  for (int i = tid; i < 4 * H + NOUT; i += TR_NT)
+    bias[i] = i < 4 * H ? theta[b_off(i / H) + i % H] : theta[OB4 + i - 4 * H];
+  if (tid < XB0 / 16) {
+    const uint32_t o = 0x3f803f80u;  // two BF16 ones
+    reinterpret_cast<uint4*>(sm + TR_ONE)[tid] = make_uint4(o, o, o, o);
+  }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_sh;
-  const uint32_t Dx = tmem, Dw = tmem + 128;
-  const uint32_t lane = (uint32_t)(warp * 32) << 16;
-  const uint32_t sWb = tc::smem_addr(Wb), sXb = tc::smem_addr(Xb), sDZ = tc::smem_addr(DZ);
-  const uint32_t sDZT = tc::smem_addr(DZT), sXT = tc::smem_addr(XT);
-  uint32_t ph = 0;
-  bool failed = false;
+  const uint32_t Dx = tmem, Dw = tmem + 128, Db = tmem + 256, D4 = tmem + 272;
+  const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
+  const uint32_t sS = tc::smem_addr(sm);
+  uint32_t ph = 0, wph[3] = {0, 0, 0};
+  bool failed = false, bad = false;
   auto wait_mma = [&]() -> bool {
     const bool ok = tc::mbar_wait(&bar, ph, WAIT_TRIES);
     ph ^= 1u;
     tc::fence_after_sync();
-    return !__syncthreads_or(!ok);
+    return !__syncthreads_or(!ok || bad);
   };
   auto sync_for_mma = [&]() {
     tc::fence_async_smem();
     tc::fence_before_sync();
     __syncthreads();
   };
+  // thread 0: the copy that fills weight buffer i next has arrived
+  auto wait_w = [&](int i) {
+    if (!tc::mbar_wait(&wbar[i], wph[i], WAIT_TRIES)) bad = true;
+    wph[i] ^= 1u;
+  };
+  // D = A^T B over the tile's samples, both operands [sample][.] tiles of ka
+  // and kb columns
+  auto issue_t = [&](uint32_t d, uint32_t a, int ka, uint32_t b, int kb, int N) {
+    const uint32_t id = tc::idesc_bf16(TM, N, true, true);
+    for (int ks = 0; ks < TM / 16; ++ks)
+      tc::mma_bf16(d, tc::smem_desc(a + ks * 32 * ka, 16 * ka, 128), tc::smem_desc(b + ks * 32 * kb, 16 * kb, 128), id,
+                   ks > 0 ? 1u : 0u);
+  };
 
   do {
     // ---------------- forward
-    copy16(Wb, pack + PB_W0, H * KIN * 2, tid);
-    {
+    if (col0 == 0) {
       float f[16];
       load_input_row(feat, q, n, f);
-      store8(Xb + tc::kmajor_offset(tid, 0, KIN), f);
-      store8(Xb + tc::kmajor_offset(tid, 8, KIN), f + 8);
-      __align__(16) __nv_bfloat16 h[16];
-      for (int i = 0; i < 16; ++i) h[i] = __float2bfloat16_rn(f[i]);
-      reinterpret_cast<uint4*>(X0s + (size_t)tid * KIN)[0] = reinterpret_cast<const uint4*>(h)[0];
-      reinterpret_cast<uint4*>(X0s + (size_t)tid * KIN)[1] = reinterpret_cast<const uint4*>(h)[1];
+      store8(Xt(0) + tc::kmajor_offset(row, 0, KIN), f);
+      store8(Xt(0) + tc::kmajor_offset(row, 8, KIN), f + 8);
     }
-    sync_for_mma();
-    if (tid == 0) { tc::fence_after_sync(); issue_gemm(Dx, sXb, sWb, KIN, H, false); tc::mma_commit(&bar); }
-    if (!wait_mma()) { failed = true; break; }
-    for (int l = 0; l < 4; ++l) {
-      const float* b = theta + b_off(l);
-      float* Zl = Zs + (size_t)l * TM * H + (size_t)tid * H;
-      __nv_bfloat16* Xn = Xs + (size_t)l * TM * H + (size_t)tid * H;  // X_{l+1}
-      for (int c = 0; c < H; c += 16) {
-        float v[16];
-        tc::tmem_ld16(Dx + lane + c, v);
-        __align__(16) __nv_bfloat16 h[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          v[j] += b[c + j];
-          Zl[c + j] = v[j];
-          v[j] = silu(v[j]);
-          h[j] = __float2bfloat16_rn(v[j]);
-        }
-        reinterpret_cast<uint4*>(Xn + c)[0] = reinterpret_cast<const uint4*>(h)[0];
-        reinterpret_cast<uint4*>(Xn + c)[1] = reinterpret_cast<const uint4*>(h)[1];
-        store8(Xb + tc::kmajor_offset(tid, c, H), v);
-        store8(Xb + tc::kmajor_offset(tid, c + 8, H), v + 8);
-      }
-      if (l < 3) copy16(Wb, pack + PB_W1 + l * H * H * 2, H * H * 2, tid);
-      else copy16(Wb, pack + PB_W4, NOUTP * H * 2, tid);
+    for (int l = 0; l < 5; ++l) {
       sync_for_mma();
       if (tid == 0) {
         tc::fence_after_sync();
-        issue_gemm(Dx, sXb, sWb, H, l < 3 ? H : NOUTP, false);
+        if (l == 0) { wait_w(0); issue_gemm(Dx, sS + TR_X0, sS + TR_S0, KIN, H, false); }
+        else if (l < 4) {
+          const int w = l == 2 ? 2 : 1;
+          wait_w(w);
+          issue_gemm(Dx, tc::smem_addr(Xt(l)), w == 2 ? tc::smem_addr(Xt(4)) : sS + TR_WA, H, H, false);
+        } else issue_gemm(Dx, tc::smem_addr(Xt(4)), sS + TR_S1, H, NOUTP, false);
         tc::mma_commit(&bar);
       }
       if (!wait_mma()) { failed = true; break; }
+      // the weight buffer just read takes the next weights
+      if (tid == 0) {
+        if (l == 0) tc::bulk_load(sm + TR_S0, pack + PB_W4T, XB0, &wbar[0]);
+        if (l == 1) tc::bulk_load(sm + TR_WA, pack + PB_W1 + 2 * XB, XB, &wbar[1]);   // W_3
+        if (l == 3) tc::bulk_load(sm + TR_WA, pack + PB_W1T + 2 * XB, XB, &wbar[1]);  // W_3^T
+      }
+      if (l == 4) break;
+      const float* b = bias + l * H;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = col0 + 16 * h;
+        float v[16];
+        tc::tmem_ld16(Dx + lane + c, v);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] += b[c + j];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          Zs[(size_t)(l * 8 + h * 4 + j) * TR_NT + tid] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = silu_fast(v[j]);
+        store8(Xt(l + 1) + tc::kmajor_offset(row, c, H), v);
+        store8(Xt(l + 1) + tc::kmajor_offset(row, c + 8, H), v + 8);
+      }
     }
     if (failed) break;
     // ---------------- loss and dZ_4 (BF16-rounded)
-    float loss = 0.0f;
-    {
+    if (col0 == 0) {
+      float loss = 0.0f;
       float v[16];
       tc::tmem_ld16(Dx + lane, v);
       float d0 = 0.0f, d1 = 0.0f;
       if (valid) {
-        const float mu = v[0] + theta[OB4], s = v[1] + theta[OB4 + 1];
+        const float mu = v[0] + bias[4 * H], s = v[1] + bias[4 * H + 1];
         const float r = target[q] - mu, e = expf(-s);
         loss = 0.5f * (r * r * e + s);
         d0 = -r * e / (float)n;
@@ -367,113 +395,143 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
       }
       float g16[16];
       for (int j = 0; j < 16; ++j) g16[j] = 0.0f;
-      g16[0] = __bfloat162float(__float2bfloat16_rn(d0));
-      g16[1] = __bfloat162float(__float2bfloat16_rn(d1));
-      dz4[tid * 2] = g16[0];
-      dz4[tid * 2 + 1] = g16[1];
-      store8(DZ + tc::kmajor_offset(tid, 0, KIN), g16);
-      store8(DZ + tc::kmajor_offset(tid, 8, KIN), g16 + 8);
+      g16[0] = d0;
+      g16[1] = d1;
+      store8(DZ + tc::kmajor_offset(row, 0, KIN), g16);
+      store8(DZ + tc::kmajor_offset(row, 8, KIN), g16 + 8);
+      for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+      if (lanei == 0) red[warp] = loss;
     }
-    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-    if (lanei == 0) red[warp] = loss;
-    copy16(Wb, pack + PB_W4T, H * NOUTP * 2, tid);
     sync_for_mma();
     if (tid == 0) {
-      tc::fence_after_sync();
-      issue_gemm(Dx, sDZ, sWb, KIN, H, false);  // dX_4 = dZ_4 W_4
-      tc::mma_commit(&bar);
       lossp[0] = red[0] + red[1] + red[2] + red[3];
-    }
-    // dW_4, db_4 on the CUDA cores (two outputs): column k of X_4 is in Xb
-    {
-      float a0 = 0.0f, a1 = 0.0f;
-      for (int m = 0; m < TM; ++m) {
-        const float x = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(Xb + tc::kmajor_offset(m, tid, H)));
-        a0 = fmaf(dz4[m * 2], x, a0);
-        a1 = fmaf(dz4[m * 2 + 1], x, a1);
+      tc::fence_after_sync();
+      wait_w(0);
+      issue_gemm(Dx, sS + TR_DZ, sS + TR_S0, KIN, H, false);                         // dX_4 = dZ_4 W_4
+      issue_t(D4, tc::smem_addr(Xt(4)), H, sS + TR_DZ, KIN, NOUTP);                  // dW_4^T = X_4^T dZ_4
+      {
+        // db_4: every row of the ones' product is the column sums of dZ_4
+        const uint32_t id = tc::idesc_bf16(TM, NOUTP, false, true);
+        for (int ks = 0; ks < TM / 16; ++ks)
+          tc::mma_bf16(Db, tc::smem_desc(sS + TR_ONE, 128, 16 * KIN), tc::smem_desc(sS + TR_DZ + ks * 32 * KIN, 16 * KIN, 128),
+                       id, ks > 0 ? 1u : 0u);
       }
-      Gs[OW4 + tid] = a0;
-      Gs[OW4 + H + tid] = a1;
-      if (tid < 2) {
-        float sb = 0.0f;
-        for (int m = 0; m < TM; ++m) sb += dz4[m * 2 + tid];
-        Gs[OB4 + tid] = sb;
-      }
+      tc::mma_commit(&bar);
     }
     if (!wait_mma()) { failed = true; break; }
+    if (tid == 0) tc::bulk_load(Xt(4), pack + PB_W1T + XB, XB, &wbar[2]);  // W_2^T
+    if (col0 == 0) {
+      float v[16];
+      tc::tmem_ld16(D4 + lane, v);
+      Gs[OW4 + row] = v[0];
+      Gs[OW4 + H + row] = v[1];
+    } else if (warp == 4) {
+      float v[16];
+      tc::tmem_ld16(Db + lane, v);
+      if (lanei == 0) { Gs[OB4] = v[0]; Gs[OB4 + 1] = v[1]; }
+    }
     // ---------------- hidden layers, top down
-    for (int l = 3; l >= 0 && !failed; --l) {
+    for (int l = 3; l >= 0; --l) {
       const int Kl = l == 0 ? KIN : H;
       const int nin = l == 0 ? NIN : H;
-      const float* Zl = Zs + (size_t)l * TM * H + (size_t)tid * H;
-      for (int c = 0; c < H; c += 16) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = col0 + 16 * h;
         float v[16];
         tc::tmem_ld16(Dx + lane + c, v);
-        __align__(16) __nv_bfloat16 h[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          v[j] *= silu_prime(Zl[c + j]);
-          h[j] = __float2bfloat16_rn(v[j]);
+        for (int j = 0; j < 4; ++j) {
+          const float4 z = Zs[(size_t)(l * 8 + h * 4 + j) * TR_NT + tid];
+          v[4 * j] *= silu_prime(z.x);
+          v[4 * j + 1] *= silu_prime(z.y);
+          v[4 * j + 2] *= silu_prime(z.z);
+          v[4 * j + 3] *= silu_prime(z.w);
         }
-        store8(DZ + tc::kmajor_offset(tid, c, H), v);
-        store8(DZ + tc::kmajor_offset(tid, c + 8, H), v + 8);
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-          *reinterpret_cast<__nv_bfloat16*>(DZT + tc::kmajor_offset(c + j, tid, H)) = h[j];
+        store8(DZ + tc::kmajor_offset(row, c, H), v);
+        store8(DZ + tc::kmajor_offset(row, c + 8, H), v + 8);
       }
-      // X_l^T [k][m] from this row of X_l
-      const __nv_bfloat16* Xl = l == 0 ? X0s + (size_t)tid * KIN : Xs + (size_t)(l - 1) * TM * H + (size_t)tid * H;
-      for (int k = 0; k < Kl; ++k) *reinterpret_cast<__nv_bfloat16*>(XT + tc::kmajor_offset(k, tid, H)) = Xl[k];
-      if (l > 0) copy16(Wb, pack + PB_W1T + (l - 1) * H * H * 2, H * H * 2, tid);
       sync_for_mma();
       if (tid == 0) {
         tc::fence_after_sync();
-        issue_gemm(Dw, sDZT, sXT, H, Kl, false);       // dW_l = dZ_l^T X_l
-        if (l > 0) issue_gemm(Dx, sDZ, sWb, H, H, false);  // dX_l = dZ_l W_l
+        if (l > 0) {
+          const int w = l == 2 ? 2 : 1;
+          wait_w(w);
+          issue_gemm(Dx, sS + TR_DZ, w == 2 ? tc::smem_addr(Xt(4)) : sS + TR_WA, H, H, false);  // dX_l = dZ_l W_l
+        }
+        issue_t(Dw, sS + TR_DZ, H, tc::smem_addr(Xt(l)), Kl, Kl);                               // dW_l = dZ_l^T X_l
+        {
+          // db_l: dZ_l^T times ones
+          const uint32_t id = tc::idesc_bf16(TM, NOUTP, true, false);
+          for (int ks = 0; ks < TM / 16; ++ks)
+            tc::mma_bf16(Db, tc::smem_desc(sS + TR_DZ + ks * 32 * H, 16 * H, 128), tc::smem_desc(sS + TR_ONE, 128, 16 * KIN),
+                         id, ks > 0 ? 1u : 0u);
+        }
         tc::mma_commit(&bar);
       }
-      // db_l: row n = tid of dZ^T (the BF16 values the contractions use)
-      {
-        float sb = 0.0f;
-        for (int m = 0; m < TM; m += 8) {
-          const uint4 u = *reinterpret_cast<const uint4*>(DZT + tc::kmajor_offset(tid, m, H));
-          const __nv_bfloat16* hh = reinterpret_cast<const __nv_bfloat16*>(&u);
-          for (int j = 0; j < 8; ++j) sb += __bfloat162float(hh[j]);
-        }
-        Gs[b_off(l) + tid] = sb;
-      }
       if (!wait_mma()) { failed = true; break; }
-      for (int c = 0; c < Kl; c += 16) {
+      if (tid == 0 && l == 3) tc::bulk_load(sm + TR_WA, pack + PB_W1T, XB, &wbar[1]);  // W_1^T
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = col0 + 16 * h;
+        if (c >= Kl) continue;  // (a whole warp)
         float v[16];
         tc::tmem_ld16(Dw + lane + c, v);
         for (int j = 0; j < 16; ++j)
-          if (c + j < nin) Gs[w_off(l) + tid * nin + c + j] = v[j];
+          if (c + j < nin) Gs[w_off(l) + row * nin + c + j] = v[j];
       }
-      tc::fence_before_sync();
-      __syncthreads();
+      if (col0 == 0) {
+        float v[16];
+        tc::tmem_ld16(Db + lane, v);
+        Gs[b_off(l) + row] = v[0];
+      }
     }
   } while (false);
-  if (failed && tid == 0 && err) atomicExch(err, 1);
+  if ((failed || bad) && tid == 0 && err) atomicExch(err, 1);
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 256);
+  if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
-// Sum of the tile gradients (fixed order), optional output, Adam update.
-__global__ void reduce_adam_kernel(float* __restrict__ theta, float* __restrict__ m1, float* __restrict__ m2,
-                                   const uint8_t* __restrict__ ws, int ntiles, int n, int step, float lr,
-                                   float* __restrict__ grad_out, float* __restrict__ loss_out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0 && loss_out) {
+// Byte of the BF16 weight (no, ni) of layer l in the packed operands (and of
+// its transposed copy, l > 0).
+__device__ __forceinline__ void packed_offsets(int l, int no, int ni, int* w, int* wt) {
+  if (l == 0) { *w = PB_W0 + tc::kmajor_offset(no, ni, KIN); *wt = -1; }
+  else if (l < 4) {
+    *w = PB_W1 + (l - 1) * XB + tc::kmajor_offset(no, ni, H);
+    *wt = PB_W1T + (l - 1) * XB + tc::kmajor_offset(ni, no, H);
+  } else {
+    *w = PB_W4 + tc::kmajor_offset(no, ni, H);
+    *wt = PB_W4T + tc::kmajor_offset(ni, no, NOUTP);
+  }
+}
+
+// Sum of the tile gradients (fixed order: eight interleaved partial sums, then
+// their sum), optional output, Adam update, and the updated weights into the
+// packed operands (whose padding stays zero).  A block takes 32 parameters
+// with 8 threads each: one thread per parameter walked the 64 tiles of a batch
+// of 8192 one load after another.
+constexpr int RA_P = 32, RA_T = 8;
+__global__ void __launch_bounds__(RA_P * RA_T)
+reduce_adam_kernel(float* __restrict__ theta, float* __restrict__ m1, float* __restrict__ m2,
+                   const uint8_t* __restrict__ ws, int ntiles, int n, int step, float lr,
+                   float* __restrict__ grad_out, float* __restrict__ loss_out, uint8_t* __restrict__ pack) {
+  __shared__ float part[RA_T][RA_P];
+  const int x = threadIdx.x % RA_P, y = threadIdx.x / RA_P;
+  const int i = blockIdx.x * RA_P + x;
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0 && loss_out) {
     double L = 0.0;
-    for (int t = 0; t < ntiles; ++t)
-      L += *reinterpret_cast<const float*>(ws + (size_t)t * WS_TILE + WS_Z + WS_X0 + WS_X + WS_G);
+    for (int t = 0; t < ntiles; ++t) L += *reinterpret_cast<const float*>(ws + (size_t)t * WS_TILE + WS_Z + WS_G);
     *loss_out = (float)(L / n);
   }
-  if (i >= NPARAM) return;
   float g = 0.0f;
-  for (int t = 0; t < ntiles; ++t)
-    g += reinterpret_cast<const float*>(ws + (size_t)t * WS_TILE + WS_Z + WS_X0 + WS_X)[i];
+  if (i < NPARAM)
+#pragma unroll 4
+    for (int t = y; t < ntiles; t += RA_T) g += reinterpret_cast<const float*>(ws + (size_t)t * WS_TILE + WS_Z)[i];
+  part[y][x] = g;
+  __syncthreads();
+  if (y != 0 || i >= NPARAM) return;
+#pragma unroll
+  for (int k = 1; k < RA_T; ++k) g += part[k][x];
   if (grad_out) grad_out[i] = g;
   if (lr > 0.0f) {
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -483,7 +541,18 @@ __global__ void reduce_adam_kernel(float* __restrict__ theta, float* __restrict_
     m2[i] = v;
     const float mh = a / (1.0f - powf(b1, (float)step));
     const float vh = v / (1.0f - powf(b2, (float)step));
-    theta[i] -= lr * mh / (sqrtf(vh) + eps);
+    const float th = theta[i] - lr * mh / (sqrtf(vh) + eps);
+    theta[i] = th;
+    int l = 0;
+    while (l < 4 && i >= w_off(l + 1)) ++l;
+    if (i < b_off(l)) {  // a weight
+      const int nin = l == 0 ? NIN : H, k = i - w_off(l);
+      int w, wt;
+      packed_offsets(l, k / nin, k % nin, &w, &wt);
+      const __nv_bfloat16 h = __float2bfloat16_rn(th);
+      *reinterpret_cast<__nv_bfloat16*>(pack + w) = h;
+      if (wt >= 0) *reinterpret_cast<__nv_bfloat16*>(pack + wt) = h;
+    }
   }
 }
 
@@ -736,7 +805,7 @@ __global__ void batch_kernel(const float4* __restrict__ feat, const float* __res
 //   - host-side schedulers with a fixed memory budget that own no allocator;
 //   - processes that must leave the device allocator untouched between steps.
 // For them the step can use this file-scope array: 32 tiles, i.e. batches of
-// up to 4096 samples, about 19 MB, reserved when this module is loaded.
+// up to 4096 samples, about 15 MB, reserved when this module is loaded.
 constexpr int STATIC_MAX_N = ICRS_MLP_STATIC_MAX_N;
 constexpr size_t STATIC_WS_BYTES = (size_t)((STATIC_MAX_N + TM - 1) / TM) * WS_TILE;
 static __device__ __align__(256) uint8_t g_train_scratch[STATIC_WS_BYTES];
@@ -814,14 +883,10 @@ int icrs_mlp_train_step(float* theta, float* adam_m, float* adam_v, void* pack, 
   if (cudaFuncSetAttribute(mlp_train_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TR_SMEM) != cudaSuccess)
     return ICRS_ECUDA;
   const int ntiles = (n + TM - 1) / TM;
-  mlp_train_tile_kernel<<<ntiles, NT, TR_SMEM, st>>>((const uint8_t*)pack, theta, feat, target, n,
-                                                     (uint8_t*)workspace, err);
-  reduce_adam_kernel<<<(NPARAM + 255) / 256, 256, 0, st>>>(theta, adam_m, adam_v, (const uint8_t*)workspace, ntiles,
-                                                           n, step, lr, grad, loss);
-  if (lr > 0.0f) {
-    const int chunks = PACK_BYTES / 16;
-    pack_kernel<<<(chunks + 255) / 256, 256, 0, st>>>(theta, (uint8_t*)pack);
-  }
+  mlp_train_tile_kernel<<<ntiles, TR_NT, TR_SMEM, st>>>((const uint8_t*)pack, theta, feat, target, n,
+                                                        (uint8_t*)workspace, err);
+  reduce_adam_kernel<<<(NPARAM + RA_P - 1) / RA_P, RA_P * RA_T, 0, st>>>(
+      theta, adam_m, adam_v, (const uint8_t*)workspace, ntiles, n, step, lr, grad, loss, (uint8_t*)pack);
   return cudaGetLastError() == cudaSuccess ? ICRS_OK : ICRS_ECUDA;
 }
 

@@ -10,6 +10,12 @@
 // with LBO = 128 (core matrices adjacent along K) and SBO = 16 * K (row groups
 // after a full K extent).  One MMA consumes K = 16, i.e. two core matrices
 // along K, so successive K-steps advance the descriptor start by 256 bytes.
+//
+// The same tile read the other way round ("MN-major": the operand's M or N
+// index runs along k, its contraction along r) needs no copy: the core
+// matrices are the same, LBO is then the step between groups of 8 rows along
+// the contraction (16 * K) and SBO the step between groups of 8 along M or N
+// (128), and one MMA's K = 16 is two row groups, 32 * K bytes.
 #pragma once
 
 #include <stdint.h>
@@ -38,9 +44,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
 // Instruction descriptor of kind::f16 with BF16 A and B, FP32 D, both
 // operands K-major, dense: D format (bits 4-5) = 1 (F32), A format (bits 7-9)
 // = 1 (BF16), B format (bits 10-12) = 1 (BF16), N >> 3 in bits 17-22, M >> 4
-// in bits 24-28.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// in bits 24-28; bits 15 and 16: A, B MN-major.
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn = false, bool b_mn = false) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
+         ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -76,6 +83,20 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_addr(dst)),
                "l"(src), "r"(bytes), "r"(smem_addr(bar))
+               : "memory");
+}
+
+// Two bulk copies that complete one phase together.
+__device__ __forceinline__ void bulk_load2(void* d0, const void* s0, uint32_t b0, void* d1, const void* s1, uint32_t b1,
+                                           uint64_t* bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(b0 + b1) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_addr(d0)),
+               "l"(s0), "r"(b0), "r"(smem_addr(bar))
+               : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_addr(d1)),
+               "l"(s1), "r"(b1), "r"(smem_addr(bar))
                : "memory");
 }
 

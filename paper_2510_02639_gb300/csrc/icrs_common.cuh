@@ -283,6 +283,7 @@ __device__ inline void cauchy_start(const cf* b, cf* z) {
 // the number of iterations, or -1 if the cap was hit; last[k] = |last step|.
 template <int N>
 __device__ inline int ehrlich_aberth_f32(const cf* b, cf* z, int max_iter, float tol, float* last) {
+  constexpr int U = N > 5 ? 1 : N;
   float ab[N + 1];
 #pragma unroll
   for (int l = 0; l <= N; ++l) ab[l] = sqrtf(abs2(b[l]));
@@ -290,7 +291,9 @@ __device__ inline int ehrlich_aberth_f32(const cf* b, cf* z, int max_iter, float
     cf dz[N];
     float noise[N];
     bool done = true;
-#pragma unroll
+    // (unrolled, the ten roots of a triple lens are 40 KB of code an iteration,
+    // more than the instruction cache holds)
+#pragma unroll U
     for (int k = 0; k < N; ++k) {
       cf p, dp;
       horner2<N, float>(b, z[k], p, dp);
@@ -307,7 +310,7 @@ __device__ inline int ehrlich_aberth_f32(const cf* b, cf* z, int max_iter, float
       dz[k] = dv(W, den);
       if (!(abs2(p) > 0.0f)) dz[k] = mk(0.0f, 0.0f);
     }
-#pragma unroll
+#pragma unroll U
     for (int k = 0; k < N; ++k) {
       z[k] = z[k] - dz[k];
       float st = sqrtf(abs2(dz[k]));
@@ -323,21 +326,22 @@ __device__ inline int ehrlich_aberth_f32(const cf* b, cf* z, int max_iter, float
 // Ehrlich-Aberth iteration in FP64 (Sec. 3.1): the fallback for positions
 // whose FP32 roots do not give a trustworthy image set (clusters of close
 // roots next to a critical curve, which FP32 cannot separate).  Stops when every step is
-// below 1e-14 max(1, |z|) or twice the FP64 rounding level of P at the root.
+// below 1e-14 max(1, |z|) or twice the FP64 rounding level of P at the root
+// (the test's moduli are taken in FP32: they are only compared).
 template <int N>
 __device__ inline int ehrlich_aberth_f64(const cd* b, cd* z, int max_iter) {
-  double ab[N + 1];
-  for (int l = 0; l <= N; ++l) ab[l] = sqrt(abs2(b[l]));
+  float ab[N + 1];
+  for (int l = 0; l <= N; ++l) ab[l] = sqrtf((float)abs2(b[l]));
   for (int it = 0; it < max_iter; ++it) {
     cd dz[N];
-    double noise[N];
+    float noise[N];
     bool done = true;
     for (int k = 0; k < N; ++k) {
       cd p, dp;
       horner2<N, double>(b, z[k], p, dp);
-      double az = sqrt(abs2(z[k])), pa = ab[N];
-      for (int l = N - 1; l >= 0; --l) pa = fma(pa, az, ab[l]);
-      noise[k] = 1.1102230246251565e-16 * pa / fmax(sqrt(abs2(dp)), 1e-300);
+      float az = sqrtf((float)abs2(z[k])), pa = ab[N];
+      for (int l = N - 1; l >= 0; --l) pa = fmaf(pa, az, ab[l]);
+      noise[k] = 1.1102230246251565e-16f * pa / fmaxf(sqrtf((float)abs2(dp)), 1e-30f);
       cd W = dv(p, dp);
       cd S = mk(0.0, 0.0);
       for (int j = 0; j < N; ++j)
@@ -347,8 +351,8 @@ __device__ inline int ehrlich_aberth_f64(const cd* b, cd* z, int max_iter) {
     }
     for (int k = 0; k < N; ++k) {
       z[k] = z[k] - dz[k];
-      double st = sqrt(abs2(dz[k]));
-      if (!(st <= fmax(1e-14 * fmax(1.0, sqrt(abs2(z[k]))), 2.0 * noise[k]))) done = false;
+      const float st = sqrtf((float)abs2(dz[k]));
+      if (!(st <= fmaxf(1e-14f * fmaxf(1.0f, sqrtf((float)abs2(z[k]))), 2.0f * noise[k]))) done = false;
     }
     if (done) return it + 1;
   }

@@ -84,6 +84,7 @@ struct Shared {
   float eps32[3];
   cf aj32[3][3];       // [frame j][lens i]: a_i - a_j (FP32)
   cf D32[3][4], E32[3][3];  // polynomial parts in frame j (FP32)
+  cd D64[3][4], E64[3][3];  // the same in FP64
   df adf[3][3][2];     // [frame j][lens i][x/y]: a_i - a_j (double-float)
   df adf_ll[2];        // a_ll (original frame, double-float)
   df epsdf[3];
@@ -106,6 +107,7 @@ struct Shared {
   int startT[MAXT];
   unsigned int t_rlo_u[MAXT], t_rhi_l[MAXT];
   unsigned long long t_rlo[MAXT], t_rhi[MAXT];
+  unsigned int t_s[MAXT][2];                // FP32 keys of the refined radius: rmin_hi, rmax_lo
   double rlo[MAXT], hr[MAXT];
   float rlh[MAXT], rll[MAXT], ihr[MAXT];  // rlo as a float pair, 1 / hr
   int rsmall[MAXT];    // 1: hr > 0 but the run is below TINY_EXTENT rho; 2: hr = 0
@@ -117,7 +119,7 @@ struct Shared {
   int origin_in;
   int c_cnt[MAXCELL];
   unsigned int c_u[MAXCELL][4];             // FP32 keys: rmin_hi, rmax_lo, tmin_hi, tmax_lo
-  unsigned int c_s[MAXCELL][2];             // FP32 keys of the refined angle: tmin_hi, tmax_lo
+  unsigned int c_s[MAXCELL][4];             // FP32 keys of the refined radius and angle: rmin_hi, rmax_lo, tmin_hi, tmax_lo
   float2 c_ref[MAXCELL][2];                 // direction of the FP32 angle extremes
   unsigned long long c_x[MAXCELL][4];       // FP64 keys: rmin, rmax, tmin, tmax
   int nbox;
@@ -216,10 +218,9 @@ __device__ inline int validate_root64(const Shared& sh, cd z0, cd w, double img_
   double eps[NL];
   cd a[NL];
   for (int i = 0; i < NL; ++i) { eps[i] = sh.L.eps[i]; a[i] = sh.L.a[i] - sh.L.a[j]; }
-  cd D[NL + 1], E[NL], b[N + 1];
-  poly_DE<NL, double>(eps, a, D, E);
+  cd b[N + 1];
   cd wj = w - sh.L.a[j];
-  lens_poly<NL, double>(eps, a, D, E, wj, b);
+  lens_poly<NL, double>(eps, a, sh.D64[j], sh.E64[j], wj, b);
   cd x = z0 - sh.L.a[j];
   bool done = false;
   for (int it = 0; it < 8; ++it) {
@@ -283,10 +284,136 @@ __device__ inline void point_tangents(const Shared& sh, const DerShared& ds, dou
   }
 }
 
-// FP64 re-solve of limb point k (all roots, FP64 Ehrlich-Aberth warm-started
-// from the FP32 roots in the lightest lens's frame, FP64 validation of each
-// root); rewrites the point's slots and returns its image count.  Kept out of
-// line: it runs only for limb points with an illegal FP32 image count.
+// FP64 Ehrlich-Aberth by one warp, root j of limb point g on lane g N + j (np
+// points): the same iteration, operation by operation, as one thread's over
+// all roots.  With one point the differences 1 / (z_k - z_j) are spread over
+// the lanes besides.  Only the stopping test's moduli are taken in FP32: it
+// compares steps with a rounding level.  b: this lane's point's polynomial.
+// Returns whether this lane's point converged.
+template <int N>
+__device__ inline bool ehrlich_aberth_f64_warp(const cd* b, cd* zj, int np, int max_iter) {
+  constexpr int NP2 = N * (N - 1), R = (NP2 + 31) / 32;
+  const int lane = threadIdx.x & 31;
+  const bool act = lane < np * N;
+  const int g = act ? lane / N : 0, k = act ? lane - g * N : 0;
+  const unsigned mine = ((1u << N) - 1u) << (g * N);  // the lanes of this point
+  float ab[N + 1];
+#pragma unroll
+  for (int l = 0; l <= N; ++l) ab[l] = sqrtf((float)abs2(b[l]));
+  cd z = *zj;
+  bool done = false;
+#pragma unroll 1
+  for (int it = 0; it < max_iter; ++it) {
+    cd S = mk(0.0, 0.0);
+    if (np == 1) {
+      cd iv[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int t = min(lane + 32 * r, NP2 - 1), kk = t / (N - 1), jj = t % (N - 1), j = jj + (jj >= kk ? 1 : 0);
+        const cd a = mk(__shfl_sync(0xffffffffu, z.x, kk), __shfl_sync(0xffffffffu, z.y, kk));
+        const cd c = mk(__shfl_sync(0xffffffffu, z.x, j), __shfl_sync(0xffffffffu, z.y, j));
+        iv[r] = inv(a - c);
+      }
+#pragma unroll
+      for (int jj = 0; jj < N - 1; ++jj) {  // j = 0 .. N - 1 without k, in order
+        const int t = k * (N - 1) + jj;
+        cd v = mk(0.0, 0.0);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const cd u = mk(__shfl_sync(0xffffffffu, iv[r].x, t & 31), __shfl_sync(0xffffffffu, iv[r].y, t & 31));
+          if ((t >> 5) == r) v = u;
+        }
+        S = S + v;
+      }
+    } else {
+#pragma unroll 1
+      for (int jj = 0; jj < N - 1; ++jj) {
+        const int j = g * N + jj + (jj >= k ? 1 : 0);
+        const cd c = mk(__shfl_sync(0xffffffffu, z.x, j), __shfl_sync(0xffffffffu, z.y, j));
+        S = S + inv(z - c);
+      }
+    }
+    cd p, dp;
+    horner2<N, double>(b, z, p, dp);
+    const float az = sqrtf((float)abs2(z));
+    float pa = ab[N];
+#pragma unroll
+    for (int l = N - 1; l >= 0; --l) pa = fmaf(pa, az, ab[l]);
+    const float noise = 1.1102230246251565e-16f * pa / fmaxf(sqrtf((float)abs2(dp)), 1e-30f);
+    const cd W = dv(p, dp);
+    cd dz = dv(W, mk(1.0, 0.0) - W * S);
+    if (!(abs2(p) > 0.0)) dz = mk(0.0, 0.0);
+    if (!done) z = z - dz;
+    const float st = sqrtf((float)abs2(dz));
+    const bool conv = st <= fmaxf(1e-14f * fmaxf(1.0f, sqrtf((float)abs2(z))), 2.0f * noise);
+    const unsigned cb = __ballot_sync(0xffffffffu, conv);  // (every lane votes, done or not)
+    done = done || (cb & mine) == mine;
+    if (__all_sync(0xffffffffu, done)) break;
+  }
+  *zj = z;
+  return done;
+}
+
+// FP64 re-solve of the limb points queue[0 .. np - 1] (all roots, FP64
+// Ehrlich-Aberth warm-started from the FP32 roots in the lightest lens's
+// frame, FP64 validation of each root) by one warp, one root per lane;
+// rewrites the points' slots and flags an illegal image count.  It runs only
+// for limb points with an untrustworthy FP32 image set, but with a thread for
+// each a single one held its block for 400k cycles (an FP64 division takes 570,
+// an iteration 35 of them).
+template <int NL>
+__device__ __noinline__ void resolve_limb_points64(Shared& sh, const int* queue, int np, int K, int max_iter,
+                                                   double img_tol, int PMAX, cf* phi, float* r32, float* rl32, float* t32,
+                                                   float* e32, short* pidx, uint8_t* meta, double* pr, double* pt) {
+  constexpr int N = NL * NL + 1;
+  const int lane = threadIdx.x & 31;
+  const bool act = lane < np * N;
+  const int g = act ? lane / N : 0, jr = act ? lane - g * N : 0;
+  const int k = queue[g];
+  const int ll = sh.L.ll;
+  const cd w = limb_point64(sh, k, K);
+  cd b[N + 1], zj;
+  {
+    double eps[NL];
+    cd a[NL], z[N];
+    for (int i2 = 0; i2 < NL; ++i2) { eps[i2] = sh.L.eps[i2]; a[i2] = sh.L.a[i2] - sh.L.a[ll]; }
+    lens_poly<NL, double>(eps, a, sh.D64[ll], sh.E64[ll], w - sh.L.a[ll], b);
+    for (int j = 0; j < N; ++j) z[j] = tod(phi[k * N + j]);
+    // separate coincident starts
+    for (int j = 1; j < N; ++j)
+      for (int i2 = 0; i2 < j; ++i2)
+        if (abs2(z[j] - z[i2]) < 1e-20) z[j] = z[j] + mk(1e-7 * (j + 1), 1e-7 * j);
+    zj = z[0];
+#pragma unroll
+    for (int j = 1; j < N; ++j) if (jr == j) zj = z[j];
+  }
+  __syncwarp();
+  if (!ehrlich_aberth_f64_warp<N>(b, &zj, np, max_iter) && act) atomicOr(&sh.status, ICRS_ST_NONCONV);
+  bool img = false;
+  if (act) {
+    const int ps = k * N + jr;
+    phi[ps] = tof(zj);
+    pidx[ps] = -1;
+    uint8_t mm = 0;
+    double r, th;
+    if (validate_root64<NL>(sh, zj + sh.L.a[ll], w, img_tol, &r, &th)) {
+      img = true;
+      const int pi = atomicAdd(&sh.pn, 1);
+      const float rh = (float)r;
+      r32[ps] = rh; rl32[ps] = (float)(r - (double)rh); t32[ps] = (float)th;
+      if (pi < PMAX) { pr[pi] = r; pt[pi] = th; pidx[ps] = (short)pi; e32[ps] = 0.f; mm = M_VALID | M_EXACT; }
+      else { e32[ps] = 1e-12f; mm = M_VALID; atomicOr(&sh.status, ICRS_ST_OVERFLOW); }
+    }
+    meta[ps] = mm;
+  }
+  const int m = __popc(__ballot_sync(0xffffffffu, img) & (((1u << N) - 1u) << (g * N)));
+  const bool legal = (NL == 2) ? (m == 3 || m == 5) : (m == 4 || m == 6 || m == 8 || m == 10);
+  if (act && !legal) atomicOr(&sh.status, ICRS_ST_IMGCOUNT);
+}
+
+// The same for one limb point by one thread, for queues that fill the warps:
+// the FP64 pipe then bounds either form, and this one forms a point's
+// polynomial once.  Returns the image count.
 template <int NL>
 __device__ __noinline__ int resolve_limb_point64(Shared& sh, int k, int K, int max_iter, double img_tol, int PMAX,
                                                  cf* phi, float* r32, float* rl32, float* t32, float* e32, short* pidx,
@@ -295,10 +422,9 @@ __device__ __noinline__ int resolve_limb_point64(Shared& sh, int k, int K, int m
   const int ll = sh.L.ll;
   const cd w = limb_point64(sh, k, K);
   double eps[NL];
-  cd a[NL], D[NL + 1], Ee[NL], b[N + 1], z[N];
+  cd a[NL], b[N + 1], z[N];
   for (int i2 = 0; i2 < NL; ++i2) { eps[i2] = sh.L.eps[i2]; a[i2] = sh.L.a[i2] - sh.L.a[ll]; }
-  poly_DE<NL, double>(eps, a, D, Ee);
-  lens_poly<NL, double>(eps, a, D, Ee, w - sh.L.a[ll], b);
+  lens_poly<NL, double>(eps, a, sh.D64[ll], sh.E64[ll], w - sh.L.a[ll], b);
   for (int j = 0; j < N; ++j) z[j] = tod(phi[k * N + j]);
   // separate coincident starts
   for (int j = 1; j < N; ++j)
@@ -306,6 +432,7 @@ __device__ __noinline__ int resolve_limb_point64(Shared& sh, int k, int K, int m
       if (abs2(z[j] - z[i2]) < 1e-20) z[j] = z[j] + mk(1e-7 * (j + 1), 1e-7 * j);
   if (ehrlich_aberth_f64<N>(b, z, max_iter) < 0) atomicOr(&sh.status, ICRS_ST_NONCONV);
   int m = 0;
+#pragma unroll 1
   for (int j = 0; j < N; ++j) {
     const int ps = k * N + j;
     phi[ps] = tof(z[j]);
@@ -490,8 +617,8 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
           cd a[NL], D[NL + 1], Ee[NL];
           for (int i = 0; i < NL; ++i) { eps[i] = sh.L.eps[i]; a[i] = sh.L.a[i] - sh.L.a[j]; sh.aj32[j][i] = tof(a[i]); }
           poly_DE<NL, double>(eps, a, D, Ee);
-          for (int i = 0; i <= NL; ++i) sh.D32[j][i] = tof(D[i]);
-          for (int i = 0; i < NL; ++i) sh.E32[j][i] = tof(Ee[i]);
+          for (int i = 0; i <= NL; ++i) { sh.D32[j][i] = tof(D[i]); sh.D64[j][i] = D[i]; }
+          for (int i = 0; i < NL; ++i) { sh.E32[j][i] = tof(Ee[i]); sh.E64[j][i] = Ee[i]; }
           for (int i = 0; i < NL; ++i) { sh.adf[j][i][0] = df_from_double(a[i].x); sh.adf[j][i][1] = df_from_double(a[i].y); }
           sh.epsdf[j] = df_from_double(sh.L.eps[j]);
         }
@@ -899,9 +1026,17 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
         const float r = ex ? (float)pr[pidx[ps]] : r32[ps];
         const float th = ex ? (float)pt[pidx[ps]] : t32[ps];
         if (!ex && !(e32[ps] <= EE_SUSPECT * fmaxf(1.0f, r))) suspect = true;
-        float sn, cs;
-        sincosf(th, &sn, &cs);
-        const float x = r * cs, y = r * sn;
+        // (the refined position itself; a polished or validated root's is r e^{i th})
+        float x, y;
+        if (ex) {
+          float sn, cs;
+          sincosf(th, &sn, &cs);
+          x = r * cs - (float)sh.L.a[ll].x;
+          y = r * sn - (float)sh.L.a[ll].y;
+        } else {
+          x = phi[ps].x;
+          y = phi[ps].y;
+        }
         for (int i2 = 0; i2 < m; ++i2) {
           const float dx = x - zx[i2], dy = y - zy[i2];
           const float tol = DUP_TOL * fmaxf(1.0f, r);
@@ -915,12 +1050,22 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     __syncthreads();
     {
       const int qn = min(sh.qn, QMAX);
-      for (int qi = tid; qi < qn; qi += NT) {
-        const int k = queue[qi];
-        atomicAdd(&sh.cnt[1], 1);
-        const int m = resolve_limb_point64<NL>(sh, k, K, g.max_iter, g.img_tol, PMAX, phi, r32, rl32, t32, e32, pidx,
-                                               meta, pr, pt);
-        if (!legal_count(m)) atomicOr(&sh.status, ICRS_ST_IMGCOUNT);
+      // a few points: one per warp; more: as many as a warp has lanes for;
+      // beyond one round of those: one per thread
+      const int np = qn <= NW ? 1 : 32 / N;
+      if (qn <= NW * (32 / N)) {
+        for (int qi = warp * np; qi < qn; qi += NW * np) {
+          if (lane == 0) atomicAdd(&sh.cnt[1], min(np, qn - qi));
+          resolve_limb_points64<NL>(sh, queue + qi, min(np, qn - qi), K, g.max_iter, g.img_tol, PMAX, phi, r32, rl32,
+                                    t32, e32, pidx, meta, pr, pt);
+        }
+      } else {
+        for (int qi = tid; qi < qn; qi += NT) {
+          atomicAdd(&sh.cnt[1], 1);
+          const int m = resolve_limb_point64<NL>(sh, queue[qi], K, g.max_iter, g.img_tol, PMAX, phi, r32, rl32, t32, e32,
+                                                 pidx, meta, pr, pt);
+          if (!legal_count(m)) atomicOr(&sh.status, ICRS_ST_IMGCOUNT);
+        }
       }
     }
     __syncthreads();
@@ -1051,6 +1196,7 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
       if (b == 0) {
         sh.t_rlo_u[T] = 0xffffffffu; sh.t_rhi_l[T] = 0u;
         sh.t_rlo[T] = ~0ull; sh.t_rhi[T] = 0ull;
+        sh.t_s[T][0] = 0xffffffffu; sh.t_s[T][1] = 0u;
         sh.rocc[T] = 0u;
       }
     }
@@ -1125,33 +1271,43 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     });
     __syncthreads();
     const float tiny = TINY_EXTENT * rho32;
-    // r of a slot and its error bound (FP64 if polished, else double-float)
-    auto re = [&](int ps) -> double { return (meta[ps] & M_EXACT) ? 0.0 : (double)e32[ps]; };
+    // r of a slot (the double-float r32 + rl32, which a polish sets too) less a
+    // nearby float, and its error bound: the difference of the high parts is
+    // exact, so the sum keeps 1e-7 of the difference
+    auto r_from = [&](int ps, float ref, float* err) -> float {
+      const float d = (r32[ps] - ref) + rl32[ps];
+      *err = ((meta[ps] & M_EXACT) ? 0.f : e32[ps]) + 2e-7f * fabsf(d) + 1e-14f * r32[ps];
+      return d;
+    };
     for (int ps = tid; ps < NP; ps += NT) {
       if (!(meta[ps] & M_VALID)) continue;
       int T = sh.runT[tb[ps]];
       float r = r32[ps], er = (meta[ps] & M_EXACT) ? 4.0f * EPS32 * r : e32[ps] + 4.0f * EPS32 * r;
       if (fkey(r - er) <= sh.t_rlo_u[T] || fkey(r + er) >= sh.t_rhi_l[T]) {
         meta[ps] |= M_CAND;
-        const double R = rv(ps), E_ = re(ps);
-        atomicMin(&sh.t_rlo[T], dkey(R + E_));
-        atomicMax(&sh.t_rhi[T], dkey(R - E_));
+        float e_;
+        const float lo = r_from(ps, fkey_inv(sh.t_rlo_u[T]), &e_);
+        atomicMin(&sh.t_s[T][0], fkey(lo + e_));
+        const float hi = r_from(ps, fkey_inv(sh.t_rhi_l[T]), &e_);
+        atomicMax(&sh.t_s[T][1], fkey(hi - e_));
       }
     }
     __syncthreads();
     for (int ps = tid; ps < NP; ps += NT) {
       if (!(meta[ps] & M_CAND)) continue;
       int T = sh.runT[tb[ps]];
-      const double R = rv(ps), E_ = re(ps);
-      if (!(dkey(R - E_) <= sh.t_rlo[T] || dkey(R + E_) >= sh.t_rhi[T])) { meta[ps] &= (uint8_t)~M_CAND; continue; }
+      float e_;
+      const float lo = r_from(ps, fkey_inv(sh.t_rlo_u[T]), &e_);
+      bool cand = fkey(lo - e_) <= sh.t_s[T][0];
+      const float hi = r_from(ps, fkey_inv(sh.t_rhi_l[T]), &e_);
+      cand = cand || fkey(hi + e_) >= sh.t_s[T][1];
+      if (!cand) { meta[ps] &= (uint8_t)~M_CAND; continue; }
       // an image smaller than tiny contributes below the parity tolerance:
       // its decisions stay in FP32
       bool is_tiny = fkey_inv(sh.t_rhi_l[T]) - fkey_inv(sh.t_rlo_u[T]) < tiny;
       // the double-float r (error e32) is exact enough unless e32 is large
       if (!(meta[ps] & M_EXACT) && !is_tiny && !(e32[ps] <= 1e-11f)) q_push(sh, queue, ps);
     }
-    __syncthreads();
-    if (tid < nT) { sh.t_rlo[tid] = ~0ull; sh.t_rhi[tid] = 0ull; }
     run_polish();
     for (int ps = tid; ps < NP; ps += NT) {
       if (!(meta[ps] & M_CAND)) continue;
@@ -1222,7 +1378,7 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
       const int c = i >> 2, k = i & 3;
       sh.c_u[c][k] = (k & 1) ? 0u : 0xffffffffu;
       sh.c_x[c][k] = (k & 1) ? 0ull : ~0ull;
-      if (k < 2) sh.c_s[c][k] = k ? 0u : 0xffffffffu;
+      sh.c_s[c][k] = (k & 1) ? 0u : 0xffffffffu;
       if (k == 0) sh.c_cnt[c] = 0;
     }
     if constexpr (DER) {
@@ -1397,17 +1553,19 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
       er_et(ps, &er, &et);
       if (fkey(r - er) <= sh.c_u[c][0] || fkey(r + er) >= sh.c_u[c][1]) {
         meta[ps] |= M_CAND;
-        const double R = rv(ps), E_ = re(ps);
-        atomicMin(&sh.c_x[c][0], dkey(R + E_));
-        atomicMax(&sh.c_x[c][1], dkey(R - E_));
+        float e_;
+        const float lo = r_from(ps, fkey_inv(sh.c_u[c][0]), &e_);
+        atomicMin(&sh.c_s[c][0], fkey(lo + e_));
+        const float hi = r_from(ps, fkey_inv(sh.c_u[c][1]), &e_);
+        atomicMax(&sh.c_s[c][1], fkey(hi - e_));
       }
       const bool lo = fkey(th - et) <= sh.c_u[c][2], hi = fkey(th + et) >= sh.c_u[c][3];
       if (lo || hi) {
         meta[ps] |= M_CANDT;
         if (refine && !tiny_cell(c, r)) {
           float e_;
-          if (lo) { const float s_ = sine_from(ps, c, 0, &e_); atomicMin(&sh.c_s[c][0], fkey(s_ + e_)); }
-          if (hi) { const float s_ = sine_from(ps, c, 1, &e_); atomicMax(&sh.c_s[c][1], fkey(s_ - e_)); }
+          if (lo) { const float s_ = sine_from(ps, c, 0, &e_); atomicMin(&sh.c_s[c][2], fkey(s_ + e_)); }
+          if (hi) { const float s_ = sine_from(ps, c, 1, &e_); atomicMax(&sh.c_s[c][3], fkey(s_ - e_)); }
         }
       }
     }
@@ -1420,16 +1578,19 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
       const bool is_tiny = tiny_cell(c, r);
       bool cand_r = m_ & M_CAND, cand_t = m_ & M_CANDT;
       if (cand_r) {
-        const double R = rv(ps), E_ = re(ps);
-        cand_r = dkey(R - E_) <= sh.c_x[c][0] || dkey(R + E_) >= sh.c_x[c][1];
+        float e_;
+        const float lo = r_from(ps, fkey_inv(sh.c_u[c][0]), &e_);
+        cand_r = fkey(lo - e_) <= sh.c_s[c][0];
+        const float hi = r_from(ps, fkey_inv(sh.c_u[c][1]), &e_);
+        cand_r = cand_r || fkey(hi + e_) >= sh.c_s[c][1];
       }
       if (cand_t && refine && !is_tiny) {
         const float th = unwrap_f(ps);
         float er, et, e_;
         er_et(ps, &er, &et);
         cand_t = false;
-        if (fkey(th - et) <= sh.c_u[c][2]) { const float s_ = sine_from(ps, c, 0, &e_); cand_t = fkey(s_ - e_) <= sh.c_s[c][0]; }
-        if (fkey(th + et) >= sh.c_u[c][3]) { const float s_ = sine_from(ps, c, 1, &e_); cand_t = cand_t || fkey(s_ + e_) >= sh.c_s[c][1]; }
+        if (fkey(th - et) <= sh.c_u[c][2]) { const float s_ = sine_from(ps, c, 0, &e_); cand_t = fkey(s_ - e_) <= sh.c_s[c][2]; }
+        if (fkey(th + et) >= sh.c_u[c][3]) { const float s_ = sine_from(ps, c, 1, &e_); cand_t = cand_t || fkey(s_ + e_) >= sh.c_s[c][3]; }
       }
       meta[ps] = (uint8_t)((m_ & ~(M_CAND | M_CANDT)) | (cand_r ? M_CAND : 0) | (cand_t ? M_CANDT : 0));
       // theta extremes need an FP64 angle; r extremes only if the
@@ -1437,8 +1598,6 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
       const bool need = (cand_t && !sh.full) || ((cand_r || cand_t) && !(e32[ps] <= 1e-11f));
       if (need && !(m_ & M_EXACT) && !is_tiny) q_push(sh, queue, ps);
     }
-    __syncthreads();
-    for (int i = tid; i < sh.ncell * 2; i += NT) sh.c_x[i >> 1][i & 1] = (i & 1) ? 0ull : ~0ull;
     run_polish();
     for (int ps = tid; ps < NP; ps += NT) {
       const uint8_t m_ = meta[ps];

@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(NTB, 1)
 mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ T_, int E,
            icrs_grid g, int tiles_per_block, double* __restrict__ A_out, uint32_t* __restrict__ st_out,
            double* __restrict__ diag_sect, int32_t* __restrict__ diag_cnt, float* __restrict__ diag_pts, int PMAX,
-           int has_plo, int tabcap, int ccap, DerOut dout, const int32_t* __restrict__ items, int n_items) {
+           int has_plo, int tabcap, int ccap, int tcap, DerOut dout, const int32_t* __restrict__ items, int n_items) {
   constexpr int N = NL * NL + 1;
   constexpr int NT = NTB;
   constexpr int NW = NT / 32;
@@ -518,7 +518,10 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
   float* tabf = (float*)pr_;     pr_ += sizeof(cf) * tabcap;        // group offsets (cos d - 1, sin d)
   AnchorF* anch = (AnchorF*)pr_; pr_ += sizeof(AnchorF) * MAXANCH;
   float2* spc = (float2*)pr_;    pr_ += sizeof(float2) * MAXANCH;  // spot centre in each anchor's frame
-  int* wqueue = (int*)pr_;       pr_ += sizeof(int) * NW * DQ;     // boundary points, a queue per warp
+  int* wqueue = (int*)pr_;       pr_ += DER ? sizeof(int) * NW * DQ : sizeof(int2) * NW * FQ;  // boundary points, a queue per warp
+  float* rowp = (float*)pr_;     pr_ += sizeof(float) * 32 * tcap;    // forward: the tasks' terms
+  float* pterm = (float*)pr_;    pr_ += sizeof(float) * PCAP * tcap;
+  int* pcnt = (int*)pr_;         pr_ += sizeof(int) * tcap;
   float* r32 = (float*)p;        p += sizeof(float) * NP;
   float* rl32 = (float*)p;       p += sizeof(float) * NP;   // r = r32 + rl32 (double-float)
   float* t32 = (float*)p;        p += sizeof(float) * NP;
@@ -544,7 +547,7 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
       double* ws = (double*)(sums + NW * DSUM * 32);
       der_sh = {acs, aA, sums, ws, ccap ? (double2*)(ws + 5 * DSUM * TASK_WARPS) : nullptr};
     }
-    rays_sh.P = {anch, spc, tabf, wqueue, tabcap, ccap, g.n_r, g.n_theta, g.uniform, g.ld_split && !g.uniform ? 1 : 0,
+    rays_sh.P = {anch, spc, tabf, wqueue, rowp, pterm, pcnt, DER ? 1 << 30 : tcap, tabcap, ccap, g.n_r, g.n_theta, g.uniform, g.ld_split && !g.uniform ? 1 : 0,
                  diag_cnt ? 1 : 0, 1.0f, (float)g.s_fac, g.grad_rule, g.delta_c};
   }
   for (int k = tid; k < K; k += NT) {
@@ -1870,7 +1873,7 @@ marginal_nll_kernel(const double* __restrict__ A, const double* __restrict__ F, 
 // (forward), about three (derivative, where shared memory is shorter).
 static int mag_tabcap(int NL, bool der) { return (der ? 3 : NL * NL + 1) * (GTH_MAX + 2); }
 
-static size_t mag_smem_bytes(int NL, const icrs_grid& g, int pmax, int has_plo, bool der, int nt, int ccap = 0) {
+static size_t mag_smem_bytes(int NL, const icrs_grid& g, int pmax, int has_plo, bool der, int nt, int ccap, int tcap) {
   const int N = NL * NL + 1;
   const size_t NP = (size_t)g.n_limb * N;
   size_t b = sizeof(cf) * NP * (has_plo ? 2 : 1) + sizeof(cdf) * g.n_limb + 16;
@@ -1879,7 +1882,8 @@ static size_t mag_smem_bytes(int NL, const icrs_grid& g, int pmax, int has_plo, 
   size_t slots = 4 * sizeof(float) * NP + sizeof(short) * ((NP + 7) & ~(size_t)7) + 3 * ((NP + 15) & ~(size_t)15);
   slots += 2 * sizeof(double) * pmax + sizeof(int) * QMAX;
   const size_t rays = sizeof(cf) * mag_tabcap(NL, der) + (sizeof(AnchorF) + sizeof(float2)) * MAXANCH +
-                      sizeof(int) * (nt / 32) * DQ + (der ? der_rays_bytes(nt / 32) : 0) + sizeof(double2) * ccap;
+                      (der ? sizeof(int) * (nt / 32) * DQ + der_rays_bytes(nt / 32) : sizeof(int2) * (nt / 32) * FQ) +
+                      sizeof(double2) * ccap + (size_t)tcap * (sizeof(float) * (32 + PCAP) + sizeof(int));
   return b + (slots > rays ? slots : rays);
 }
 
@@ -1919,7 +1923,7 @@ template <int NL, bool DER, int NTB, int LAW>
 static int launch_nt(const icrs_params* p, int S, const double* t, int E, const icrs_grid* g, double* A,
                      uint32_t* status, double* dsect, int32_t* dcnt, float* dpts, const DerOut& dout,
                      cudaStream_t st, const int32_t* items, int n_items, int nsm, size_t smem, int pmax,
-                     int has_plo, int ccap) {
+                     int has_plo, int ccap, int tcap) {
   if (cudaFuncSetAttribute(mag_kernel<NL, DER, NTB, LAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)
     return ICRS_ECUDA;
@@ -1934,7 +1938,7 @@ static int launch_nt(const icrs_params* p, int S, const double* t, int E, const 
   long long blocks = (tiles + per_block - 1) / per_block;
   mag_kernel<NL, DER, NTB, LAW><<<(unsigned)blocks, NTB, smem, st>>>(p, S, t, E, *g, (int)per_block, A, status,
                                                                       dsect, dcnt, dpts, pmax, has_plo,
-                                                                      mag_tabcap(NL, DER), ccap, dout, items, n_items);
+                                                                      mag_tabcap(NL, DER), ccap, tcap, dout, items, n_items);
   return cudaGetLastError() == cudaSuccess ? ICRS_OK : ICRS_ECUDA;
 }
 
@@ -1954,8 +1958,12 @@ static int launch_inst(const icrs_params* p, int S, const double* t, int E, cons
   // shared memory beside the dynamic part
   cudaFuncAttributes fa;
   if (cudaFuncGetAttributes(&fa, mag_kernel<NL, DER, NT_BASE, LAW>) != cudaSuccess) return ICRS_ECUDA;
+  // forward: the tasks of one sector at least, of as many as fit once the rest
+  // is chosen
+  const int nt1 = DER ? 0 : sector_tasks(g->n_r, g->n_theta);
+  int tcap = nt1;
   auto fits = [&](int pm, int plo) {
-    return mag_smem_bytes(NL, *g, pm, plo, DER, NT_BASE) + fa.sharedSizeBytes <= (size_t)optin;
+    return mag_smem_bytes(NL, *g, pm, plo, DER, NT_BASE, 0, tcap) + fa.sharedSizeBytes <= (size_t)optin;
   };
   int pmax = PMAX_MIN;
   if (!fits(pmax, 0)) return ICRS_EUNSUPPORTED;
@@ -1971,11 +1979,15 @@ static int launch_inst(const icrs_params* p, int S, const double* t, int E, cons
   int ccap = 0;
   if (DER)
     for (int k = NL * NL + 1; k > 0 && !ccap; --k)
-      if (mag_smem_bytes(NL, *g, pmax, has_plo, DER, NT_BASE, k * g->n_theta) + fa.sharedSizeBytes <= (size_t)optin)
+      if (mag_smem_bytes(NL, *g, pmax, has_plo, DER, NT_BASE, k * g->n_theta, 0) + fa.sharedSizeBytes <= (size_t)optin)
         ccap = k * g->n_theta;
-  const size_t smem = mag_smem_bytes(NL, *g, pmax, has_plo, DER, NT_BASE, ccap);
+  for (int k = NL * NL + 1; k > 1 && !DER && tcap == nt1; --k) {
+    tcap = k * nt1;
+    if (!fits(pmax, has_plo)) tcap = nt1;
+  }
+  const size_t smem = mag_smem_bytes(NL, *g, pmax, has_plo, DER, NT_BASE, ccap, tcap);
   return launch_nt<NL, DER, NT_BASE, LAW>(p, S, t, E, g, A, status, dsect, dcnt, dpts, dout, st, items, n_items, nsm,
-                                          smem, pmax, has_plo, ccap);
+                                          smem, pmax, has_plo, ccap, tcap);
 }
 
 // Binary forward: the linear instantiation, then the generic one (each takes

@@ -30,7 +30,9 @@ constexpr int MAXANCH = 128;     // FP64 anchors of a batch of sectors
 constexpr int GTH_MAX = 256;     // columns per theta group (at most)
 constexpr int MAXSEC = 10;       // sectors of an epoch (N_deg of the triple lens)
 constexpr int TASK_WARPS = 16;   // the theta chunks are cut for this many warps
-constexpr int DQ = 32;           // deferred boundary points per warp: one per lane at a flush
+constexpr int DQ = 32;           // deferred boundary points per warp (derivative): one per lane at a flush
+constexpr int FQ = 64;           // the same, forward: flushed 32 at a time
+constexpr int PCAP = 64;         // boundary points per task that keep their place in the sum (forward)
 constexpr int XQ = 8;            // boundary points per warp whose crossing needs FP64
 constexpr float EPS32 = 5.9604645e-8f;  // 2^-24
 constexpr int KB = 8;            // columns per block (even: column pairs load as 16 bytes)
@@ -70,7 +72,7 @@ struct Sec {
   int ch, nch;           // columns per chunk, chunks
   int ntask;
   int sb;                // columns per superblock
-  int spread;            // the order of the tasks, see ray_stage
+  int task0;             // its first task in the batch
   float sag;             // (sb dth)^2 / 8
 };
 
@@ -86,6 +88,18 @@ __device__ __noinline__ cd sec_offset64(const double* eps, const cd* a, cd wc, c
   sincos(th, &s, &c);
   cd z = mk(r * c, r * s);
   return lens_map<NL, double>(eps, a, z) - wc;
+}
+
+// Columns per theta chunk of a sector, and its number of tasks: 32 rows (one
+// per lane) x a chunk of an even number of columns, about 8 tasks per warp.
+__host__ __device__ inline int chunk_columns(int NR, int NTH) {
+  const int nrb = (NR + 31) >> 5, nch = (8 * TASK_WARPS + nrb - 1) / nrb;
+  const int c = 2 * ((NTH + 2 * nch - 1) / (2 * nch));
+  return NTH < 16 ? NTH : (c < 16 ? 16 : (c < NTH ? c : NTH));
+}
+__host__ __device__ inline int sector_tasks(int NR, int NTH) {
+  const int c = chunk_columns(NR, NTH);
+  return ((NR + 31) >> 5) * ((NTH + c - 1) / c);
 }
 
 // Group layout of sector B (one thread).
@@ -117,18 +131,13 @@ __device__ inline void sec_setup(Sec& S, const Box& B, int NR, int NTH) {
   // (here both <= 8192)
   S.gmagic = (unsigned int)((0xFFFFFFFFull / (unsigned long long)S.gth) + 1ull);
   for (int gi = 0; gi < mr; ++gi) S.rc[gi] = (float)(B.r_lo + (gi * S.gr + 0.5 * S.gr) * S.dr64);
-  // tasks of 32 rows (one per lane) x a theta chunk of an even number of
-  // columns, about 8 tasks per warp per sector
-  const int nrb = (NR + 31) >> 5;
-  const int nch = max(1, (8 * TASK_WARPS + nrb - 1) / nrb);
-  S.ch = min(NTH, max(16, 2 * ((NTH + 2 * nch - 1) / (2 * nch))));
+  S.ch = chunk_columns(NR, NTH);
   S.nch = (NTH + S.ch - 1) / S.ch;
-  S.ntask = nrb * S.nch;
+  S.ntask = ((NR + 31) >> 5) * S.nch;
   // A superblock's test costs about two ray evaluations a row, and what it
   // saves grows with the number of superblocks across the image: about 32 of
   // them; none when a chunk holds only two blocks.
   S.sb = S.ch <= 2 * KB ? 0 : (NTH >= 2048 ? 64 : (NTH >= 1024 ? 32 : 16));
-  S.spread = S.sb && nrb >= 2 * TASK_WARPS;
   const float ls = (float)S.sb * S.dth32;
   S.sag = 0.125f * ls * ls;
 }
@@ -339,6 +348,10 @@ struct RayArgs {
   float2* spc;      // spot centre in each anchor's frame
   float* tabf;      // group offsets (cos d - 1, sin d) of the batch's sectors
   int* wqueue;      // boundary points, DQ per warp
+  float* rowp;      // [task][32] the rows' r_i x sum (forward)
+  float* pterm;     // [task][PCAP] the boundary points' terms
+  int* pcnt;        // [task] their number
+  int tcap;         // tasks of a batch
   int tabcap;       // columns that tabf holds
   int ccap;         // columns that the derivative's cosine table holds (0: none)
   int NR, NTH, uniform, split, diag;
@@ -351,8 +364,8 @@ struct RayArgs {
 struct RayShared {
   RayArgs P;
   Sec sec[MAXSEC];
-  int b0, b1, nanch, ncol;
-  int xq[32][XQ];   // boundary points whose crossing needs FP64, per warp
+  int b0, b1, nanch, ncol, ntask, next;
+  int2 xq[TASK_WARPS][XQ];   // boundary points whose crossing needs FP64, per warp
 };
 
 // c + a b in FP32, each operation rounded as written.
@@ -556,11 +569,12 @@ __device__ __forceinline__ void kahan_add(float2& acc, float term) {
   acc.x = tt;
 }
 
-// The product a b added with its rounding error (two-sum and two-product).
-__device__ __forceinline__ void sum_add(float2& acc, float a, float b) {
-  const df p = two_prod(a, b), t = two_sum(acc.x, p.hi);
-  acc.x = t.hi;
-  acc.y -= t.lo + p.lo;
+// The product a b, rounded with the compensation in one operation.
+__device__ __forceinline__ void kahan_add(float2& acc, float a, float b) {
+  const float y = __fmaf_rn(a, b, -acc.y);
+  const float tt = __fadd_rn(acc.x, y);
+  acc.y = __fsub_rn(__fsub_rn(tt, acc.x), y);
+  acc.x = tt;
 }
 
 // The weight W of a boundary point (Appendix A) from the signed squared
@@ -651,12 +665,13 @@ template <int NL, int LAW, class SH>
 __device__ __noinline__ float2 flush_exact(SH& sh, RayShared& rs, int n, float2 acc) {
   const RayArgs& P = rs.P;
   const int lane = threadIdx.x & 31;
-  const int* xq = rs.xq[threadIdx.x >> 5];
+  const int2* xq = rs.xq[threadIdx.x >> 5];
   __syncwarp();
   for (int e0 = 0; e0 < n; e0 += 4) {
     const int e = e0 + (lane >> 3), k = lane & 7;
     const bool has = e < n;
-    const int v = has ? xq[e] : 0;
+    const int2 v2 = has ? xq[e] : make_int2(0, -1);
+    const int v = v2.x;
     const Sec& S = rs.sec[v >> 25];
     const int irow = (v >> 13) & 4095, m = v & 8191;
     const int gi_ = irow / S.gr;
@@ -685,7 +700,9 @@ __device__ __noinline__ float2 flush_exact(SH& sh, RayShared& rs, int n, float2 
       float W, WU;
       (void)boundary_weight(sh, P, sv, dist, &W, &WU);
       if (P.diag) atomicAdd(&sh.cnt[3], 1);
-      kahan_add(acc, point_term<LAW>(sh, P, S, ri_, -sv[2], fsc, W, WU));
+      const float term = point_term<LAW>(sh, P, S, ri_, -sv[2], fsc, W, WU);
+      if (v2.y >= 0) P.pterm[v2.y] = term;
+      else kahan_add(acc, term);
     }
   }
   __syncwarp();
@@ -693,16 +710,20 @@ __device__ __noinline__ float2 flush_exact(SH& sh, RayShared& rs, int n, float2 
 }
 
 // n <= 32 queued points q, one per lane: each re-evaluates its stencil (rays m
-// - 2 .. m + 2, signed squared distances, negative inside) and adds its term.
-// Points that need FP64 go to the warp's second queue (*xn entries).
+// - 2 .. m + 2, signed squared distances, negative inside) and writes its term
+// to its place (the point's second word; -1: its task has no more, the term is
+// added here).  Points that need FP64 go to the warp's second queue (*xn
+// entries).
 template <int NL, int LAW, class SH>
-__device__ __noinline__ float2 flush_points(SH& sh, RayShared& rs, const int* q, int n, int* xn, float2 acc) {
+__device__ __noinline__ float2 flush_points(SH& sh, RayShared& rs, const int2* q, int n, int* xn, float2 acc) {
   const int lane = threadIdx.x & 31;
   __syncwarp();
   bool exact = false;
-  int v = 0;
+  int2 v2 = make_int2(0, -1);
   if (lane < n) {
-    v = q[lane];
+    v2 = q[lane];
+    const int v = v2.x;
+    float term = 0.f;
     const Sec& S = rs.sec[v >> 25];
     const int irow = (v >> 13) & 4095, m = v & 8191;
     const int gi_ = irow / S.gr;
@@ -719,17 +740,17 @@ __device__ __noinline__ float2 flush_points(SH& sh, RayShared& rs, const int* q,
     }
     if (signbit(sv[2])) {
       float W, WU;
-      if (boundary_weight(sh, rs.P, sv, nullptr, &W, &WU))
-        kahan_add(acc, point_term<LAW>(sh, rs.P, S, ri_, -sv[2], fsc, W, WU));
-      else
-        exact = true;
+      if (boundary_weight(sh, rs.P, sv, nullptr, &W, &WU)) term = point_term<LAW>(sh, rs.P, S, ri_, -sv[2], fsc, W, WU);
+      else exact = true;
     }
+    if (v2.y >= 0) rs.P.pterm[v2.y] = term;
+    else if (!exact) kahan_add(acc, term);
   }
   unsigned todo = __ballot_sync(0xffffffffu, exact);
   while (todo) {
     if (*xn == XQ) { acc = flush_exact<NL, LAW>(sh, rs, XQ, acc); *xn = 0; }
     const int src = __ffs(todo) - 1;
-    if (lane == src) rs.xq[threadIdx.x >> 5][*xn] = v;
+    if (lane == src) rs.xq[threadIdx.x >> 5][*xn] = v2;
     ++*xn;
     todo &= todo - 1u;
   }
@@ -752,17 +773,17 @@ __device__ __noinline__ void ray_tables(SH& sh, RayShared& rs, const DR& dr) {
   const bool spot = LAW != 0 && sh.spot;
   const int nbox = sh.nbox;
   if (tid == 0) {
-    int b = rs.b1, na = 0, nc = 0;
+    int b = rs.b1, na = 0, nc = 0, nt = 0;
     rs.b0 = b;
     for (; b < nbox; ++b) {
       Sec& S = rs.sec[b];
       if (b > rs.b0 && (na + S.nanch > MAXANCH || nc + S.gth + 2 > P.tabcap ||
-                        (P.ccap && (b - rs.b0 + 1) * P.NTH > P.ccap)))
+                        nt + S.ntask > P.tcap || (P.ccap && (b - rs.b0 + 1) * P.NTH > P.ccap)))
         break;
-      S.abase = na; S.tbase = nc; S.cbase = (b - rs.b0) * P.NTH;
-      na += S.nanch; nc += S.gth + 2;
+      S.abase = na; S.tbase = nc; S.cbase = (b - rs.b0) * P.NTH; S.task0 = nt;
+      na += S.nanch; nc += S.gth + 2; nt += S.ntask;
     }
-    rs.b1 = b; rs.nanch = na; rs.ncol = nc;
+    rs.b1 = b; rs.nanch = na; rs.ncol = nc; rs.ntask = nt; rs.next = 0;
   }
   __syncthreads();
   const int b0 = rs.b0, b1 = rs.b1;
@@ -811,7 +832,7 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
   const unsigned lt_mask = (1u << lane) - 1u;
   const AnchorF* const anf = P.anch;
   const float* const tabf = P.tabf;
-  int* const dq = P.wqueue + warp * DQ;
+  int2* const dq = reinterpret_cast<int2*>(P.wqueue) + warp * FQ;
   int dq_n = 0, xq_n = 0;
   const int nbox = sh.nbox;
 
@@ -872,22 +893,22 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
     const int b0 = rs.b0, b1 = rs.b1;
     if (b0 >= b1) break;
 
-    // ---- tasks, in a static order (warp, warp + NW, ...): the same sums in
-    // the same order on every run.  Row block by row block, which gives the
-    // chunks of a row block to neighbouring warps; where that leaves a warp
-    // only chunks at one angle (32 row blocks and more: 4 chunks or fewer,
-    // those at the sector's edges mostly skipped), row blocks change fastest,
-    // shifted from chunk to chunk (1024 x 2048: 55.6 against 59.2 ms for 6400
-    // epochs; at 512 x 1024 the other way round, 29.3 against 27.4).  There
-    // the rows' terms are added with their rounding errors, since a plain
-    // compensated sum in another order rounds each term differently.
-    for (int b = b0; b < b1; ++b) {
-    const Sec& S = rs.sec[b];
-    for (int tk = warp; tk < S.ntask; tk += NW) {
-      const int nrb = (NR + 31) >> 5;
-      int rbk, chk;
-      if (S.spread) { chk = tk / nrb; rbk = (tk - chk * nrb + 5 * chk) % nrb; }
-      else { rbk = tk / S.nch; chk = tk - rbk * S.nch; }
+    // ---- tasks.  A warp takes the next one when it is free: with superblocks
+    // their costs differ by what is skipped (handed out in a fixed order, a
+    // third of a 1024 x 2048 epoch's ray time was waiting for the last warp).
+    // The sums do not depend on who computed what: a task leaves its rows' and
+    // its boundary points' terms in shared memory, and they are added
+    // afterwards in a fixed order.
+    int b = b0;
+    for (;;) {
+      int task = 0;
+      if (lane == 0) task = atomicAdd(&rs.next, 1);
+      task = __shfl_sync(0xffffffffu, task, 0);
+      if (task >= rs.ntask) break;
+      while (b + 1 < b1 && task >= rs.sec[b + 1].task0) ++b;
+      const Sec& S = rs.sec[b];
+      const int rbk = (task - S.task0) / S.nch, chk = task - S.task0 - rbk * S.nch;
+      int npt = 0;  // boundary points so far
       const int i = rbk * 32 + lane;
       const bool rowok = i < NR;
       const int ii = rowok ? i : NR - 1;
@@ -924,18 +945,12 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
           const bool has = bm != 0u;
           const int m = base - (has ? __ffs(bm) - 1 : 0);
           bm &= bm - 1u;
-          unsigned rem = __ballot_sync(0xffffffffu, has);
-          // up to 32 points: the lowest lanes that fit, a flush whenever the
-          // queue is full, then the rest
-          while (rem) {
-            if (dq_n == DQ) { acc = flush_points<NL, LAW>(sh, rs, dq, DQ, &xq_n, acc); dq_n = 0; }
-            const int at = dq_n + __popc(rem & lt_mask);
-            const bool take = ((rem >> lane) & 1u) && at < DQ;
-            if (take) dq[at] = pack_point(b, i, m);
-            const unsigned tk = __ballot_sync(0xffffffffu, take);
-            dq_n += __popc(tk);
-            rem &= ~tk;
-          }
+          if (dq_n > FQ - 32) { dq_n -= 32; acc = flush_points<NL, LAW>(sh, rs, dq + dq_n, 32, &xq_n, acc); }
+          const unsigned hm = __ballot_sync(0xffffffffu, has);
+          const int at = __popc(hm & lt_mask), seq = npt + at;
+          if (has) dq[dq_n + at] = make_int2(pack_point(b, i, m), seq < PCAP ? task * PCAP + seq : -1);
+          dq_n += __popc(hm);
+          npt += __popc(hm);
         }
       };
       // boundary centres among columns l0 - 1 .. l0 + nb - 2 (bit j = column
@@ -1130,18 +1145,42 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
       // right halo column c1: finalizes column c1 - 1
       win = (win << 1) | halo_flag<NL, LAW>(sh, rs, b, gi, ri, dri, ii, c1);
       push_bits(rowok ? (((win & ~((win << 1) & (win >> 1))) >> 1) & 1u) : 0u, c1 - 1);
-      if (rowok) {
-        const float rowacc = c0f * (float)cnt + (sj + (sj2.x + sj2.y));
-        if (S.spread) sum_add(acc, ri * rowacc, S.bxw);
-        else kahan_add(acc, ri * rowacc * S.bxw);
-      }
+      const float rowacc = c0f * (float)cnt + (sj + (sj2.x + sj2.y));
+      P.rowp[task * 32 + lane] = ri * rowacc;
+      if (lane == 0) P.pcnt[task] = min(npt, PCAP);
     }
+    if (dq_n > 32) { dq_n -= 32; acc = flush_points<NL, LAW>(sh, rs, dq + dq_n, 32, &xq_n, acc); }
     if (dq_n) acc = flush_points<NL, LAW>(sh, rs, dq, dq_n, &xq_n, acc);
     dq_n = 0;
-    }
     if (xq_n) acc = flush_exact<NL, LAW>(sh, rs, xq_n, acc);
     xq_n = 0;
     __syncthreads();
+
+    // ---- the sums, as a fixed assignment of the tasks would take them: thread
+    // (warp, lane) adds the rows of tasks warp, warp + NW, ... of each sector,
+    // and of these tasks' boundary points, 32 to a batch, its lane's, a batch
+    // when the first point after it comes (a compensated sum rounds each term
+    // together with what it carries, so its order shows in the tenth digit)
+    for (int bb = b0; bb < b1; ++bb) {
+      const Sec& S = rs.sec[bb];
+      int n = 0, q = lane;         // points so far, this lane's next
+      int pt_ = warp, base = 0;    // the task that holds it, its first point
+      auto add_points = [&](int upto) {  // q while q < upto
+        while (q < upto) {
+          int c = P.pcnt[S.task0 + pt_];
+          while (q >= base + c) { base += c; pt_ += NW; c = P.pcnt[S.task0 + pt_]; }
+          kahan_add(acc, P.pterm[(S.task0 + pt_) * PCAP + q - base]);
+          q += 32;
+        }
+      };
+      for (int tk = warp; tk < S.ntask; tk += NW) {
+        n += P.pcnt[S.task0 + tk];
+        // whole batches that a later point has pushed out
+        if (n > 32) add_points((n - 1) & ~31);
+        if ((tk / S.nch) * 32 + lane < NR) kahan_add(acc, P.rowp[(S.task0 + tk) * 32 + lane], S.bxw);
+      }
+      add_points(n);
+    }
   }
   return (double)acc.x - (double)acc.y;
 }

@@ -1790,7 +1790,8 @@ __global__ void point_source_kernel(const icrs_params* __restrict__ P, int S, co
   long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)S * n) return;
   const int s = (int)(idx / n);
-  const Lens L = make_lens(P[s]);
+  PsLens<NL> L;
+  ps_lens<NL>(make_lens(P[s]), L);
   const cd w = mk(W[2 * idx], W[2 * idx + 1]);
   const PointSource<NL> r = point_source_solve<NL>(L, w, g.max_iter, g.img_tol, images ? images + idx * N * 2 : nullptr);
   A[idx] = r.A;

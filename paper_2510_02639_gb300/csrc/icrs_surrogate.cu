@@ -597,7 +597,8 @@ __global__ void features_kernel(const icrs_params* __restrict__ P, int S, const 
   if (idx >= (long long)S * E) return;
   const int s = (int)(idx / E);
   const icrs_params prm = P[s];
-  const Lens L = make_lens(prm);
+  PsLens<2> L;
+  ps_lens<2>(make_lens(prm), L);
   const cd w = source_centre(prm, T[idx]);
   PointSource<2> ps = point_source_solve<2>(L, w, g.max_iter, g.img_tol, nullptr);
   // 32 source-limb points: a caustic inside the disk changes the image count

@@ -128,13 +128,15 @@ __device__ __forceinline__ void load_input_row(const float* __restrict__ feat, i
 // SiLU z / (1 + e^-z), the division written out: the reciprocal's
 // approximation, one correction of the quotient by its exact remainder (the
 // usual correctly rounded division without its range handling: d >= 1; d = inf
-// gives 0, where the plain division gives -0).
+// gives 0, where the plain division gives -0; a NaN stays one).  Paired
+// operations around the two exponentials are slower: 356 us against 341 for
+// 2^20 queries.
 __device__ __forceinline__ float silu_fast(float z) {
   const float d = 1.0f + expf(-z);
   const float r = rcp_fast(d);
   const float q = z * r;
   const float y = fmaf(fmaf(-q, d, z), r, q);
-  return d < 1e37f ? y : 0.0f;
+  return d >= 1e37f ? 0.0f : y;
 }
 
 // ---------------------------------------------------------------- inference
@@ -146,10 +148,11 @@ __device__ __forceinline__ float silu_fast(float z) {
 // row read half a row each from TMEM, add the bias, apply SiLU and write the
 // next layer's BF16 operand.
 //
-// The SiLU bounds it: 512 a query, each with two special-function operations
-// (16 a cycle and SM): 0.22 ms for 2^20 queries, against 0.056 ms for the
-// contractions.  One group of 128 threads took 2.14 ms: one warp per scheduler,
-// latency after latency.  Three groups fill shared memory (212 KB).
+// The SiLU bounds it: 512 a query, 18 instructions each with the bias, the
+// rounding and the store: issue slots 79 % busy, special functions 34 %, tensor
+// cores 14 % (0.056 ms of 2^20 queries' contractions).  One group of 128
+// threads took 2.14 ms for 2^20 queries: one warp per scheduler, latency after
+// latency; three groups, which fill shared memory (212 KB), 0.34.
 constexpr int INF_GROUPS = 3, INF_GT = 256, INF_NT = INF_GROUPS * INF_GT;
 constexpr int INF_X = H * H * 2;  // bytes of a group's operand tile (X_0 takes its head)
 constexpr int INF_SMEM = PB_FWD + INF_GROUPS * INF_X;
@@ -252,7 +255,7 @@ mlp_infer_kernel(const uint8_t* __restrict__ pack, const float* __restrict__ the
 // transposed copies); the bias gradients are contractions with a tile of ones;
 // the next weights arrive by bulk copies meanwhile.  128 threads with
 // transposed 2-byte stores, activations through the workspace and weights
-// copied by hand took 185 us of a 245 us step.
+// copied by hand took 185 us of a 245 us step; the step takes 84 us now.
 constexpr int TR_NT = 512;
 constexpr int XB = H * H * 2, XB0 = H * KIN * 2;          // bytes of a [128][128] and a [128][16] tile
 constexpr size_t WS_Z = (size_t)4 * TM * H * 4;           // Z_l  [4][8][512] float4
@@ -580,6 +583,10 @@ constexpr int NLIMB_SG = 32;  // source-limb points of the feature kernel
 constexpr int FEAT_THREADS = 128;  // threads (epochs) per feature block
 static_assert((NLIMB_SG & (NLIMB_SG - 1)) == 0, "the harmonic index wraps with a mask");
 
+// Bounded by FP64 throughput (a warp's FP64 instruction occupies the SM for 16
+// cycles): 33 solves an epoch, each about 60 FP64 operations a Newton step and
+// root, see ps_polish_validate for the figures.  Blocks of 32 threads instead
+// of 128 take the same time.
 __global__ void features_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ T, int E,
                                 icrs_grid g, float* __restrict__ feat, double* __restrict__ A_ps,
                                 uint32_t* __restrict__ status) {

@@ -105,6 +105,21 @@ def test_infer_row_tiles(G, n):
     assert np.all(ratio <= 1.0), (np.argwhere(ratio > 1.0)[:5], ratio.max())
 
 
+def test_infer_non_finite_features(G):
+    """A query with a NaN or an infinite feature comes back NaN, the others of
+    its tile untouched."""
+    import torch
+    f = rand_features(300, 16)
+    tt = torch.tensor(theta_for_test(17), device="cuda")
+    pack = G.mlp_pack(tt)
+    ref = G.mlp_infer(pack, tt, torch.tensor(f, device="cuda")).cpu().numpy()
+    f[5, 0], f[130, 6], f[299, 3] = np.nan, np.inf, -np.inf
+    out = G.mlp_infer(pack, tt, torch.tensor(f, device="cuda")).cpu().numpy()
+    bad = np.zeros(300, dtype=bool)
+    bad[[5, 130, 299]] = True
+    assert np.all(np.isnan(out[bad])) and np.array_equal(out[~bad], ref[~bad])
+
+
 @pytest.mark.parametrize("n", [127, 128, 129, 152 * 128 + 1])
 def test_train_row_tiles(G, n):
     """Gradient and loss, and the weights repacked by the same step."""

@@ -44,7 +44,6 @@ namespace icrs {
 // registers for independent column pairs pay more than further warps.
 constexpr int NT_BASE = 512;
 constexpr int NW_MAX = NT_BASE / 32;  // warps per block
-constexpr int NW_DER = NT_BASE / 32;
 static_assert(TASK_WARPS == NW_MAX, "the ray stage's chunks are cut for this many warps");
 constexpr int QMAX = 2048;       // work queue
 constexpr int PMAX_MIN = 512;    // FP64-polished image-limb points per epoch (at least)
@@ -493,7 +492,7 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
   constexpr int N = NL * NL + 1;
   constexpr int NT = NTB;
   constexpr int NW = NT / 32;
-  static_assert(NT % 32 == 0 && NW <= NW_MAX && (!DER || NW == NW_DER), "per-warp tables are sized for these block sizes");
+  static_assert(NT % 32 == 0 && NW <= NW_MAX && (!DER || NW == NW_MAX), "per-warp tables are sized for these block sizes");
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ Shared sh;
   __shared__ RayShared rays_sh;
@@ -1054,7 +1053,11 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     {
       const int qn = min(sh.qn, QMAX);
       // a few points: one per warp; more: as many as a warp has lanes for;
-      // beyond one round of those: one per thread
+      // beyond one round of those: one per thread, since a warp's FP64
+      // instruction occupies the SM for 16 cycles however many lanes are
+      // active (64 sets, always by warps: 32,000 epochs at 64 x 256 55.5 ms
+      // against 48.4; always by threads: 6,400 at 512 x 1024 27.5 against 26.9,
+      // and one epoch alone waits up to 400k cycles)
       const int np = qn <= NW ? 1 : 32 / N;
       if (qn <= NW * (32 / N)) {
         for (int qi = warp * np; qi < qn; qi += NW * np) {

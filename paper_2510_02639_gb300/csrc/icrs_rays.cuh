@@ -12,10 +12,16 @@
 // A warp takes a task of 32 rows (lane = row) and a chunk of theta columns.
 // Columns are taken in superblocks: the source-plane offsets of a row at a
 // superblock's two ends bound the offsets between them (chord plus sagitta, see
-// AnchorF::out2), so a superblock that lies outside the source on all 32 rows
+// AnchorF::rout), so a superblock that lies outside the source on all 32 rows
 // is skipped and one that lies inside on all rows needs no per-ray decisions.
 // What is skipped would have added exactly zero and what is summed is summed
 // in the same order as without the test, so the results are the same bits.
+//
+// Bounded by the FP32 pipes and the latency of a ray's chain at fine grids (FMA
+// pipe 54 % busy at 1024 x 2048, nine tenths of an epoch's time) and by the
+// FP64 chains of the other phases at coarse ones.  The magnification kernel,
+// 64 sets: 8,000 epochs at 1024 x 2048 341 ms before and 227 with this stage;
+// 32,000 at 64 x 256 72 ms and 48 (with the binning and re-solve phases).
 #pragma once
 
 #include "icrs_common.cuh"
@@ -79,7 +85,7 @@ struct Sec {
 // A boundary point: sector of the batch (4 bits), row (12), column (13).
 __device__ __forceinline__ int pack_point(int b, int row, int col) { return (b << 25) | (row << 13) | col; }
 
-// FP64 fallback of a ray, see ray_offset64 (icrs_mag.cu).
+// Offset of ray (i, l) from the source centre in FP64.
 template <int NL>
 __device__ __noinline__ cd sec_offset64(const double* eps, const cd* a, cd wc, const Sec& S, int i, int l) {
   double r = S.r_lo + (i + 0.5) * S.dr64;
@@ -136,7 +142,9 @@ __device__ inline void sec_setup(Sec& S, const Box& B, int NR, int NTH) {
   S.ntask = ((NR + 31) >> 5) * S.nch;
   // A superblock's test costs about two ray evaluations a row, and what it
   // saves grows with the number of superblocks across the image: about 32 of
-  // them; none when a chunk holds only two blocks.
+  // them; none when a chunk holds only two blocks.  (64 sets, without and with
+  // 16, 32, 64 columns: 12,800 epochs at 256 x 1024 44.6 and 41.8, 40.4, 40.5 ms;
+  // 6,400 at 1024 x 2048 80.2 and 60.6, 55.2, 53.5 ms.)
   S.sb = S.ch <= 2 * KB ? 0 : (NTH >= 2048 ? 64 : (NTH >= 1024 ? 32 : 16));
   const float ls = (float)S.sb * S.dth32;
   S.sag = 0.125f * ls * ls;
@@ -1073,26 +1081,25 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
               }
               win = 0xffffffffu;
               cnt += ls - l;
-              auto in_block = [&](auto hh) {
+              // binary: blocks of columns in pairs.  (The triple lens takes one
+              // column at a time: its evaluation is twice as long, and with an
+              // unrolled block the fetches held up the warps.  A curve of 2,000
+              // epochs at 1024 x 2048: 108 ms unrolled, 76 now.)
+              if constexpr (NL == 2) {
+                auto in_block = [&](auto hh) {
 #pragma unroll
-                for (int k = 0; k < KB; k += 2) {
-                  const float4 t4 = *reinterpret_cast<const float4*>(tpf + 2 * (l + k));
-                  if constexpr (NL == 2) {
+                  for (int k = 0; k < KB; k += 2) {
+                    const float4 t4 = *reinterpret_cast<const float4*>(tpf + 2 * (l + k));
                     const float2 J = share2(
                         ray_eval2(ap, make_float2(t4.x, t4.y), make_float2(t4.z, t4.w), ri2, nri2, dri2), hh);
                     sj2 = __ffma2_rn(J, one_rt, sj2);  // a sum: see one_rt
-                  } else {
-                    const float x0 = __fmaf_rn(-ray_eval<NL>(ar, t4.x, t4.z, ri, dri, nullptr, nullptr), irho2, 1.0f);
-                    const float x1 = __fmaf_rn(-ray_eval<NL>(ar, t4.y, t4.w, ri, dri, nullptr, nullptr), irho2, 1.0f);
-                    add_in(true, __fmul_rn(x0, rsqrt_fast(x0)), generic && sh.half != 0, 1.0f);
-                    add_in(true, __fmul_rn(x1, rsqrt_fast(x1)), generic && sh.half != 0, 1.0f);
                   }
-                }
-              };
+                };
 #pragma unroll 1
-              for (; l + KB <= ls; l += KB) {
-                if (LAW == 1 && NL == 2 && generic) in_block(std::true_type{});
-                else in_block(std::false_type{});
+                for (; l + KB <= ls; l += KB) {
+                  if (LAW == 1 && generic) in_block(std::true_type{});
+                  else in_block(std::false_type{});
+                }
               }
 #pragma unroll 1
               for (; l < ls; ++l) {

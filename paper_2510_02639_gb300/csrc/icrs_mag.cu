@@ -79,6 +79,7 @@ struct Shared {
   // its u1 derivative over itself times c F_spot' ... (see the chain);
   // spot_new: the set changed and has a spot; generic: half or spot
   double spot_x, spot_y, spot_r, spot_c, spot_norm, spot_gu, spot_acc[2];
+  float spot_rr32, spot_f32;  // its radius, and 1 - contrast
   int spot, spot_bad, spot_new, generic;
   float eps32[3];
   cf aj32[3][3];       // [frame j][lens i]: a_i - a_j (FP32)
@@ -607,6 +608,8 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
         sh.spot = prm.spot_c != 0.0;
         sh.generic = sh.half || sh.spot;
         sh.spot_x = prm.spot_x; sh.spot_y = prm.spot_y; sh.spot_r = prm.spot_r; sh.spot_c = prm.spot_c;
+        sh.spot_rr32 = (float)(sh.rho * prm.spot_r);
+        sh.spot_f32 = (float)(1.0 - prm.spot_c);
         sh.spot_bad = sh.spot && !(prm.spot_r >= 0.0 && prm.spot_c < 1.0 &&
                                    hypot(prm.spot_x, prm.spot_y) + prm.spot_r <= 1.0);
         sh.spot_new = sh.spot && !sh.spot_bad;

@@ -497,6 +497,7 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
         float4 A01 = make_float4(0.f, 0.f, 0.f, 0.f);
         float2 cs = make_float2(1.f, 0.f);
         int gbase = 0;
+        SpotBand spb;
         auto push_bits = [&](unsigned bm, int base) {
           while (__any_sync(0xffffffffu, bm != 0u)) {
             const bool has = bm != 0u;
@@ -524,8 +525,7 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
         // ray of the warp's column is known to be inside.
         auto colD = [&](int l, const cf t, bool& unc, auto hc, auto sure) {
           cf dz, dw;
-          float eb = 0.f;
-          const float d2 = ray_eval<2>(ar, t.x, t.y, ri, dri, decltype(hc)::value ? &eb : nullptr, &dw, &dz);
+          const float d2 = ray_eval<2>(ar, t.x, t.y, ri, dri, nullptr, &dw, &dz);
           bool in = true, u_ = false;
           if constexpr (!decltype(sure)::value) {
             in = d2 < ar.lo2;
@@ -535,7 +535,8 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
           }
           if (!u_) {
             float fs = 1.f;
-            if constexpr (decltype(hc)::value) fs = in ? spot_factor<2, 2>(sh, rs, S, aidx, dw, eb, ii, l) : 1.f;
+            if constexpr (decltype(hc)::value)
+              fs = in && spot ? spot_sweep<2, 2>(sh, rs, S, aidx, spb, dw, t.x, t.y, ri, dri, ii, l) : 1.f;
             const float a = seed_of(w, in, d2, pg, rowacc, hc, fs);
             if (a != 0.f) grad_core(w, dz, dw, t.x, t.y, ri, (float)l + 0.5f, A01, cs, a, pg);
           }
@@ -548,6 +549,7 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
           ar = anf[aidx];
           A01 = dr.aA[aidx];
           cs = dr.acs[aidx];
+          if (spot) spb = spot_band(sh, rs, ar, aidx);
           gbase = mgrp * gth;
           const int lend = min(gbase + gth, c1);
           const bool test = __any_sync(0xffffffffu, sb && ar.rout < __int_as_float(0x7f800000));

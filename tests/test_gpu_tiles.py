@@ -39,13 +39,17 @@ def test_forward_grids(G, oracle_mod, n_r, n_theta, n_limb):
     assert_status(st, so, what=str((n_r, n_theta)))
 
 
-@pytest.mark.parametrize("law", ["quadratic", "powers", "spot", "uniform", "triple"])
+@pytest.mark.parametrize("law", ["quadratic", "powers", "spot", "uniform", "triple", "triple spot"])
 def test_forward_laws_on_ragged_superblocks(G, oracle_mod, law):
     """Every instantiation of the sweep on a grid with superblocks and
     remainders (97 x 1029)."""
-    if law == "triple":
+    n_limb = 200
+    if law.startswith("triple"):
         params, t = I.triple_curve()
         t = t[:, 700:1300:120]
+        if law == "triple spot":
+            n_limb = 580  # the largest that fits
+            params = [dict(params[0], spot_x=0.3, spot_y=-0.2, spot_r=0.4, spot_c=0.7)]
     else:
         params, t = I.caustic_crossing_binary(n_epochs=500)
         t = t[:, 40:470:100]
@@ -55,7 +59,7 @@ def test_forward_laws_on_ragged_superblocks(G, oracle_mod, law):
             params = [dict(params[0], a1=0.3, a2=0.2, a3=-0.1, a4=0.05)]
         elif law == "spot":
             params = [dict(params[0], spot_x=0.3, spot_y=-0.2, spot_r=0.4, spot_c=0.7)]
-    g = I.grid(n_r=97, n_theta=1029, n_limb=200, uniform=1 if law == "uniform" else 0)
+    g = I.grid(n_r=97, n_theta=1029, n_limb=n_limb, uniform=1 if law == "uniform" else 0)
     A, st = run_gpu(G, params, t, g)
     Ao, so = oracle_mod.magnification(params, t, g)
     assert_parity(A, Ao, what=law)

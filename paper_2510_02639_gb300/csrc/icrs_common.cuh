@@ -323,36 +323,49 @@ __device__ inline int ehrlich_aberth_f32(const cf* b, cf* z, int max_iter, float
   return -1;
 }
 
+// The rounding part of the FP64 iteration's stopping test: whether the step dz
+// from z is at most twice the FP64 rounding level u sum_l |b_l| |z|^l / |P'| of
+// P at the root (ab: |b_l|; dp: P').  Compared as squares, which leaves one
+// square root; in FP64, since the coefficients of a wide lens or of a far
+// source leave FP32's range, and an infinite level would accept any step.
+template <int N>
+__device__ __forceinline__ bool ea64_at_rounding(const double* ab, cd z, cd dz, cd dp) {
+  const double az = sqrt(abs2(z));
+  double pa = ab[N];
+#pragma unroll
+  for (int l = N - 1; l >= 0; --l) pa = fma(pa, az, ab[l]);
+  const double t = 2.220446049250313e-16 * pa, t2 = t * t;
+  return t2 <= 1.7976931348623157e308 && abs2(dz) * abs2(dp) <= t2;
+}
+// The other part, with z after the step: at most 1e-14 max(1, |z|).
+__device__ __forceinline__ bool ea64_small(cd z, cd dz) { return abs2(dz) <= 1e-28 * fmax(1.0, abs2(z)); }
+
 // Ehrlich-Aberth iteration in FP64 (Sec. 3.1): the fallback for positions
 // whose FP32 roots do not give a trustworthy image set (clusters of close
 // roots next to a critical curve, which FP32 cannot separate).  Stops when every step is
-// below 1e-14 max(1, |z|) or twice the FP64 rounding level of P at the root
-// (the test's moduli are taken in FP32: they are only compared).
+// below 1e-14 max(1, |z|) or twice the FP64 rounding level of P at the root.
 template <int N>
 __device__ inline int ehrlich_aberth_f64(const cd* b, cd* z, int max_iter) {
-  float ab[N + 1];
-  for (int l = 0; l <= N; ++l) ab[l] = sqrtf((float)abs2(b[l]));
+  double ab[N + 1];
+  for (int l = 0; l <= N; ++l) ab[l] = sqrt(abs2(b[l]));
   for (int it = 0; it < max_iter; ++it) {
     cd dz[N];
-    float noise[N];
+    bool rnd[N];
     bool done = true;
     for (int k = 0; k < N; ++k) {
       cd p, dp;
       horner2<N, double>(b, z[k], p, dp);
-      float az = sqrtf((float)abs2(z[k])), pa = ab[N];
-      for (int l = N - 1; l >= 0; --l) pa = fmaf(pa, az, ab[l]);
-      noise[k] = 1.1102230246251565e-16f * pa / fmaxf(sqrtf((float)abs2(dp)), 1e-30f);
       cd W = dv(p, dp);
       cd S = mk(0.0, 0.0);
       for (int j = 0; j < N; ++j)
         if (j != k) S = S + inv(z[k] - z[j]);
       dz[k] = dv(W, mk(1.0, 0.0) - W * S);
       if (!(abs2(p) > 0.0)) dz[k] = mk(0.0, 0.0);
+      rnd[k] = ea64_at_rounding<N>(ab, z[k], dz[k], dp);
     }
     for (int k = 0; k < N; ++k) {
       z[k] = z[k] - dz[k];
-      const float st = sqrtf((float)abs2(dz[k]));
-      if (!(st <= fmaxf(1e-14f * fmaxf(1.0f, sqrtf((float)abs2(z[k]))), 2.0f * noise[k]))) done = false;
+      if (!(rnd[k] || ea64_small(z[k], dz[k]))) done = false;
     }
     if (done) return it + 1;
   }

@@ -287,9 +287,8 @@ __device__ inline void point_tangents(const Shared& sh, const DerShared& ds, dou
 // FP64 Ehrlich-Aberth by one warp, root j of limb point g on lane g N + j (np
 // points): the same iteration, operation by operation, as one thread's over
 // all roots.  With one point the differences 1 / (z_k - z_j) are spread over
-// the lanes besides.  Only the stopping test's moduli are taken in FP32: it
-// compares steps with a rounding level.  b: this lane's point's polynomial.
-// Returns whether this lane's point converged.
+// the lanes besides.  b: this lane's point's polynomial.  Returns whether this
+// lane's point converged.
 template <int N>
 __device__ inline bool ehrlich_aberth_f64_warp(const cd* b, cd* zj, int np, int max_iter) {
   constexpr int NP2 = N * (N - 1), R = (NP2 + 31) / 32;
@@ -297,9 +296,17 @@ __device__ inline bool ehrlich_aberth_f64_warp(const cd* b, cd* zj, int np, int 
   const bool act = lane < np * N;
   const int g = act ? lane / N : 0, k = act ? lane - g * N : 0;
   const unsigned mine = ((1u << N) - 1u) << (g * N);  // the lanes of this point
-  float ab[N + 1];
+  // |b_l| of the lane's point: lane k of the point forms |b_k|, all form |b_N|
+  double ab[N + 1];
+  {
+    cd bk = b[0];
 #pragma unroll
-  for (int l = 0; l <= N; ++l) ab[l] = sqrtf((float)abs2(b[l]));
+    for (int l = 1; l < N; ++l) if (k == l) bk = b[l];
+    const double m = sqrt(abs2(bk));
+#pragma unroll
+    for (int l = 0; l < N; ++l) ab[l] = __shfl_sync(0xffffffffu, m, g * N + l);
+    ab[N] = sqrt(abs2(b[N]));
+  }
   cd z = *zj;
   bool done = false;
 #pragma unroll 1
@@ -335,17 +342,12 @@ __device__ inline bool ehrlich_aberth_f64_warp(const cd* b, cd* zj, int np, int 
     }
     cd p, dp;
     horner2<N, double>(b, z, p, dp);
-    const float az = sqrtf((float)abs2(z));
-    float pa = ab[N];
-#pragma unroll
-    for (int l = N - 1; l >= 0; --l) pa = fmaf(pa, az, ab[l]);
-    const float noise = 1.1102230246251565e-16f * pa / fmaxf(sqrtf((float)abs2(dp)), 1e-30f);
     const cd W = dv(p, dp);
     cd dz = dv(W, mk(1.0, 0.0) - W * S);
     if (!(abs2(p) > 0.0)) dz = mk(0.0, 0.0);
+    const bool rnd = ea64_at_rounding<N>(ab, z, dz, dp);
     if (!done) z = z - dz;
-    const float st = sqrtf((float)abs2(dz));
-    const bool conv = st <= fmaxf(1e-14f * fmaxf(1.0f, sqrtf((float)abs2(z))), 2.0f * noise);
+    const bool conv = rnd || ea64_small(z, dz);
     const unsigned cb = __ballot_sync(0xffffffffu, conv);  // (every lane votes, done or not)
     done = done || (cb & mine) == mine;
     if (__all_sync(0xffffffffu, done)) break;

@@ -38,7 +38,7 @@ constexpr int MAXSEC = 10;       // sectors of an epoch (N_deg of the triple len
 constexpr int TASK_WARPS = 16;   // the theta chunks are cut for this many warps
 constexpr int DQ = 32;           // deferred boundary points per warp (derivative): one per lane at a flush
 constexpr int FQ = 64;           // the same, forward: flushed 32 at a time
-constexpr int PCAP = 64;         // boundary points per task that keep their place in the sum (forward)
+constexpr int PCAP = 64;         // places for a task's boundary points (forward; more are gathered, see gather_points)
 constexpr int XQ = 8;            // boundary points per warp whose crossing needs FP64
 constexpr float EPS32 = 5.9604645e-8f;  // 2^-24
 constexpr int KB = 8;            // columns per block (even: column pairs load as 16 bytes)
@@ -358,7 +358,7 @@ struct RayArgs {
   int* wqueue;      // boundary points, DQ per warp
   float* rowp;      // [task][32] the rows' r_i x sum (forward)
   float* pterm;     // [task][PCAP] the boundary points' terms
-  int* pcnt;        // [task] their number
+  int* pcnt;        // [task] the places they take
   int tcap;         // tasks of a batch
   int tabcap;       // columns that tabf holds
   int ccap;         // columns that the derivative's cosine table holds (0: none)
@@ -697,7 +697,7 @@ __device__ __forceinline__ float point_term(const SH& sh, const RayArgs& P, cons
 // The warp's points whose crossing needs FP64: four at a time, the five
 // stencil rays of a point on five of its eight lanes.
 template <int NL, int LAW, class SH>
-__device__ __noinline__ float2 flush_exact(SH& sh, RayShared& rs, int n, float2 acc) {
+__device__ __noinline__ void flush_exact(SH& sh, RayShared& rs, int n) {
   const RayArgs& P = rs.P;
   const int lane = threadIdx.x & 31;
   const int2* xq = rs.xq[threadIdx.x >> 5];
@@ -705,7 +705,7 @@ __device__ __noinline__ float2 flush_exact(SH& sh, RayShared& rs, int n, float2 
   for (int e0 = 0; e0 < n; e0 += 4) {
     const int e = e0 + (lane >> 3), k = lane & 7;
     const bool has = e < n;
-    const int2 v2 = has ? xq[e] : make_int2(0, -1);
+    const int2 v2 = has ? xq[e] : make_int2(0, 0);
     const int v = v2.x;
     const Sec& S = rs.sec[v >> 25];
     const int irow = (v >> 13) & 4095, m = v & 8191;
@@ -735,26 +735,22 @@ __device__ __noinline__ float2 flush_exact(SH& sh, RayShared& rs, int n, float2 
       float W, WU;
       (void)boundary_weight(sh, P, sv, dist, &W, &WU);
       if (P.diag) atomicAdd(&sh.cnt[3], 1);
-      const float term = point_term<LAW>(sh, P, S, ri_, -sv[2], fsc, W, WU);
-      if (v2.y >= 0) P.pterm[v2.y] = term;
-      else kahan_add(acc, term);
+      P.pterm[v2.y] = point_term<LAW>(sh, P, S, ri_, -sv[2], fsc, W, WU);
     }
   }
   __syncwarp();
-  return acc;
 }
 
 // n <= 32 queued points q, one per lane: each re-evaluates its stencil (rays m
 // - 2 .. m + 2, signed squared distances, negative inside) and writes its term
-// to its place (the point's second word; -1: its task has no more, the term is
-// added here).  Points that need FP64 go to the warp's second queue (*xn
-// entries).
+// to its place (the point's second word).  Points that need FP64 go to the
+// warp's second queue; xn of its entries are taken, the new number comes back.
 template <int NL, int LAW, class SH>
-__device__ __noinline__ float2 flush_points(SH& sh, RayShared& rs, const int2* q, int n, int* xn, float2 acc) {
+__device__ __noinline__ int flush_points(SH& sh, RayShared& rs, const int2* q, int n, int xn) {
   const int lane = threadIdx.x & 31;
   __syncwarp();
   bool exact = false;
-  int2 v2 = make_int2(0, -1);
+  int2 v2 = make_int2(0, 0);
   if (lane < n) {
     v2 = q[lane];
     const int v = v2.x;
@@ -778,19 +774,67 @@ __device__ __noinline__ float2 flush_points(SH& sh, RayShared& rs, const int2* q
       if (boundary_weight(sh, rs.P, sv, nullptr, &W, &WU)) term = point_term<LAW>(sh, rs.P, S, ri_, -sv[2], fsc, W, WU);
       else exact = true;
     }
-    if (v2.y >= 0) rs.P.pterm[v2.y] = term;
-    else if (!exact) kahan_add(acc, term);
+    rs.P.pterm[v2.y] = term;
   }
   unsigned todo = __ballot_sync(0xffffffffu, exact);
   while (todo) {
-    if (*xn == XQ) { acc = flush_exact<NL, LAW>(sh, rs, XQ, acc); *xn = 0; }
+    if (xn == XQ) { flush_exact<NL, LAW>(sh, rs, XQ); xn = 0; }
     const int src = __ffs(todo) - 1;
-    if (lane == src) rs.xq[threadIdx.x >> 5][*xn] = v2;
-    ++*xn;
+    if (lane == src) rs.xq[threadIdx.x >> 5][xn] = v2;
+    ++xn;
     todo &= todo - 1u;
   }
   __syncwarp();
-  return acc;
+  return xn;
+}
+
+// The warp's queued points: all q[0 .. n - 1] (n <= FQ) and the xn that need
+// FP64.
+template <int NL, int LAW, class SH>
+__device__ __noinline__ void flush_all(SH& sh, RayShared& rs, const int2* q, int n, int xn) {
+  for (; n > 0; n -= min(n, 32)) {
+    const int m = min(n, 32);
+    xn = flush_points<NL, LAW>(sh, rs, q + n - m, m, xn);
+  }
+  if (xn) flush_exact<NL, LAW>(sh, rs, xn);
+}
+
+// A task that has more boundary points than places: the n <= PCAP terms so far
+// become one, in the first two places (as a float pair), and the next points
+// take the places after them.  (Two images in one sector and whole rows to a
+// task give 4 points a row, 128 a task.)  The terms are added in the order of
+// the points, which is the task's own, so the sum does not depend on the warp
+// that took the task.
+constexpr int PGATHERED = 2;
+__device__ __forceinline__ void gather_points(float* pterm, int n) {
+  static_assert(PCAP == 64, "two terms a lane");
+  const int lane = threadIdx.x & 31;
+  double s = lane < n ? (double)pterm[lane] : 0.0;
+  if (lane + 32 < n) s += (double)pterm[lane + 32];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) {
+    const float h = (float)s;
+    pterm[0] = h;
+    pterm[1] = isfinite(h) ? (float)(s - (double)h) : 0.0f;
+  }
+  __syncwarp();
+}
+
+// What a warp has queued, and the places that its task's points have taken.
+struct Queued { int n, xn, npt; };
+
+// Room for c <= 32 more points of a task (its places: pterm).  One function for
+// both reasons to flush: its call is inlined at every place that pushes points.
+template <int NL, int LAW, class SH>
+__device__ __noinline__ Queued make_room(SH& sh, RayShared& rs, const int2* q, float* pterm, int c, Queued u) {
+  if (u.npt + c > PCAP) {
+    flush_all<NL, LAW>(sh, rs, q, u.n, u.xn);
+    gather_points(pterm, u.npt);
+    return {0, 0, PGATHERED};
+  }
+  u.n -= 32;
+  u.xn = flush_points<NL, LAW>(sh, rs, q + u.n, 32, u.xn);
+  return u;
 }
 
 // The next batch of sectors (rs.b0 .. rs.b1 - 1, none left: b0 = b1): its
@@ -943,7 +987,7 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
       while (b + 1 < b1 && task >= rs.sec[b + 1].task0) ++b;
       const Sec& S = rs.sec[b];
       const int rbk = (task - S.task0) / S.nch, chk = task - S.task0 - rbk * S.nch;
-      int npt = 0;  // boundary points so far
+      int npt = 0;  // places taken by its boundary points
       const int i = rbk * 32 + lane;
       const bool rowok = i < NR;
       const int ii = rowok ? i : NR - 1;
@@ -981,10 +1025,13 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
           const bool has = bm != 0u;
           const int m = base - (has ? __ffs(bm) - 1 : 0);
           bm &= bm - 1u;
-          if (dq_n > FQ - 32) { dq_n -= 32; acc = flush_points<NL, LAW>(sh, rs, dq + dq_n, 32, &xq_n, acc); }
           const unsigned hm = __ballot_sync(0xffffffffu, has);
-          const int at = __popc(hm & lt_mask), seq = npt + at;
-          if (has) dq[dq_n + at] = make_int2(pack_point(b, i, m), seq < PCAP ? task * PCAP + seq : -1);
+          const int at = __popc(hm & lt_mask);
+          if (dq_n > FQ - 32 || npt + __popc(hm) > PCAP) {
+            const Queued u = make_room<NL, LAW>(sh, rs, dq, P.pterm + task * PCAP, __popc(hm), {dq_n, xq_n, npt});
+            dq_n = u.n; xq_n = u.xn; npt = u.npt;
+          }
+          if (has) dq[dq_n + at] = make_int2(pack_point(b, i, m), task * PCAP + npt + at);
           dq_n += __popc(hm);
           npt += __popc(hm);
         }
@@ -1183,12 +1230,10 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
       push_bits(rowok ? (((win & ~((win << 1) & (win >> 1))) >> 1) & 1u) : 0u, c1 - 1);
       const float rowacc = c0f * (float)cnt + (sj + (sj2.x + sj2.y));
       P.rowp[task * 32 + lane] = ri * rowacc;
-      if (lane == 0) P.pcnt[task] = min(npt, PCAP);
+      if (lane == 0) P.pcnt[task] = npt;
     }
-    if (dq_n > 32) { dq_n -= 32; acc = flush_points<NL, LAW>(sh, rs, dq + dq_n, 32, &xq_n, acc); }
-    if (dq_n) acc = flush_points<NL, LAW>(sh, rs, dq, dq_n, &xq_n, acc);
+    flush_all<NL, LAW>(sh, rs, dq, dq_n, xq_n);
     dq_n = 0;
-    if (xq_n) acc = flush_exact<NL, LAW>(sh, rs, xq_n, acc);
     xq_n = 0;
     __syncthreads();
 

@@ -59,7 +59,14 @@ constexpr int PB_W4T = PB_W1T + 3 * H * H * 2; // W4^T [128][16]
 constexpr int PACK_BYTES = PB_W4T + H * NOUTP * 2;
 static_assert(PACK_BYTES == ICRS_MLP_PACK_BYTES, "pack size");
 
-constexpr int WAIT_TRIES = 1 << 20;  // bounded mbarrier waits
+// Bounded mbarrier waits (the tests build a library in which the first wait of
+// each kernel runs out).  A kernel that gives up waits once more, again with a
+// limit, for the copies and contractions that it has in flight, since they
+// write to shared and tensor memory which the next block may be given.
+#ifndef ICRS_MLP_WAIT_TRIES
+#define ICRS_MLP_WAIT_TRIES (1 << 20)
+#endif
+constexpr int WAIT_TRIES = ICRS_MLP_WAIT_TRIES, LAST_WAIT_TRIES = 1 << 20;
 
 // ---------------------------------------------------------------- packing
 // One thread per 16-byte chunk (8 BF16 of one tile row).
@@ -236,7 +243,12 @@ mlp_infer_kernel(const uint8_t* __restrict__ pack, const float* __restrict__ the
     }
     tc::fence_before_sync();
   }
-  if (bad && err) atomicExch(err, 1);
+  if (bad) {
+    // (whatever ran out: the weights, or the layer that this group last committed)
+    (void)tc::mbar_wait(&bar[INF_GROUPS], 0, LAST_WAIT_TRIES);
+    (void)tc::mbar_wait(&bar[grp], ph ^ 1u, LAST_WAIT_TRIES);
+    if (err) atomicExch(err, 1);
+  }
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem_sh, 512);
@@ -310,7 +322,7 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
   const uint32_t Dx = tmem, Dw = tmem + 128, Db = tmem + 256, D4 = tmem + 272;
   const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
   const uint32_t sS = tc::smem_addr(sm);
-  uint32_t ph = 0, wph[3] = {0, 0, 0};
+  uint32_t ph = 0, wph = 0;  // bit i of wph: phase of wbar[i]
   bool failed = false, bad = false;
   auto wait_mma = [&]() -> bool {
     const bool ok = tc::mbar_wait(&bar, ph, WAIT_TRIES);
@@ -323,10 +335,16 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
     tc::fence_before_sync();
     __syncthreads();
   };
-  // thread 0: the copy that fills weight buffer i next has arrived
+  // thread 0: the copy that fills weight buffer i next is issued, has arrived
+  uint32_t inflight = 0b111;  // (the three issued above)
+  auto load_w = [&](int i, void* dst, int from, int bytes) {
+    tc::bulk_load(dst, pack + from, bytes, &wbar[i]);
+    inflight |= 1u << i;
+  };
   auto wait_w = [&](int i) {
-    if (!tc::mbar_wait(&wbar[i], wph[i], WAIT_TRIES)) bad = true;
-    wph[i] ^= 1u;
+    if (!tc::mbar_wait(&wbar[i], (wph >> i) & 1u, WAIT_TRIES)) { bad = true; return; }
+    wph ^= 1u << i;
+    inflight &= ~(1u << i);
   };
   // D = A^T B over the tile's samples, both operands [sample][.] tiles of ka
   // and kb columns
@@ -360,9 +378,9 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
       if (!wait_mma()) { failed = true; break; }
       // the weight buffer just read takes the next weights
       if (tid == 0) {
-        if (l == 0) tc::bulk_load(sm + TR_S0, pack + PB_W4T, XB0, &wbar[0]);
-        if (l == 1) tc::bulk_load(sm + TR_WA, pack + PB_W1 + 2 * XB, XB, &wbar[1]);   // W_3
-        if (l == 3) tc::bulk_load(sm + TR_WA, pack + PB_W1T + 2 * XB, XB, &wbar[1]);  // W_3^T
+        if (l == 0) load_w(0, sm + TR_S0, PB_W4T, XB0);
+        if (l == 1) load_w(1, sm + TR_WA, PB_W1 + 2 * XB, XB);   // W_3
+        if (l == 3) load_w(1, sm + TR_WA, PB_W1T + 2 * XB, XB);  // W_3^T
       }
       if (l == 4) break;
       const float* b = bias + l * H;
@@ -422,7 +440,7 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
       tc::mma_commit(&bar);
     }
     if (!wait_mma()) { failed = true; break; }
-    if (tid == 0) tc::bulk_load(Xt(4), pack + PB_W1T + XB, XB, &wbar[2]);  // W_2^T
+    if (tid == 0) load_w(2, Xt(4), PB_W1T + XB, XB);  // W_2^T
     if (col0 == 0) {
       float v[16];
       tc::tmem_ld16(D4 + lane, v);
@@ -472,7 +490,7 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
         tc::mma_commit(&bar);
       }
       if (!wait_mma()) { failed = true; break; }
-      if (tid == 0 && l == 3) tc::bulk_load(sm + TR_WA, pack + PB_W1T, XB, &wbar[1]);  // W_1^T
+      if (tid == 0 && l == 3) load_w(1, sm + TR_WA, PB_W1T, XB);  // W_1^T
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int c = col0 + 16 * h;
@@ -489,7 +507,14 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
       }
     }
   } while (false);
-  if ((failed || bad) && tid == 0 && err) atomicExch(err, 1);
+  if (failed) {
+    (void)tc::mbar_wait(&bar, ph ^ 1u, LAST_WAIT_TRIES);
+    if (tid == 0) {
+      for (int i = 0; i < 3; ++i)
+        if ((inflight >> i) & 1u) (void)tc::mbar_wait(&wbar[i], (wph >> i) & 1u, LAST_WAIT_TRIES);
+      if (err) atomicExch(err, 1);
+    }
+  }
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem, 512);

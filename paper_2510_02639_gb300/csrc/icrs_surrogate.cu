@@ -27,6 +27,7 @@
 #include "icrs.h"
 #include "icrs_common.cuh"
 #include "icrs_ps.cuh"
+#include "icrs_silu.cuh"
 #include "icrs_tc.cuh"
 
 namespace icrs {
@@ -97,13 +98,6 @@ __global__ void pack_kernel(const float* __restrict__ theta, uint8_t* __restrict
   *reinterpret_cast<uint4*>(pack + byte) = *reinterpret_cast<const uint4*>(v);
 }
 
-__device__ __forceinline__ float silu_prime(float z) {
-  // (the reciprocal with one Newton correction)
-  const float d = 1.0f + expf(-z), r = rcp_fast(d);
-  const float sg = d < 1e37f ? fmaf(fmaf(-d, r, 1.0f), r, r) : 0.0f;
-  return sg * (1.0f + z * (1.0f - sg));
-}
-
 __device__ __forceinline__ void store8(uint8_t* dst, const float* x) {
   __align__(16) __nv_bfloat16 h[8];
 #pragma unroll
@@ -130,20 +124,6 @@ __device__ __forceinline__ void load_input_row(const float* __restrict__ feat, i
     const float4 b = reinterpret_cast<const float4*>(feat + (size_t)q * 8)[1];
     f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z;
   }
-}
-
-// SiLU z / (1 + e^-z), the division written out: the reciprocal's
-// approximation, one correction of the quotient by its exact remainder (the
-// usual correctly rounded division without its range handling: d >= 1; d = inf
-// gives 0, where the plain division gives -0; a NaN stays one).  Paired
-// operations around the two exponentials are slower: 356 us against 341 for
-// 2^20 queries.
-__device__ __forceinline__ float silu_fast(float z) {
-  const float d = 1.0f + expf(-z);
-  const float r = rcp_fast(d);
-  const float q = z * r;
-  const float y = fmaf(fmaf(-q, d, z), r, q);
-  return d >= 1e37f ? 0.0f : y;
 }
 
 // ---------------------------------------------------------------- inference
@@ -228,7 +208,8 @@ mlp_infer_kernel(const uint8_t* __restrict__ pack, const float* __restrict__ the
           float v[16];
           tc::tmem_ld16(tmem + lane + c, v);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = silu_fast(v[j] + b[c + j]);
+          for (int j = 0; j < 16; ++j) v[j] += b[c + j];
+          silu_n<16>(v);
           store8(X + tc::kmajor_offset(row, c, H), v);
           store8(X + tc::kmajor_offset(row, c + 8, H), v + 8);
         }
@@ -394,8 +375,7 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           Zs[(size_t)(l * 8 + h * 4 + j) * TR_NT + tid] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = silu_fast(v[j]);
+        silu_n<16>(v);
         store8(Xt(l + 1) + tc::kmajor_offset(row, c, H), v);
         store8(Xt(l + 1) + tc::kmajor_offset(row, c + 8, H), v + 8);
       }
@@ -458,16 +438,14 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int c = col0 + 16 * h;
-        float v[16];
-        tc::tmem_ld16(Dx + lane + c, v);
+        float v[16], z[16];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const float4 z = Zs[(size_t)(l * 8 + h * 4 + j) * TR_NT + tid];
-          v[4 * j] *= silu_prime(z.x);
-          v[4 * j + 1] *= silu_prime(z.y);
-          v[4 * j + 2] *= silu_prime(z.z);
-          v[4 * j + 3] *= silu_prime(z.w);
+          const float4 z4 = Zs[(size_t)(l * 8 + h * 4 + j) * TR_NT + tid];
+          z[4 * j] = z4.x; z[4 * j + 1] = z4.y; z[4 * j + 2] = z4.z; z[4 * j + 3] = z4.w;
         }
+        tc::tmem_ld16(Dx + lane + c, v);
+        silu_prime_n<16>(z, v);
         store8(DZ + tc::kmajor_offset(row, c, H), v);
         store8(DZ + tc::kmajor_offset(row, c + 8, H), v + 8);
       }

@@ -545,8 +545,8 @@ mag_kernel(const icrs_params* __restrict__ P, int S, const double* __restrict__ 
     sh.htf = (float)sh.ht;
     if constexpr (DER) {
       float4* aA = (float4*)pr_;
-      float2* acs = (float2*)(aA + MAXANCH), *sums = acs + MAXANCH;
-      double* ws = (double*)(sums + NW * DSUM * 32);
+      float2* acs = (float2*)(aA + MAXANCH);
+      double* sums = (double*)(acs + MAXANCH), *ws = sums + NW * DSUM * 32;
       der_sh = {acs, aA, sums, ws, ccap ? (double2*)(ws + 5 * DSUM * TASK_WARPS) : nullptr};
     }
     rays_sh.P = {anch, spc, tabf, wqueue, rowp, pterm, pcnt, DER ? 1 << 30 : tcap, tabcap, ccap, g.n_r, g.n_theta, g.uniform, g.ld_split && !g.uniform ? 1 : 0,

@@ -17,8 +17,8 @@
 //     the basis, which shows), but the columns' sines and cosines, more than
 //     half of that, come from a table formed once per sector;
 //   * a warp reduction of twelve FP64 row terms per task.  The rows' terms
-//     are now added, exactly rounded products in double-float, to a column of
-//     sums per lane in shared memory, and reduced once per sector.
+//     are now added, still in FP64, to a column of sums per lane in shared
+//     memory, and reduced once per sector.
 // What bounds it now: at 64 x 256 the FP64 flush and the tangents, at 1024 x
 // 2048 the sweep's issue rate (196 instructions a ray in which a gradient is
 // formed, FMA pipe 42 % busy) and the wait for the slowest warp.  chi^2 and its
@@ -35,7 +35,7 @@ constexpr int DSUM = 15;  // sums per lane, see row_add
 struct DerRays {
   float2* acs;       // cos, sin of each anchor angle
   float4* aA;        // A_0, A_1 of each anchor (FP32)
-  float2* sums;      // [warp][DSUM][32] double-float, lane i of sum k at (i + k) & 31
+  double* sums;      // [warp][DSUM][32], lane i of sum k at (i + k) & 31
   double* wsum;      // [sector][DSUM][warp]
   double2* ctab;     // cosine and sine of the batch's columns, or NULL (no room)
 
@@ -59,42 +59,15 @@ struct DerRays {
 };
 // Shared memory of these tables (bytes), for nw warps.
 constexpr size_t der_rays_bytes(int nw) {
-  return MAXANCH * (sizeof(float2) + sizeof(float4)) + sizeof(float2) * nw * DSUM * 32 +
+  return MAXANCH * (sizeof(float2) + sizeof(float4)) + sizeof(double) * nw * DSUM * 32 +
          sizeof(double) * 5 * DSUM * TASK_WARPS;
 }
 
-// Double-float sum with a relative error of a few 2^-48 of |a| + |b| (Dekker).
-__device__ __forceinline__ df df_sum(df a, df b) {
-  const df s = two_sum(a.hi, b.hi);
-  return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
-}
-__device__ __forceinline__ df df_mulf(df a, float b) {
-  const df p = two_prod(a.hi, b);
-  return fast_two_sum(p.hi, __fmaf_rn(a.lo, b, p.lo));
-}
 // FP64 distance of a ray from the source centre, (c, sn) its column's cosine
 // and sine.
 __device__ __noinline__ double ray_distance_cs(const double* eps, const cd* a, cd wc, double r, double c, double sn) {
   const cd z = mk(r * c, r * sn);
   return sqrt(abs2(lens_map<2, double>(eps, a, z) - wc));
-}
-
-__device__ __forceinline__ double to_double(df a) { return (double)a.hi + (double)a.lo; }
-
-// a b (b exact) added to a double-float sum in shared memory.
-__device__ __forceinline__ void slot_add(float2* s, float a, float b) {
-  const df p = two_prod(a, b);
-  const float2 v = *s;
-  const df t = two_sum(v.x, p.hi);
-  const df n = fast_two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(v.y, p.lo)));
-  *s = make_float2(n.hi, n.lo);
-}
-__device__ __forceinline__ void slot_add(float2* s, df a, float b) {
-  const df p = df_mulf(a, b);
-  const float2 v = *s;
-  const df t = two_sum(v.x, p.hi);
-  const df n = fast_two_sum(t.hi, __fadd_rn(t.lo, __fadd_rn(v.y, p.lo)));
-  *s = make_float2(n.hi, n.lo);
 }
 
 // A row's sums v (v[0] = sum of I W, v[1 + k] = pg[k]) into the lane's column
@@ -103,16 +76,20 @@ __device__ __forceinline__ void slot_add(float2* s, df a, float b) {
 // S_b with respect to the bounds and the rest (bounds_of) are combinations of
 //   sum Row, sum Row (i + 1/2), sum Row r_i, sum r_i v1, sum r_i v1 (i + 1/2),
 //   sum r_i v2, sum r_i v3, sum r_i v4 .. sum r_i v11.
-__device__ __forceinline__ void row_add(float2* sums, int lane, int irow, float r, const float* v) {
-  auto at = [&](int k) -> float2* { return sums + k * 32 + ((lane + k) & 31); };
-  const float h = (float)irow + 0.5f;
-  slot_add(at(0), v[0], 1.0f);
-  slot_add(at(1), v[0], h);
-  slot_add(at(2), v[0], r);
-  slot_add(at(3), v[1], r);
-  slot_add(at(4), two_prod(v[1], r), h);
+// (The products of two floats are exact in FP64, so each addition rounds once.)
+__device__ __forceinline__ void row_add(double* sums, int lane, int irow, float r, const float* v) {
+  auto add = [&](int k, double a, double b) {
+    double* const s = sums + k * 32 + ((lane + k) & 31);
+    *s = fma(a, b, *s);
+  };
+  const double h = irow + 0.5, rd = (double)r, v0 = (double)v[0], v1 = (double)v[1];
+  add(0, v0, 1.0);
+  add(1, v0, h);
+  add(2, v0, rd);
+  add(3, v1, rd);
+  add(4, v1 * rd, h);
 #pragma unroll
-  for (int k = 2; k < 12; ++k) slot_add(at(3 + k), v[k], r);
+  for (int k = 2; k < 12; ++k) add(3 + k, (double)v[k], rd);
 }
 
 // What the law and the gradient rule need per ray.
@@ -449,7 +426,7 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
   float2 acc = make_float2(0.f, 0.f);  // Kahan sum of this thread
   const unsigned lt_mask = (1u << lane) - 1u;
   const AnchorF* const anf = P.anch;
-  float2* const sums = dr.sums + warp * DSUM * 32;
+  double* const sums = dr.sums + warp * DSUM * 32;
   // Tasks are dealt out in a fixed order (this thread's tasks tw, tw + NW, ...:
   // a compensated sum's order shows in A).  Their column chunks repeat with a
   // period of 4, 8 or 16, and an SM's four schedulers take the warps by their
@@ -474,7 +451,7 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
     for (int b = b0; b < b1; ++b) {
       const Sec& S = rs.sec[b];
 #pragma unroll
-      for (int k = 0; k < DSUM; ++k) sums[k * 32 + lane] = make_float2(0.f, 0.f);
+      for (int k = 0; k < DSUM; ++k) sums[k * 32 + lane] = 0.0;
       __syncwarp();
       for (int tk = tw; tk < S.ntask; tk += NW) {
         const int rbk = tk / S.nch, chk = tk - rbk * S.nch;
@@ -633,7 +610,12 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
           v[0] = rowacc;
 #pragma unroll
           for (int k = 0; k < 11; ++k) v[k + 1] = pg[k];
-          row_add(sums, lane, ii, ri, v);
+          // (a chunk beside the image adds nothing; FP64 instructions are what
+          // the rows' terms cost)
+          unsigned nz = 0u;
+#pragma unroll
+          for (int k = 0; k < 12; ++k) nz |= __float_as_uint(v[k]) << 1;
+          if (nz) row_add(sums, lane, ii, ri, v);
           kahan_add(acc, ri * rowacc * S.bxw);
         }
       }
@@ -642,13 +624,10 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
       // the warp's sums of this sector, lane k sum k over the 32 columns
       __syncwarp();
       if (lane < DSUM) {
-        df t = df_make(0.f, 0.f);
+        double t = 0.0;
 #pragma unroll 4
-        for (int j = 0; j < 32; ++j) {
-          const float2 v = sums[lane * 32 + ((j + lane) & 31)];
-          t = df_sum(t, df_make(v.x, v.y));
-        }
-        dr.wsum[(b * DSUM + lane) * TASK_WARPS + warp] = to_double(t);
+        for (int j = 0; j < 32; ++j) t += sums[lane * 32 + ((j + lane) & 31)];
+        dr.wsum[(b * DSUM + lane) * TASK_WARPS + warp] = t;
       }
       __syncwarp();
     }

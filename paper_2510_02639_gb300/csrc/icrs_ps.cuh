@@ -48,14 +48,17 @@ __device__ inline void ps_lens(const Lens& L, PsLens<NL>& P) {
 // FP64 Newton on the polynomial b about lens nj, the nearest one of z0, then
 // the lens-equation residual in that frame against img_tol.  Returns 1 and the
 // polished image (original frame) and |det J| if z0 converges to an image.
-// Newton converges quadratically: after a step below 1e-9 min(1, |x|), with the
-// next root a distance d away, what is left is about 1e-18 / d, and the rounding
-// of the polynomial already puts 1e-16 / d into the root.  (Waiting for a step
-// below 1e-15, which rounding often prevents, took up to eight iterations a root:
-// the features of 60,000 epochs 25.6 ms, 17.5 with this and the polynomials set up
-// once a position instead of once a root.)  *conv is
-// cleared when the steps stay larger (linear convergence next to a near-double
-// root, where an iterate can still pass the residual test).
+// Newton converges quadratically: after a step below 1e-10 min(1, |x|), with
+// the next root a distance d away, what is left is about 1e-20 / d, and the
+// rounding of the polynomial already puts 1e-16 / d into the root (40,000
+// positions around 50 binaries: A_ps is off by 2.03e-13 rms, 1.20e-11 at most, as
+// with a step of 1e-15; a step of 1e-9 adds a hundredth of the rounding).  Far
+// from every lens, |x| > 1e5, a step of 1e-15 |x| is all that rounding allows.
+// (Waiting for a step below 1e-15 everywhere, which rounding often prevents,
+// took up to eight iterations a root: the features of 60,000 epochs 24.5 ms,
+// 16.7 with this and the polynomials set up once a position instead of once a
+// root.)  *conv is cleared when the steps stay larger (linear convergence next to
+// a near-double root, where an iterate can still pass the residual test).
 template <int NL>
 __device__ inline int ps_polish_validate(const PsLens<NL>& P, const cd* b, int nj, cd w, cd z0, double img_tol, cd* zi,
                                          double* det, int* conv) {
@@ -70,7 +73,8 @@ __device__ inline int ps_polish_validate(const PsLens<NL>& P, const cd* b, int n
     if (!(abs2(dp) > 0.0)) break;
     const cd stp = dv(p, dp);
     x = x - stp;
-    if (abs2(stp) <= 1e-18 * fmin(1.0, abs2(x))) { *conv = 1; break; }
+    const double x2 = abs2(x);
+    if (abs2(stp) <= fmax(1e-20 * fmin(1.0, x2), 1e-30 * x2)) { *conv = 1; break; }
   }
   // residual and shear from one reciprocal per lens
   cd F = x - (w - an), gm = mk(0.0, 0.0);

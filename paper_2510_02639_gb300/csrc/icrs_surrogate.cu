@@ -511,9 +511,20 @@ __device__ __forceinline__ void packed_offsets(int l, int no, int ni, int* w, in
   }
 }
 
+// Byte of the i-th padding element of the packed operands (all of them zero):
+// columns 7 .. 15 of W_0, rows 2 .. 15 of W_4 and their transposes.
+constexpr int NPAD0 = H * (KIN - NIN), NPAD4 = (NOUTP - NOUT) * H, NPAD = NPAD0 + 2 * NPAD4;
+__device__ __forceinline__ int padding_offset(int i) {
+  if (i < NPAD0) return PB_W0 + tc::kmajor_offset(i / (KIN - NIN), NIN + i % (KIN - NIN), KIN);
+  i -= NPAD0;
+  const bool t = i >= NPAD4;
+  if (t) i -= NPAD4;
+  return t ? PB_W4T + tc::kmajor_offset(i % H, NOUT + i / H, NOUTP) : PB_W4 + tc::kmajor_offset(NOUT + i / H, i % H, H);
+}
+
 // Sum of the tile gradients (fixed order: eight interleaved partial sums, then
-// their sum), optional output, Adam update, and the updated weights into the
-// packed operands (whose padding stays zero).  A block takes 32 parameters
+// their sum), optional output, Adam update, and the updated weights (and the
+// padding) into the packed operands.  A block takes 32 parameters
 // with 8 threads each: one thread per parameter walked the 64 tiles of a batch
 // of 8192 one load after another.
 constexpr int RA_P = 32, RA_T = 8;
@@ -534,6 +545,8 @@ reduce_adam_kernel(float* __restrict__ theta, float* __restrict__ m1, float* __r
 #pragma unroll 4
     for (int t = y; t < ntiles; t += RA_T) g += reinterpret_cast<const float*>(ws + (size_t)t * WS_TILE + WS_Z)[i];
   part[y][x] = g;
+  if (lr > 0.0f && y == RA_T - 1 && i < NPAD)
+    *reinterpret_cast<__nv_bfloat16*>(pack + padding_offset(i)) = __float2bfloat16_rn(0.0f);
   __syncthreads();
   if (y != 0 || i >= NPARAM) return;
 #pragma unroll

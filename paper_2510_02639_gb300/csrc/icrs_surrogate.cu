@@ -250,6 +250,11 @@ mlp_infer_kernel(const uint8_t* __restrict__ pack, const float* __restrict__ the
 // transposed 2-byte stores, activations through the workspace and weights
 // copied by hand took 185 us of a 245 us step; the step takes 84 us now.
 constexpr int TR_NT = 512;
+// Accumulators of dW_4: the tensor core truncates where it aligns a step's terms,
+// so one chain of 8 steps is further off than FP32 additions of the 128 products
+// (rms 0.099 against 0.072 in units of 2^-24 of the terms' moduli, one tile, and
+// off to one side); four of 2 steps, added in FP32, 0.062.
+constexpr int PARTS4 = 4;
 constexpr int XB = H * H * 2, XB0 = H * KIN * 2;          // bytes of a [128][128] and a [128][16] tile
 constexpr size_t WS_Z = (size_t)4 * TM * H * 4;           // Z_l  [4][8][512] float4
 constexpr size_t WS_G = (((size_t)NPARAM * 4 + 255) / 256) * 256;
@@ -328,12 +333,13 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
     inflight &= ~(1u << i);
   };
   // D = A^T B over the tile's samples, both operands [sample][.] tiles of ka
-  // and kb columns
-  auto issue_t = [&](uint32_t d, uint32_t a, int ka, uint32_t b, int kb, int N) {
+  // and kb columns; as the sum of `parts` accumulators of N columns each
+  auto issue_t = [&](uint32_t d, uint32_t a, int ka, uint32_t b, int kb, int N, int parts) {
     const uint32_t id = tc::idesc_bf16(TM, N, true, true);
+    const int len = TM / 16 / parts;
     for (int ks = 0; ks < TM / 16; ++ks)
-      tc::mma_bf16(d, tc::smem_desc(a + ks * 32 * ka, 16 * ka, 128), tc::smem_desc(b + ks * 32 * kb, 16 * kb, 128), id,
-                   ks > 0 ? 1u : 0u);
+      tc::mma_bf16(d + ks / len * N, tc::smem_desc(a + ks * 32 * ka, 16 * ka, 128),
+                   tc::smem_desc(b + ks * 32 * kb, 16 * kb, 128), id, ks % len > 0 ? 1u : 0u);
   };
 
   do {
@@ -409,7 +415,7 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
       tc::fence_after_sync();
       wait_w(0);
       issue_gemm(Dx, sS + TR_DZ, sS + TR_S0, KIN, H, false);                         // dX_4 = dZ_4 W_4
-      issue_t(D4, tc::smem_addr(Xt(4)), H, sS + TR_DZ, KIN, NOUTP);                  // dW_4^T = X_4^T dZ_4
+      issue_t(D4, tc::smem_addr(Xt(4)), H, sS + TR_DZ, KIN, NOUTP, PARTS4);          // dW_4^T = X_4^T dZ_4
       {
         // db_4: every row of the ones' product is the column sums of dZ_4
         const uint32_t id = tc::idesc_bf16(TM, NOUTP, false, true);
@@ -422,10 +428,15 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
     if (!wait_mma()) { failed = true; break; }
     if (tid == 0) load_w(2, Xt(4), PB_W1T + XB, XB);  // W_2^T
     if (col0 == 0) {
-      float v[16];
-      tc::tmem_ld16(D4 + lane, v);
-      Gs[OW4 + row] = v[0];
-      Gs[OW4 + H + row] = v[1];
+      float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll
+      for (int i = 0; i < PARTS4; ++i) {
+        float v[16];
+        tc::tmem_ld16(D4 + lane + i * NOUTP, v);
+        s0 += v[0]; s1 += v[1];
+      }
+      Gs[OW4 + row] = s0;
+      Gs[OW4 + H + row] = s1;
     } else if (warp == 4) {
       float v[16];
       tc::tmem_ld16(Db + lane, v);
@@ -457,7 +468,7 @@ mlp_train_tile_kernel(const uint8_t* __restrict__ pack, const float* __restrict_
           wait_w(w);
           issue_gemm(Dx, sS + TR_DZ, w == 2 ? tc::smem_addr(Xt(4)) : sS + TR_WA, H, H, false);  // dX_l = dZ_l W_l
         }
-        issue_t(Dw, sS + TR_DZ, H, tc::smem_addr(Xt(l)), Kl, Kl);                               // dW_l = dZ_l^T X_l
+        issue_t(Dw, sS + TR_DZ, H, tc::smem_addr(Xt(l)), Kl, Kl, 1);                            // dW_l = dZ_l^T X_l
         {
           // db_l: dZ_l^T times ones
           const uint32_t id = tc::idesc_bf16(TM, NOUTP, true, false);

@@ -350,7 +350,6 @@ __device__ inline int ehrlich_aberth_f64(const cd* b, cd* z, int max_iter) {
   for (int l = 0; l <= N; ++l) ab[l] = sqrt(abs2(b[l]));
   for (int it = 0; it < max_iter; ++it) {
     cd dz[N];
-    bool rnd[N];
     bool done = true;
     for (int k = 0; k < N; ++k) {
       cd p, dp;
@@ -361,12 +360,10 @@ __device__ inline int ehrlich_aberth_f64(const cd* b, cd* z, int max_iter) {
         if (j != k) S = S + inv(z[k] - z[j]);
       dz[k] = dv(W, mk(1.0, 0.0) - W * S);
       if (!(abs2(p) > 0.0)) dz[k] = mk(0.0, 0.0);
-      rnd[k] = ea64_at_rounding<N>(ab, z[k], dz[k], dp);
+      // (the first root that is not there yet leaves the others untested)
+      if (done) done = ea64_small(z[k] - dz[k], dz[k]) || ea64_at_rounding<N>(ab, z[k], dz[k], dp);
     }
-    for (int k = 0; k < N; ++k) {
-      z[k] = z[k] - dz[k];
-      if (!(rnd[k] || ea64_small(z[k], dz[k]))) done = false;
-    }
+    for (int k = 0; k < N; ++k) z[k] = z[k] - dz[k];
     if (done) return it + 1;
   }
   return -1;

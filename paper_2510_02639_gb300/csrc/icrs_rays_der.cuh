@@ -77,19 +77,20 @@ __device__ __noinline__ double ray_distance_cs(const double* eps, const cd* a, c
 //   sum Row, sum Row (i + 1/2), sum Row r_i, sum r_i v1, sum r_i v1 (i + 1/2),
 //   sum r_i v2, sum r_i v3, sum r_i v4 .. sum r_i v11.
 // (The products of two floats are exact in FP64, so each addition rounds once.)
-__device__ __forceinline__ void row_add(double* sums, int lane, int irow, float r, const float* v) {
+struct RowTerms { float v[12]; };
+__device__ __forceinline__ void row_add(double* sums, int lane, int irow, float r, const RowTerms& t) {
   auto add = [&](int k, double a, double b) {
     double* const s = sums + k * 32 + ((lane + k) & 31);
     *s = fma(a, b, *s);
   };
-  const double h = irow + 0.5, rd = (double)r, v0 = (double)v[0], v1 = (double)v[1];
+  const double h = irow + 0.5, rd = (double)r, v0 = (double)t.v[0], v1 = (double)t.v[1];
   add(0, v0, 1.0);
   add(1, v0, h);
   add(2, v0, rd);
   add(3, v1, rd);
   add(4, v1 * rd, h);
 #pragma unroll
-  for (int k = 2; k < 12; ++k) add(3 + k, (double)v[k], rd);
+  for (int k = 2; k < 12; ++k) add(3 + k, (double)t.v[k], rd);
 }
 
 // What the law and the gradient rule need per ray.
@@ -406,7 +407,10 @@ __device__ __noinline__ float2 der_flush(SH& sh, RayShared& rs, const DerRays& d
         (void)ray_eval<2>(P.anch[ai], t.x, t.y, ri_, dri_, nullptr, &dw, &dz);
         grad_core(w, dz, dw, t.x, t.y, ri_, (float)lw + 0.5f, dr.aA[ai], dr.acs[ai], a, v + 1);
       }
-      row_add(dr.sums + (threadIdx.x >> 5) * DSUM * 32, lane, irow, ri_, v);
+      RowTerms t;
+#pragma unroll
+      for (int k = 0; k < 12; ++k) t.v[k] = v[k];
+      row_add(dr.sums + (threadIdx.x >> 5) * DSUM * 32, lane, irow, ri_, t);
       kahan_add(acc, ri_ * v[0] * S.bxw);
     }
   }
@@ -420,13 +424,15 @@ template <class SH>
 __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& dr) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int NT = blockDim.x, NW = NT >> 5;
-  const RayArgs P = rs.P;
+  // (The launch's arguments, the anchors, the queue and the lane sums are read
+  // through shared memory where they are used: kept in registers they pushed
+  // the sweep's own values into local memory, a spotted set's gradient at 1024
+  // x 2048 54 ms against 43.7.)
+  const RayArgs& P = rs.P;
   const int NR = P.NR, NTH = P.NTH;
   const DerLaw w = der_law(sh, P);
   float2 acc = make_float2(0.f, 0.f);  // Kahan sum of this thread
   const unsigned lt_mask = (1u << lane) - 1u;
-  const AnchorF* const anf = P.anch;
-  double* const sums = dr.sums + warp * DSUM * 32;
   // Tasks are dealt out in a fixed order (this thread's tasks tw, tw + NW, ...:
   // a compensated sum's order shows in A).  Their column chunks repeat with a
   // period of 4, 8 or 16, and an SM's four schedulers take the warps by their
@@ -435,7 +441,6 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
   // four warps, each has all of them (1024 x 2048 chi^2 gradient, 2,000 epochs:
   // 78 ms before, 72.5 with it; 64 x 256 the same).  The sums are the same bits.
   const int tw = (warp & ~3) | ((warp + (warp >> 2)) & 3);
-  int* const dq = P.wqueue + warp * DQ;
   int dq_n = 0;
   const int nbox = sh.nbox;
   const bool generic = sh.generic, spot = sh.spot;
@@ -451,7 +456,7 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
     for (int b = b0; b < b1; ++b) {
       const Sec& S = rs.sec[b];
 #pragma unroll
-      for (int k = 0; k < DSUM; ++k) sums[k * 32 + lane] = 0.0;
+      for (int k = 0; k < DSUM; ++k) dr.sums[(warp * DSUM + k) * 32 + lane] = 0.0;
       __syncwarp();
       for (int tk = tw; tk < S.ntask; tk += NW) {
         const int rbk = tk / S.nch, chk = tk - rbk * S.nch;
@@ -474,7 +479,7 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
         float4 A01 = make_float4(0.f, 0.f, 0.f, 0.f);
         float2 cs = make_float2(1.f, 0.f);
         int gbase = 0;
-        SpotBand spb;
+        float spx = 0.f;  // its spot band's width
         auto push_bits = [&](unsigned bm, int base) {
           while (__any_sync(0xffffffffu, bm != 0u)) {
             const bool has = bm != 0u;
@@ -482,10 +487,10 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
             bm &= bm - 1u;
             unsigned rem = __ballot_sync(0xffffffffu, has);
             while (rem) {
-              if (dq_n == DQ) { acc = der_flush(sh, rs, dr, dq, DQ, acc); dq_n = 0; }
+              if (dq_n == DQ) { acc = der_flush(sh, rs, dr, P.wqueue + warp * DQ, DQ, acc); dq_n = 0; }
               const int at = dq_n + __popc(rem & lt_mask);
               const bool take = ((rem >> lane) & 1u) && at < DQ;
-              if (take) dq[at] = pack_point(b, i, m);
+              if (take) P.wqueue[warp * DQ + at] = pack_point(b, i, m);
               const unsigned tk_ = __ballot_sync(0xffffffffu, take);
               dq_n += __popc(tk_);
               rem &= ~tk_;
@@ -513,7 +518,7 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
           if (!u_) {
             float fs = 1.f;
             if constexpr (decltype(hc)::value)
-              fs = in && spot ? spot_sweep<2, 2>(sh, rs, S, aidx, spb, dw, t.x, t.y, ri, dri, ii, l) : 1.f;
+              fs = in && spot ? spot_sweep<2, 2>(sh, rs, S, aidx, SpotBand{P.spc[aidx], spx}, dw, t.x, t.y, ri, dri, ii, l) : 1.f;
             const float a = seed_of(w, in, d2, pg, rowacc, hc, fs);
             if (a != 0.f) grad_core(w, dz, dw, t.x, t.y, ri, (float)l + 0.5f, A01, cs, a, pg);
           }
@@ -523,10 +528,10 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
         while (l < c1) {
           const int mgrp = (int)__umulhi((unsigned int)l, S.gmagic);
           aidx = S.abase + gi * S.mth + mgrp;
-          ar = anf[aidx];
+          ar = P.anch[aidx];
           A01 = dr.aA[aidx];
           cs = dr.acs[aidx];
-          if (spot) spb = spot_band(sh, rs, ar, aidx);
+          if (spot) spx = spot_band(sh, rs, ar, aidx).X;
           gbase = mgrp * gth;
           const int lend = min(gbase + gth, c1);
           const bool test = __any_sync(0xffffffffu, sb && ar.rout < __int_as_float(0x7f800000));
@@ -606,27 +611,27 @@ __device__ __noinline__ double der_stage(SH& sh, RayShared& rs, const DerRays& d
         win = (win << 1) | halo_flag<2, 2>(sh, rs, b, gi, ri, dri, ii, c1);
         push_bits(rowok ? (((win & ~((win << 1) & (win >> 1))) >> 1) & 1u) : 0u, c1 - 1);
         if (rowok) {
-          float v[12];
-          v[0] = rowacc;
+          RowTerms t;
+          t.v[0] = rowacc;
 #pragma unroll
-          for (int k = 0; k < 11; ++k) v[k + 1] = pg[k];
+          for (int k = 0; k < 11; ++k) t.v[k + 1] = pg[k];
           // (a chunk beside the image adds nothing; FP64 instructions are what
           // the rows' terms cost)
           unsigned nz = 0u;
 #pragma unroll
-          for (int k = 0; k < 12; ++k) nz |= __float_as_uint(v[k]) << 1;
-          if (nz) row_add(sums, lane, ii, ri, v);
+          for (int k = 0; k < 12; ++k) nz |= __float_as_uint(t.v[k]) << 1;
+          if (nz) row_add(dr.sums + warp * DSUM * 32, lane, ii, ri, t);
           kahan_add(acc, ri * rowacc * S.bxw);
         }
       }
-      if (dq_n) acc = der_flush(sh, rs, dr, dq, dq_n, acc);
+      if (dq_n) acc = der_flush(sh, rs, dr, P.wqueue + warp * DQ, dq_n, acc);
       dq_n = 0;
       // the warp's sums of this sector, lane k sum k over the 32 columns
       __syncwarp();
       if (lane < DSUM) {
         double t = 0.0;
 #pragma unroll 4
-        for (int j = 0; j < 32; ++j) t += sums[lane * 32 + ((j + lane) & 31)];
+        for (int j = 0; j < 32; ++j) t += dr.sums[(warp * DSUM + lane) * 32 + ((j + lane) & 31)];
         dr.wsum[(b * DSUM + lane) * TASK_WARPS + warp] = t;
       }
       __syncwarp();

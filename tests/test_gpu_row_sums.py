@@ -21,8 +21,8 @@ __global__ void rows(const float* v, const float* r, const int* row, int n, doub
   for (int k = 0; k < icrs::DSUM; ++k) sums[k * 32 + threadIdx.x] = 0.0;
   for (int i = 0; i < n; ++i) {
     const size_t o = (size_t)i * 32 + threadIdx.x;
-    float x[12];
-    for (int k = 0; k < 12; ++k) x[k] = v[o * 12 + k];
+    icrs::RowTerms x;
+    for (int k = 0; k < 12; ++k) x.v[k] = v[o * 12 + k];
     icrs::row_add(sums, threadIdx.x, row[o], r[o], x);
   }
   for (int k = 0; k < icrs::DSUM; ++k) out[k * 32 + threadIdx.x] = sums[k * 32 + ((threadIdx.x + k) & 31)];

@@ -202,7 +202,7 @@ __device__ inline AnchorF make_anchor(const Sec& S, const double* eps, const cd*
     A64[j] = R * (zc - a[j]);
     K64[j] = scl(inv(A64[j]), eps[j]);
     aa[j] = sqrtf(abs2(tof(A64[j])));
-    kk[j] = (float)eps[j] / aa[j];
+    kk[j] = fabsf((float)eps[j]) / aa[j];  // (|K_j|: a mass can be negative, see g1)
   }
   nc[2] = pc[2] = mk(0.0, 0.0);
   if constexpr (NL == 2) {
@@ -245,8 +245,9 @@ __device__ inline AnchorF make_anchor(const Sec& S, const double* eps, const cd*
     const float m_ = aa[j] - half, ih = 1.0f / (aa[j] - hx);
     um += kk[j] / m_;
     pmin *= m_;
-    g1 += (float)eps[j] * ih * ih;
-    g2 += 2.0f * (float)eps[j] * ih * ih * ih;
+    // (moduli: q2 + q3 > 1 or q < 0 make a mass negative, and the method has a value there too)
+    g1 += fabsf((float)eps[j]) * ih * ih;
+    g2 += 2.0f * fabsf((float)eps[j]) * ih * ih * ih;
   }
   if (bounded) {
     float mn = 0.f, mp = 1.f;
@@ -267,7 +268,7 @@ __device__ inline AnchorF make_anchor(const Sec& S, const double* eps, const cd*
       // superblock's ends by at most max |w''| l^2 / 8, with z'' = -z, w = z -
       // conj(sum_j eps_j / (z - a_j)): |w''| <= r (1 + |gamma|) + r^2
       // |gamma'|, |gamma| <= sum eps_j / (|A_j| - h)^2, |gamma'| <= 2 sum
-      // eps_j / (|A_j| - h)^3; plus the ends' own errors.  No test when that
+      // |eps_j| / (|A_j| - h)^3; plus the ends' own errors.  No test when that
       // is more than half the source radius.
       const float rm = (float)S.r_hi;
       const float e = 1.001f * S.sag * (rm * (1.0f + g1) + rm * rm * g2) + 4.0f * eb + 4e-6f * rho32;

@@ -18,10 +18,10 @@
 // in the same order as without the test, so the results are the same bits.
 //
 // Bounded by the FP32 pipes and the latency of a ray's chain at fine grids (FMA
-// pipe 54 % busy at 1024 x 2048, nine tenths of an epoch's time) and by the
+// pipe 58 % busy at 1024 x 2048, nine tenths of an epoch's time) and by the
 // FP64 chains of the other phases at coarse ones.  The magnification kernel,
-// 64 sets: 8,000 epochs at 1024 x 2048 341 ms before and 227 with this stage;
-// 32,000 at 64 x 256 72 ms and 48 (with the binning and re-solve phases).
+// 64 sets: 25,600 epochs at 1024 x 2048 328 ms before and 205 with this stage;
+// 32,000 at 64 x 256 65 ms and 49 (with the binning and re-solve phases).
 #pragma once
 
 #include "icrs_common.cuh"
@@ -141,10 +141,12 @@ __device__ inline void sec_setup(Sec& S, const Box& B, int NR, int NTH) {
   S.nch = (NTH + S.ch - 1) / S.ch;
   S.ntask = ((NR + 31) >> 5) * S.nch;
   // A superblock's test costs about two ray evaluations a row, and what it
-  // saves grows with the number of superblocks across the image: about 32 of
-  // them; none when a chunk holds only two blocks.  (64 sets, without and with
-  // 16, 32, 64 columns: 12,800 epochs at 256 x 1024 44.6 and 41.8, 40.4, 40.5 ms;
-  // 6,400 at 1024 x 2048 80.2 and 60.6, 55.2, 53.5 ms.)
+  // saves grows with the number of superblocks across the image: 16 columns, 32
+  // from 1024 a sector, 64 from 2048, which makes at most 64 of them up to 4096
+  // columns; none when a chunk holds only two blocks.  The optimum
+  // is flat: 64 sets, without and with 16, 32, 64 columns, 12,800 epochs at 256
+  // x 1024 44.6 and 41.8, 40.4, 40.5 ms; 6,400 at 512 x 1024 31.1 and 28.1, 27.0,
+  // 26.8; 6,400 at 1024 x 2048 80.2 and 60.6, 55.2, 53.5 ms.
   S.sb = S.ch <= 2 * KB ? 0 : (NTH >= 2048 ? 64 : (NTH >= 1024 ? 32 : 16));
   const float ls = (float)S.sb * S.dth32;
   S.sag = 0.125f * ls * ls;
@@ -221,9 +223,11 @@ __device__ inline AnchorF make_anchor(const Sec& S, const double* eps, const cd*
   for (int k = 0; k < 3; ++k) { af.n[k] = tof(nc[k]); af.p[k] = tof(pc[k]); }
   // error bound of |Delta w'|: anchor term plus rounding of the ray's offset
   // (at most the group half-diagonal) and of its image term.  (The bounds are
-  // formed in FP32: their factors 2 and 1.01 leave room for the 1e-6 by which
-  // that rounds them, and the FP64 form took ten square roots and divisions of
-  // 600 cycles each.)
+  // formed in FP32: their factors 2 and 1.01 leave room for the 1e-5 by which
+  // that rounds them, aa - half cancelling to a seventeenth of aa at the nearest
+  // lens admitted included; 400,000 random anchors a lens count, up to that
+  // edge, were off by 8e-6 at most.  The FP64 form took ten square roots and
+  // divisions of 600 cycles each.)
   const float half = 0.5f * (float)S.gr * S.dr32 + (float)S.r_hi * 0.5f * (float)S.gth * S.dth32;
   af.e0 = 16.0f * EPS32 * (fabsf(af.ws.x) + fabsf(af.ws.y) + 2.0f * half);
   // the group's band: every ray has |dz| <= half, so |Q_j| >= |A_j| - half,
@@ -356,7 +360,7 @@ struct RayArgs {
   AnchorF* anch;
   float2* spc;      // spot centre in each anchor's frame
   float* tabf;      // group offsets (cos d - 1, sin d) of the batch's sectors
-  int* wqueue;      // boundary points, DQ per warp
+  int* wqueue;      // boundary points per warp: forward FQ (point, place) pairs, derivative DQ points
   float* rowp;      // [task][32] the rows' r_i x sum (forward)
   float* pterm;     // [task][PCAP] the boundary points' terms
   int* pcnt;        // [task] the places they take
@@ -821,21 +825,24 @@ __device__ __forceinline__ void gather_points(float* pterm, int n) {
   __syncwarp();
 }
 
-// What a warp has queued, and the places that its task's points have taken.
-struct Queued { int n, xn, npt; };
+// What a warp has queued, in one register: its points (bits 0 .. 7), those that
+// need FP64 (8 .. 15), and the places that its task's points have taken (16 up).
+__device__ __forceinline__ int q_points(unsigned q) { return (int)(q & 255u); }
+__device__ __forceinline__ int q_exact(unsigned q) { return (int)((q >> 8) & 255u); }
+__device__ __forceinline__ int q_places(unsigned q) { return (int)(q >> 16); }
 
-// Room for c <= 32 more points of a task (its places: pterm).  One function for
-// both reasons to flush: its call is inlined at every place that pushes points.
+// Room for c <= 32 more points of a task.  One function for both reasons to
+// flush: its call is inlined at every place that pushes points.
 template <int NL, int LAW, class SH>
-__device__ __noinline__ Queued make_room(SH& sh, RayShared& rs, const int2* q, float* pterm, int c, Queued u) {
-  if (u.npt + c > PCAP) {
-    flush_all<NL, LAW>(sh, rs, q, u.n, u.xn);
-    gather_points(pterm, u.npt);
-    return {0, 0, PGATHERED};
+__device__ __noinline__ unsigned make_room(SH& sh, RayShared& rs, int task, int c, unsigned q) {
+  const int2* const dq = reinterpret_cast<const int2*>(rs.P.wqueue) + (threadIdx.x >> 5) * FQ;
+  if (q_places(q) + c > PCAP) {
+    flush_all<NL, LAW>(sh, rs, dq, q_points(q), q_exact(q));
+    gather_points(rs.P.pterm + task * PCAP, q_places(q));
+    return (unsigned)PGATHERED << 16;
   }
-  u.n -= 32;
-  u.xn = flush_points<NL, LAW>(sh, rs, q + u.n, 32, u.xn);
-  return u;
+  const int n = q_points(q) - 32, xn = flush_points<NL, LAW>(sh, rs, dq + n, 32, q_exact(q));
+  return (q & 0xffff0000u) | (unsigned)(xn << 8) | (unsigned)n;
 }
 
 // The next batch of sectors (rs.b0 .. rs.b1 - 1, none left: b0 = b1): its
@@ -912,8 +919,7 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
   const unsigned lt_mask = (1u << lane) - 1u;
   const AnchorF* const anf = P.anch;
   const float* const tabf = P.tabf;
-  int2* const dq = reinterpret_cast<int2*>(P.wqueue) + warp * FQ;
-  int dq_n = 0, xq_n = 0;
+  unsigned queued = 0u;  // see make_room
   const int nbox = sh.nbox;
 
   if (tid < nbox) sec_setup(rs.sec[tid], sh.box[tid], NR, NTH);
@@ -988,7 +994,7 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
       while (b + 1 < b1 && task >= rs.sec[b + 1].task0) ++b;
       const Sec& S = rs.sec[b];
       const int rbk = (task - S.task0) / S.nch, chk = task - S.task0 - rbk * S.nch;
-      int npt = 0;  // places taken by its boundary points
+      queued &= 0xffffu;  // no place taken yet
       const int i = rbk * 32 + lane;
       const bool rowok = i < NR;
       const int ii = rowok ? i : NR - 1;
@@ -1027,14 +1033,11 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
           const int m = base - (has ? __ffs(bm) - 1 : 0);
           bm &= bm - 1u;
           const unsigned hm = __ballot_sync(0xffffffffu, has);
-          const int at = __popc(hm & lt_mask);
-          if (dq_n > FQ - 32 || npt + __popc(hm) > PCAP) {
-            const Queued u = make_room<NL, LAW>(sh, rs, dq, P.pterm + task * PCAP, __popc(hm), {dq_n, xq_n, npt});
-            dq_n = u.n; xq_n = u.xn; npt = u.npt;
-          }
-          if (has) dq[dq_n + at] = make_int2(pack_point(b, i, m), task * PCAP + npt + at);
-          dq_n += __popc(hm);
-          npt += __popc(hm);
+          const int at = __popc(hm & lt_mask), c = __popc(hm);
+          if (q_points(queued) > FQ - 32 || q_places(queued) + c > PCAP)
+            queued = make_room<NL, LAW>(sh, rs, task, c, queued);
+          if (has) reinterpret_cast<int2*>(rs.P.wqueue)[warp * FQ + q_points(queued) + at] = make_int2(pack_point(b, i, m), task * PCAP + q_places(queued) + at);
+          queued += (unsigned)c * 0x10001u;
         }
       };
       // boundary centres among columns l0 - 1 .. l0 + nb - 2 (bit j = column
@@ -1231,11 +1234,10 @@ __device__ __noinline__ double ray_stage(SH& sh, RayShared& rs) {
       push_bits(rowok ? (((win & ~((win << 1) & (win >> 1))) >> 1) & 1u) : 0u, c1 - 1);
       const float rowacc = c0f * (float)cnt + (sj + (sj2.x + sj2.y));
       P.rowp[task * 32 + lane] = ri * rowacc;
-      if (lane == 0) P.pcnt[task] = npt;
+      if (lane == 0) P.pcnt[task] = q_places(queued);
     }
-    flush_all<NL, LAW>(sh, rs, dq, dq_n, xq_n);
-    dq_n = 0;
-    xq_n = 0;
+    flush_all<NL, LAW>(sh, rs, reinterpret_cast<const int2*>(rs.P.wqueue) + warp * FQ, q_points(queued), q_exact(queued));
+    queued = 0u;
     __syncthreads();
 
     // ---- the sums, as a fixed assignment of the tasks would take them: thread

@@ -22,8 +22,8 @@
 // What bounds it now: at 64 x 256 the FP64 flush and the tangents, at 1024 x
 // 2048 the sweep's issue rate (196 instructions a ray in which a gradient is
 // formed, FMA pipe 42 % busy) and the wait for the slowest warp.  chi^2 and its
-// gradient, 256 sets at 64 x 256: 80.5 ms before, 42.7 now; 8 sets of 250
-// epochs at 1024 x 2048: 99 ms and 72.
+// gradient, 32 sets of 500 epochs at 64 x 256: 80.4 ms before, 44.0 now; 8 sets
+// of 250 at 1024 x 2048: 99.1 ms and 67.2.
 #pragma once
 
 #include "icrs_rays.cuh"
@@ -253,7 +253,7 @@ __device__ __noinline__ RowSums der_undecided(SH& sh, const RayShared& rs, const
 
 // n <= 32 queued boundary points, one per lane.  The stencil's flags come from
 // the FP32 distances (as in the forward stage), the crossing and its
-// derivative from the double-float ones: the point's value I (W - 1) beyond
+// derivative from the FP64 ones: the point's value I (W - 1) beyond
 // the I that the sweep added, its seed (W - 1) dI/dd, and the crossing seeds
 // -I f'(delta) l_m(x) / p'(x) on the stencil rays (p the cubic through the
 // stencil distances, x its crossing).

@@ -136,7 +136,7 @@ __device__ __forceinline__ void load_input_row(const float* __restrict__ feat, i
 // next layer's BF16 operand.
 //
 // The SiLU bounds it: 512 a query, 18 instructions each with the bias, the
-// rounding and the store: issue slots 79 % busy, special functions 34 %, tensor
+// rounding and the store: issue slots 78 % busy, special functions 34 %, tensor
 // cores 14 % (0.056 ms of 2^20 queries' contractions).  One group of 128
 // threads took 2.14 ms for 2^20 queries: one warp per scheduler, latency after
 // latency; three groups, which fill shared memory (212 KB), 0.34.
@@ -932,7 +932,7 @@ int icrs_mlp_train_step_noalloc(float* theta, float* adam_m, float* adam_v, void
   void* ws = nullptr;
   const int rc = static_scratch(&ws);
   if (rc != ICRS_OK) return rc;
-  // Every scratch word the step reads (activations, pre-activations, the
+  // Every scratch word the step reads (pre-activations, the
   // per-tile gradients and losses) is written earlier in the same step, so
   // nothing has to be cleared between calls.
   return icrs_mlp_train_step(theta, adam_m, adam_v, pack, step, lr, feat, target, n, grad, loss, ws,
